@@ -195,7 +195,9 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
       s_cur = next_s;
       __syncthreads();
     }
-    if (win_base < 0 || s_cur + kBlock > win_base + kSegWindow) {  // uniform: the window of offsets moves up to s_cur
+    // uniform: the window of offsets moves to s_cur (back to it where the walk over the last tile's segments moved the
+    // window past the segment that straddles the tile's end)
+    if (win_base < 0 || s_cur < win_base || s_cur + kBlock > win_base + kSegWindow) {
       win_base = s_cur;
       for (int k = threadIdx.x; k <= kSegWindow; k += kBlock) off_win[k] = s_cur + k <= S ? __ldg(off + s_cur + k) : 0x7FFFFFFF;
       __syncthreads();

@@ -475,6 +475,26 @@ def test_segmented_fold_with_skewed_and_awkward_segments():
     compare(prog, ref, got, "skewed segments, equal addends")
 
 
+@pytest.mark.parametrize("tail", [0, 3])
+def test_segmented_fold_where_a_window_of_offsets_ends_at_a_straddling_segment(tail):
+    """Tiles whose last segment, one that goes on into the next tile, is the last of a chunk of 256 offsets, so that the
+    window of offsets has moved past it when the next tile begins; sources with and without 128-bit rows."""
+    import torch
+    T, blocks = 4096, 6
+    lengths = []
+    for _ in range(blocks):                                # a block's run of eight tiles
+        lengths += [T] + [6] * 259 + [5] * 508 + [4]       # one whole tile; 768 segments of which the last lies across the tile's end
+        left = 6 * T - 2
+        lengths += [7] * (left // 7) + ([left % 7] if left % 7 else [])
+    lengths += [2] * 8 + ([tail] if tail else [])
+    offsets = torch.cat([torch.zeros(1, dtype=torch.int64), torch.tensor(lengths).cumsum(0)]).to(torch.int32)
+    prog = W.segmented_sums(int(offsets[-1]), len(lengths))
+    inputs = W.make_inputs(prog)
+    inputs[0] = inputs[0].abs() + 0.5
+    inputs[1] = offsets
+    check_program(prog, [[-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2]], inputs_t=inputs)
+
+
 def test_segmented_fold_reports_bad_offsets():
     import torch
     from paper_2407_13585_b200 import binding as B
