@@ -44,6 +44,7 @@ DTYPE = {"f32": ENUM["ACC_F32"], "i32": ENUM["ACC_I32"], "u32": ENUM["ACC_U32"]}
 FN = {k[7:].lower(): v for k, v in ENUM.items() if k.startswith("ACC_FN_")}
 IDX_FN = {k[8:].lower(): v for k, v in ENUM.items() if k.startswith("ACC_IDX_")}
 STATUS_NAME = {v: k for k, v in ENUM.items() if k.startswith("ACC_ERR_") or k == "ACC_OK"}
+ERR_WORKSPACE = ENUM["ACC_ERR_WORKSPACE"]
 FUSED, UNFUSED = ENUM["ACC_EXEC_FUSED"], ENUM["ACC_EXEC_UNFUSED"]
 PLAN = {"unfused": ENUM["ACC_PLAN_UNFUSED"], "enumerate": ENUM["ACC_PLAN_ENUMERATE"],
         "greedy_topdown": ENUM["ACC_PLAN_GREEDY_TOPDOWN"], "greedy_bottomup": ENUM["ACC_PLAN_GREEDY_BOTTOMUP"],
@@ -324,18 +325,29 @@ class Graph:
 
     @staticmethod
     def _stream():
+        """The current stream of the current device as a raw handle (no Stream object is made for it)."""
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
     def run(self, executor=FUSED, finish=True):
-        ws = self.ensure_workspace(executor)
-        _check(lib().acc_run(self._h, C.c_void_p(ws.data_ptr()), ws.numel(), self._stream(), executor))
+        # One library call in the usual case: acc_run looks at the workspace's size itself, before it enqueues
+        # anything, so the size is asked for only when it says that the workspace does not do.
+        ws = self.workspace
+        if ws is None:
+            ws = self.ensure_workspace(executor)
+        acc_run = lib().acc_run
+        code = acc_run(self._h, ws.data_ptr(), ws.numel(), self._stream(), executor)
+        if code == ERR_WORKSPACE:
+            ws = self.ensure_workspace(executor)
+            code = acc_run(self._h, ws.data_ptr(), ws.numel(), self._stream(), executor)
+        if code < 0:
+            _check(code)
         if finish:
             self.finish()
 
     def finish(self):
         ws = self.workspace
-        _check(lib().acc_finish(self._h, C.c_void_p(ws.data_ptr()) if ws is not None else None, self._stream()))
+        _check(lib().acc_finish(self._h, ws.data_ptr() if ws is not None else None, self._stream()))
 
     def run_e2e(self, executor=FUSED, finish=True):
         """Host inputs in, program, host outputs out on the current stream; finish=False returns

@@ -1,6 +1,5 @@
 // extern "C" entry points declared in acc.h.
 #include <cstring>
-#include <map>
 #include <memory>
 
 #include "acc.h"
@@ -10,16 +9,6 @@
 using namespace acc;
 
 namespace {
-
-// Schedules are rebuilt only when the graph, its clustering or its bindings change.
-struct Cache {
-  uint32_t serial = ~0u;
-  Schedule sch;
-};
-std::map<const acc_graph*, std::unique_ptr<Cache[]>>& caches() {
-  static std::map<const acc_graph*, std::unique_ptr<Cache[]>> c;
-  return c;
-}
 
 // The graph a run works on: the caller's, or, for the fused executor under a clustering with
 // copies, the graph in which the copies are nodes (buffers and output marks carried over).
@@ -40,9 +29,8 @@ Graph& run_target(acc_graph* g, int executor) {
 
 int schedule_for(acc_graph* g, int executor, Schedule** out) {
   if (executor != ACC_EXEC_FUSED && executor != ACC_EXEC_UNFUSED) return set_error(ACC_ERR_ARG, "unknown executor %d", executor);
-  auto& slot = caches()[g];
-  if (!slot) slot.reset(new Cache[2]);
-  Cache& c = slot[executor];
+  if (!g->cache[executor]) g->cache[executor] = std::make_shared<ScheduleCache>();
+  ScheduleCache& c = *g->cache[executor];
   if (c.serial != g->run_serial) {
     const int rc = build_schedule(run_target(g, executor), executor, c.sch);
     if (rc != ACC_OK) return rc;
@@ -68,7 +56,6 @@ int acc_graph_create(acc_graph** out) {
 int acc_graph_destroy(acc_graph* g) {
   clear_error();
   if (!g) return set_error(ACC_ERR_ARG, "graph is null");
-  caches().erase(g);
   delete g;
   return ACC_OK;
 }

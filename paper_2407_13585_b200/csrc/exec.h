@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <string>
 #include <utility>
 #include <vector>
 
@@ -26,7 +27,15 @@ struct Schedule {
   std::vector<uint8_t> manifest;
   std::vector<int32_t> pi;
   size_t ctrl_bytes = 0, array_bytes = 0, total_bytes = 0;
+  char* resolved_for = nullptr;      // the workspace that the steps' pointers were last filled in for
+  std::string text;                  // the clusters of a run, see acc_last_schedule
   std::vector<std::pair<size_t, size_t>> to_clear;   // (offset, bytes) of what a run zeroes first: the status slot and the zeroed part of every scratch
+};
+
+// A schedule is rebuilt only when the graph, its clustering or its bindings change.
+struct ScheduleCache {
+  uint32_t serial = ~0u;
+  Schedule sch;
 };
 
 int build_schedule(Graph& g, int executor, Schedule& sch);

@@ -80,6 +80,10 @@ int64_t enumerate_all(const Graph& g, std::vector<std::vector<int32_t>>& out, in
 int     partition_cost(const Graph& g, const int32_t* pi, int cost, double* out, int recompute_depth = 0);
 bool    canonical_numbering(const Graph& g, const std::vector<int>& block_of, int n_blocks, std::vector<int32_t>& pi);
 
+struct ScheduleCache;   // exec.h
+
 }  // namespace acc
 
-struct acc_graph : acc::Graph {};
+struct acc_graph : acc::Graph {
+  std::shared_ptr<acc::ScheduleCache> cache[2];   // the schedule of either executor (kept with the handle: handles on several threads share nothing)
+};
