@@ -44,6 +44,8 @@ bool bad_node(const acc_graph* g, acc_node n) { return n < 0 || n >= (acc_node)g
 
 }  // namespace
 
+acc_graph::~acc_graph() { give_back_status_words(status_words); }
+
 extern "C" {
 
 int acc_graph_create(acc_graph** out) {
@@ -310,7 +312,7 @@ int acc_run(acc_graph* g, void* workspace, size_t workspace_bytes, void* cuda_st
   int rc = schedule_for(g, executor, &sch);
   if (rc != ACC_OK) return rc;
   Graph& target = run_target(g, executor);
-  rc = run_schedule(target, *sch, workspace, workspace_bytes, static_cast<cudaStream_t>(cuda_stream));
+  rc = run_schedule(*g, target, *sch, workspace, workspace_bytes, static_cast<cudaStream_t>(cuda_stream));
   g->launches = target.launches;
   g->schedule = target.schedule;
   return rc;
@@ -326,7 +328,7 @@ int acc_run_timed(acc_graph* g, void* workspace, size_t workspace_bytes, void* c
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   std::vector<cudaEvent_t> marks;
   Graph& target = run_target(g, executor);
-  rc = run_schedule(target, *sch, workspace, workspace_bytes, stream, &marks);
+  rc = run_schedule(*g, target, *sch, workspace, workspace_bytes, stream, &marks);
   g->launches = target.launches;
   g->schedule = target.schedule;
   if (rc == ACC_OK) rc = finish(*g, workspace, stream);

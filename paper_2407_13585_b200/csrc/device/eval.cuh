@@ -48,11 +48,25 @@ template <int N>
 struct Args {
   NodeArg n[N];
   int32_t R, C;        // iteration domain of the cluster
-  uint32_t* scratch;   // zeroed control/partials region of this cluster
-  uint32_t* status;    // device status word of the run
+  uint32_t* scratch;   // control/partials region of this cluster
+  uint32_t* status;    // the run's status words (see raise_status)
+  uint32_t run_id;     // what a raised status word holds
   uint32_t spin_limit;
   int32_t grid;        // stride of the per-block partials of a fold
 };
+
+// Status words of a run: word k is set to the run's number by whoever meets condition k.  They lie in pinned host
+// memory, so that a run clears nothing beforehand and the host, once it has waited for the stream, reads them without
+// a copy; a word that holds an earlier run's number says nothing about this one.  One lane of those that get here
+// together writes.
+constexpr int kStatusTimeout = 0;        // a bounded wait ran out
+constexpr int kStatusIndex = 1;          // a scatter index or a segment offset outside its array
+constexpr int kStatusEmptySegment = 2;
+constexpr int kStatusConditions = 3;
+template <class A>
+__device__ __forceinline__ void raise_status(const A& a, int condition) {
+  if ((int)(threadIdx.x & 31) == __ffs(__activemask()) - 1) *reinterpret_cast<volatile uint32_t*>(a.status + condition) = a.run_id;
+}
 
 struct V4 { uint32_t v[4]; };
 

@@ -176,7 +176,7 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
   const double down = exp2((double)-S);
 
   auto scatter_one = [&](uint32_t k, uint32_t xbits) {
-    if (k >= n_bins) { atomicOr(a.status, kStatusIndex); return; }
+    if (k >= n_bins) { raise_status(a, kStatusIndex); return; }
     uint32_t at = k;                                           // position among this CTA's bins
     if (group != 1) {
       const uint32_t owner = plan.shift >= 0 ? (k >> plan.shift) : (k / (uint32_t)per_cta);

@@ -230,6 +230,7 @@ struct Launcher {
     a.C = C;
     a.scratch = L.scratch;
     a.status = L.status;
+    a.run_id = L.run_id;
     a.spin_limit = L.spin_limit;
     a.grid = sm_count() * 8;             // the partials' layout is sized for the largest grid
   }

@@ -41,7 +41,6 @@ constexpr int kSegBigCap = kSegTile / (kSegMedium + 1) + 2;    // pieces of a ti
 constexpr int kSegResident = 4;                // blocks per SM the kernel is built for
 constexpr int kSegTilesPerBlock = 8;           // a block's run of tiles: short enough for the block scheduler to even out slow and fast runs
 constexpr int kSegWindow = 1024;               // offsets kept in shared memory at a time
-constexpr uint32_t kStatusEmptySegment = 4u;
 
 template <class CL> constexpr int first_segfold() {
   for (int i = 0; i < CL::c.n; ++i)
@@ -109,8 +108,8 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
   // every offset is looked at once, whatever the walk below does with it
   for (int s = blockIdx.x * kBlock + threadIdx.x; s < S; s += gridDim.x * kBlock) {
     const int lo = __ldg(off + s), hi = __ldg(off + s + 1);
-    if (lo < 0 || hi > n_src) atomicOr(a.status, kStatusIndex);
-    else if (hi <= lo) atomicOr(a.status, kStatusEmptySegment);
+    if (lo < 0 || hi > n_src) raise_status(a, kStatusIndex);
+    else if (hi <= lo) raise_status(a, kStatusEmptySegment);
   }
 
   auto fold_slot_of = [](int i) { return count_if<CL>(is_segfold_root, i); };

@@ -22,8 +22,6 @@ namespace dev {
 
 constexpr int kBlock = 256;
 constexpr int kStreamTileRows = kBlock / 32;   // rows of a rank-2 tile of k_stream (one warp each)
-constexpr uint32_t kStatusTimeout = 1u;
-constexpr uint32_t kStatusIndex = 2u;
 
 template <int FN, int DT>
 __device__ __forceinline__ uint32_t warp_reduce(uint32_t v) {
@@ -92,10 +90,9 @@ __host__ __device__ inline uint32_t stream_acc64_off(int n_scalar_folds, int gri
   return (4u + (uint32_t)(n_scalar_folds * grid) + 1u) & ~1u;
 }
 
-template <int FN, int DT>
-__device__ __forceinline__ void permute_update(uint32_t* out, double* acc64, uint32_t bins, uint32_t k, uint32_t x,
-                                               uint32_t* status) {
-  if (k >= bins) { atomicOr(status, kStatusIndex); return; }
+template <int FN, int DT, class A>
+__device__ __forceinline__ void permute_update(const A& a, uint32_t* out, double* acc64, uint32_t bins, uint32_t k, uint32_t x) {
+  if (k >= bins) { raise_status(a, kStatusIndex); return; }
   if constexpr (DT == ACC_F32 && FN == ACC_FN_ADD) {
     // lanes of the warp that hit the same bin are summed first; one fp64 atomic per bin and warp
     const unsigned peers = __match_any_sync(__activemask(), k);
@@ -198,9 +195,9 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
         double* acc64 = acc64_of<CL, i>(a, acc64_base);
         if constexpr (VEC) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) permute_update<nd.fn, nd.dtype>(out, acc64, bins, k.v[j], x.v[j], a.status);
+          for (int j = 0; j < 4; ++j) permute_update<nd.fn, nd.dtype>(a, out, acc64, bins, k.v[j], x.v[j]);
         } else {
-          permute_update<nd.fn, nd.dtype>(out, acc64, bins, k, x, a.status);
+          permute_update<nd.fn, nd.dtype>(a, out, acc64, bins, k, x);
         }
       }
     });
@@ -700,7 +697,7 @@ struct ScanTile {
       if (done) break;
       look -= 32;
     }
-    if (gave_up && lane == 0) atomicOr(a.status, kStatusTimeout);
+    if (gave_up && lane == 0) raise_status(a, kStatusTimeout);
     if constexpr (WIDE) {
       exclusive = u_((float)wide);
       if (lane == 0) st_wide(states + tile, wide + (double)f_(tile_total));

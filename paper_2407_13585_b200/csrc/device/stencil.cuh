@@ -22,7 +22,7 @@
 // computed by the same expression, at positions clamped in the same way.
 //
 // Every wait on an mbarrier is bounded: after kCopySpinLimit polls the thread records
-// ACC_ERR_DEVICE_TIMEOUT in the status word and goes on, so a lost copy cannot hang the GPU.
+// ACC_ERR_DEVICE_TIMEOUT in the status words and goes on, so a lost copy cannot hang the GPU.
 #pragma once
 #include <cuda.h>
 
@@ -233,7 +233,7 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
     // the other stage was last read before the barrier that ended the previous trip
     if (threadIdx.x == 0 && tile + gridDim.x < n_tiles) issue(tile + gridDim.x, stage ^ 1);
     const bool arrived = wait_phase(&bar[stage], parity[stage]);
-    if (!arrived) atomicOr(a.status, kStatusTimeout);
+    if (!arrived) raise_status(a, kStatusTimeout);
 
     const uint32_t ty = tile / tiles_x, tx = tile - ty * tiles_x;
     const int r0 = (int)(ty * kStRows), c0 = (int)(tx * kStCols);

@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kBlock) k_tile_pair(const __grid_constant__ Ar
 // for 64 rows by whichever block arrived last took 0.36 ms of tail at 8192 x 8192.
 //
 // Every wait is bounded (wait_phase; kCopySpinLimit polls of the counter); a wait that runs out
-// sets the time-out bit of the status word and the block's `abort` word, which ends the walk of
+// raises the time-out status and the block's `abort` word, which ends the walk of
 // every warp; the copy warp then still waits, with the same bound, for copies in flight before
 // it leaves, and the block still arrives at the counter so that no other block waits for it.
 constexpr int kTpTileWords = kTile * kTile;          // 4096 words = 16 KB per copy
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
       issue(pair, (int)(trip % S));
     }
     if (!ok) {
-      if (!*v_abort) { *v_abort = 1; atomicOr(a.status, kStatusTimeout); }
+      if (!*v_abort) { *v_abort = 1; raise_status(a, kStatusTimeout); }
       // copies still in flight must not land in the shared memory of a block that has gone
       for (uint32_t q = 1; q <= (uint32_t)S && q <= trip; ++q) wait_phase(&full[(trip - q) % S], ((trip - q) / S) & 1u);
     }
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
   for (uint32_t pair = blockIdx.x; pair < n_pairs; pair += gridDim.x, ++it) {
     const int stage = (int)(it % S);
     const bool arrived = wait_phase(&full[stage], (it / S) & 1u) && !*v_abort;
-    if (!arrived && !*v_abort) { *v_abort = 1; atomicOr(a.status, kStatusTimeout); }
+    if (!arrived && !*v_abort) { *v_abort = 1; raise_status(a, kStatusTimeout); }
     int I, J;
     pair_of(pair, blocks, I, J);
     const int n_tiles = I == J ? 1 : 2;
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
     atomicAdd(arrivals, 1u);
     uint32_t spins = 0;
     while (*reinterpret_cast<volatile uint32_t*>(arrivals) < gridDim.x) {
-      if (++spins > kCopySpinLimit) { atomicOr(a.status, kStatusTimeout); break; }
+      if (++spins > kCopySpinLimit) { raise_status(a, kStatusTimeout); break; }
       __nanosleep(200);
     }
     __threadfence();

@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstring>
 #include <map>
+#include <mutex>
 
 #include "cluster.h"
 #include "exec.h"
@@ -171,7 +172,7 @@ int build_schedule(Graph& g, int executor, Schedule& sch) {
   std::map<int, std::vector<int>> clusters;
   for (int i = 0; i < n; ++i)
     if (!is_input(g.nodes[i])) clusters[pi[i]].push_back(i);
-  size_t ctrl = 256;                                    // status word first
+  size_t ctrl = 256;                                    // (first the word that acc_check_gather_indices reports to)
   for (auto& kv : clusters) {
     ClusterStep st;
     st.first_node = kv.second.front();
@@ -196,11 +197,10 @@ int build_schedule(Graph& g, int executor, Schedule& sch) {
   }
   sch.ctrl_bytes = ctrl;
   sch.to_clear.clear();
-  sch.to_clear.emplace_back(0, 256);                       // the status slot
   for (const ClusterStep& st : sch.steps) {
     if (st.zero_bytes == 0) continue;
-    auto& last = sch.to_clear.back();
-    if (last.first + align_up(last.second, 256) == st.scratch_off) last.second = st.scratch_off - last.first + st.zero_bytes;   // one piece
+    if (!sch.to_clear.empty() && sch.to_clear.back().first + align_up(sch.to_clear.back().second, 256) == st.scratch_off)
+      sch.to_clear.back().second = st.scratch_off - sch.to_clear.back().first + st.zero_bytes;   // one piece
     else sch.to_clear.emplace_back(st.scratch_off, st.zero_bytes);
   }
   sch.total_bytes = ctrl + sch.array_bytes;
@@ -219,6 +219,43 @@ static void* buffer_of(const Graph& g, const Schedule& sch, char* ws, int node) 
   if (nd.dev) return nd.dev;
   if (sch.array_off[node] == SIZE_MAX) return nullptr;
   return ws + sch.ctrl_bytes + sch.array_off[node];
+}
+
+// Status words of the handles (see raise_status in device/eval.cuh): pinned host memory that the kernels write to, a
+// cache line for each handle that has run, in pages that stay with the process; a destroyed handle's line goes to the
+// next one.  Run numbers are unique in the process, so a kernel that outlives its handle cannot speak for another run.
+// With the words in device memory a run paid for clearing them (3 us to enqueue) and a waited-for one for a copy back
+// (7 us to enqueue, 8 us of waiting): a chain of 2^16, waited for, 29.6 -> 16.6 us with the rest of the host path.
+namespace {
+std::mutex status_guard;
+std::vector<uint32_t*> free_status_words;
+std::atomic<uint32_t> last_run{0};
+constexpr int kStatusLines = 512;                          // lines of one page of status words
+}  // namespace
+
+// The handle's status words and a number for a new run.
+static int begin_run(Graph& handle) {
+  if (!handle.status_words) {
+    std::lock_guard<std::mutex> lock(status_guard);
+    if (free_status_words.empty()) {
+      void* page = nullptr;
+      if (cudaHostAlloc(&page, kStatusLines * 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
+        return set_error(ACC_ERR_CUDA, "no pinned memory for the status words: %s", cudaGetErrorString(cudaGetLastError()));
+      memset(page, 0, kStatusLines * 64);
+      for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_back(static_cast<uint32_t*>(page) + k * 16);
+    }
+    handle.status_words = free_status_words.back();
+    free_status_words.pop_back();
+  }
+  do handle.run_id = ++last_run;
+  while (handle.run_id == 0);
+  return ACC_OK;
+}
+
+void give_back_status_words(uint32_t* words) {
+  if (!words) return;
+  std::lock_guard<std::mutex> lock(status_guard);
+  free_status_words.push_back(words);
 }
 
 static bool mark(std::vector<cudaEvent_t>* marks, cudaStream_t stream) {
@@ -243,13 +280,12 @@ static int resolve_pointers(const Graph& g, Schedule& sch, char* ws) {
       st.launch.nodes[li].ptr = p;
     }
     st.launch.scratch = reinterpret_cast<uint32_t*>(ws + st.scratch_off);
-    st.launch.status = reinterpret_cast<uint32_t*>(ws);
   }
   sch.resolved_for = ws;
   return ACC_OK;
 }
 
-int run_schedule(Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cudaStream_t stream, std::vector<cudaEvent_t>* marks) {
+int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cudaStream_t stream, std::vector<cudaEvent_t>* marks) {
   if (!workspace) return set_error(ACC_ERR_WORKSPACE, "workspace is null, %zu bytes needed", sch.total_bytes);
   if (reinterpret_cast<uintptr_t>(workspace) & 255) return set_error(ACC_ERR_WORKSPACE, "workspace is not 256-byte aligned");
   if (ws_bytes < sch.total_bytes) return set_error(ACC_ERR_WORKSPACE, "workspace has %zu bytes, %zu needed", ws_bytes, sch.total_bytes);
@@ -258,6 +294,8 @@ int run_schedule(Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cuda
     const int rc = resolve_pointers(g, sch, ws);
     if (rc != ACC_OK) return rc;
   }
+  const int begun = begin_run(handle);
+  if (begun != ACC_OK) return begun;
   for (const auto& piece : sch.to_clear)
     if (cudaMemsetAsync(ws + piece.first, 0, piece.second, stream) != cudaSuccess)
       return set_error(ACC_ERR_CUDA, "clearing the control region failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -267,6 +305,8 @@ int run_schedule(Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cuda
   for (ClusterStep& st : sch.steps) {
     st.launch.stream = stream;
     st.launch.spin_limit = g.spin_limit;
+    st.launch.status = handle.status_words;
+    st.launch.run_id = handle.run_id;
     st.launch.extra_launches = 0;
     const int rc = st.kernel->launch(st.launch);
     if (rc != ACC_OK) return rc;
@@ -283,7 +323,7 @@ __global__ void k_index_range(const uint32_t* idx, int64_t n, uint32_t bound, ui
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, 2u);
 }
 
-int check_gather_indices(Graph& g, void* workspace, size_t ws_bytes, cudaStream_t stream) {
+int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaStream_t stream) {
   if (!workspace || ws_bytes < 256 || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return set_error(ACC_ERR_WORKSPACE, "the check needs a 256-byte aligned workspace of 256 bytes");
   if (cudaMemsetAsync(workspace, 0, 256, stream) != cudaSuccess)
@@ -299,62 +339,22 @@ int check_gather_indices(Graph& g, void* workspace, size_t ws_bytes, cudaStream_
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
   }
-  return finish(g, workspace, stream);
+  uint32_t status = 0;
+  if (cudaMemcpyAsync(&status, workspace, 4, cudaMemcpyDeviceToHost, stream) != cudaSuccess)
+    return set_error(ACC_ERR_CUDA, "reading the status word failed: %s", cudaGetErrorString(cudaGetLastError()));
+  const cudaError_t e = cudaStreamSynchronize(stream);
+  if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
+  return status ? set_error(ACC_ERR_INDEX_RANGE, "a gather index falls outside its source") : ACC_OK;
 }
-
-// Pinned words for reading status words back: a copy into pageable memory is staged by the driver and costs the caller
-// more than the wait itself (a 2^16-element chain, run and waited for: 29.6 -> 21.1 us, together with one library call a run instead of two
-// and the schedule's pointers and text made once).
-// One page for the whole process, a word to each call of finish() that is under way; a caller that finds none left reads
-// into its own stack as before.
-namespace {
-struct StatusWords {
-  static constexpr int kWords = 64;
-  std::atomic<uint64_t> taken{0};
-  uint32_t* words = nullptr;
-  StatusWords() {
-    void* p = nullptr;
-    if (cudaHostAlloc(&p, kWords * 64, cudaHostAllocPortable) == cudaSuccess) words = static_cast<uint32_t*>(p);   // a cache line each
-    else cudaGetLastError();
-  }
-  // the index of a word, -1 if there is none
-  int take() {
-    if (!words) return -1;
-    uint64_t t = taken.load(std::memory_order_relaxed);
-    while (~t) {
-      const int k = __builtin_ctzll(~t);
-      if (taken.compare_exchange_weak(t, t | (1ull << k), std::memory_order_acquire)) return k;
-    }
-    return -1;
-  }
-  void give_back(int k) { taken.fetch_and(~(1ull << k), std::memory_order_release); }
-};
-StatusWords& status_words() {
-  static StatusWords* w = new StatusWords();               // lives as long as the process: the driver may be gone before static destructors run
-  return *w;
-}
-}  // namespace
 
 int finish(Graph& g, void* workspace, cudaStream_t stream) {
-  uint32_t own = 0;
-  StatusWords& pinned = status_words();
-  const int slot = workspace ? pinned.take() : -1;
-  uint32_t* status_at = slot >= 0 ? pinned.words + slot * 16 : &own;
-  *status_at = 0;
-  cudaError_t copied = cudaSuccess;
-  if (workspace) copied = cudaMemcpyAsync(status_at, workspace, 4, cudaMemcpyDeviceToHost, stream);
-  const cudaError_t e = cudaStreamSynchronize(stream);     // (also before a pinned word may go to another call)
-  const uint32_t status = *status_at;
-  if (slot >= 0) pinned.give_back(slot);
-  if (copied != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(ACC_ERR_CUDA, "reading the status word failed: %s", cudaGetErrorString(copied));
-  }
+  const cudaError_t e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
-  g.host_status = status;
-  if (status & 1u) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
-  if (status & 2u) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index, a segment offset or a checked gather index fell outside its array");
-  if (status & 4u) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
+  if (!workspace || !g.run_id) return ACC_OK;
+  const volatile uint32_t* raised = g.status_words;
+  if (raised[dev::kStatusTimeout] == g.run_id) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
+  if (raised[dev::kStatusIndex] == g.run_id) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
+  if (raised[dev::kStatusEmptySegment] == g.run_id) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
   return ACC_OK;
 }
 

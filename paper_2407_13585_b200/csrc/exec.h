@@ -29,7 +29,7 @@ struct Schedule {
   size_t ctrl_bytes = 0, array_bytes = 0, total_bytes = 0;
   char* resolved_for = nullptr;      // the workspace that the steps' pointers were last filled in for
   std::string text;                  // the clusters of a run, see acc_last_schedule
-  std::vector<std::pair<size_t, size_t>> to_clear;   // (offset, bytes) of what a run zeroes first: the status slot and the zeroed part of every scratch
+  std::vector<std::pair<size_t, size_t>> to_clear;   // (offset, bytes) of what a run zeroes first: the zeroed part of every scratch
 };
 
 // A schedule is rebuilt only when the graph, its clustering or its bindings change.
@@ -41,10 +41,12 @@ struct ScheduleCache {
 int build_schedule(Graph& g, int executor, Schedule& sch);
 // Splits clusters of `pi` that have no instantiated kernel until every cluster has one (see acc_refine_to_kernels).
 int refine_to_kernels(const Graph& g, std::vector<int32_t>& pi, int recompute_depth, int& splits);
+// Enqueues a run of `handle`, whose clusters are those of g (the handle itself, or the graph in which its copies are nodes).
 // `marks`, if given, receives one recorded event before the first launch and one after each launch
-int run_schedule(Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cudaStream_t stream,
+int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cudaStream_t stream,
                  std::vector<cudaEvent_t>* marks = nullptr);
-int check_gather_indices(Graph& g, void* workspace, size_t ws_bytes, cudaStream_t stream);
+void give_back_status_words(uint32_t* words);
+int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaStream_t stream);
 int finish(Graph& g, void* workspace, cudaStream_t stream);
 
 }  // namespace acc

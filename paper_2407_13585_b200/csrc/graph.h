@@ -45,7 +45,8 @@ struct Graph {
   bool plan_proven = false;        // ... and whether its result is proven optimal
   int32_t launches = 0;
   std::string schedule;
-  uint32_t host_status = 0;
+  uint32_t run_id = 0;             // number of the last run, unique in the process; 0: none yet
+  uint32_t* status_words = nullptr;   // pinned host words that this handle's kernels report to, taken with the first run
   uint32_t run_serial = 0;         // bumped by every change that invalidates a schedule
   uint32_t spin_limit = 1u << 22;  // polls a scan tile spends on a predecessor before it gives up (acc_set_spin_limit)
 };
@@ -85,5 +86,6 @@ struct ScheduleCache;   // exec.h
 }  // namespace acc
 
 struct acc_graph : acc::Graph {
+  ~acc_graph();
   std::shared_ptr<acc::ScheduleCache> cache[2];   // the schedule of either executor (kept with the handle: handles on several threads share nothing)
 };

@@ -100,6 +100,7 @@ extern "C" int acc_scanl_add_i32_static(const int32_t* in, int32_t* out, int64_t
   a.C = (int32_t)n;
   a.scratch = reinterpret_cast<uint32_t*>(base + kHeaderBytes);
   a.status = reinterpret_cast<uint32_t*>(base);
+  a.run_id = 1;
   a.spin_limit = 1u << 22;
   a.grid = 0;
   const bool vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
@@ -109,10 +110,10 @@ extern "C" int acc_scanl_add_i32_static(const int32_t* in, int32_t* out, int64_t
   else dev::k_scan<ScanCluster, false><<<grid, kScanBlock, 0, stream>>>(a, tiles, tiles);
   e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
-  uint32_t status = 0;
-  e = cudaMemcpyAsync(&status, base, 4, cudaMemcpyDeviceToHost, stream);
+  uint32_t timed_out = 0;
+  e = cudaMemcpyAsync(&timed_out, base + 4 * dev::kStatusTimeout, 4, cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "waiting for the scan failed: %s", cudaGetErrorString(e));
-  if (status & dev::kStatusTimeout) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
+  if (timed_out) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
   return ACC_OK;
 }

@@ -16,7 +16,8 @@ struct ClusterLaunch {
   dev::NodeArg nodes[kMaxCluster];
   int n = 0;
   uint32_t* scratch = nullptr;   // scratch_bytes() bytes, 16-byte aligned, the first zeroed_bytes() of them zero
-  uint32_t* status = nullptr;
+  uint32_t* status = nullptr;    // the handle's status words (pinned host memory) and the number of this run
+  uint32_t run_id = 0;
   uint32_t spin_limit = 1u << 22;
   cudaStream_t stream = nullptr;
   mutable int extra_launches = 0;   // set by a launcher that took more launches than its entry's `passes` (data-dependent paths)
