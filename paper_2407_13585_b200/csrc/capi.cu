@@ -44,7 +44,7 @@ bool bad_node(const acc_graph* g, acc_node n) { return n < 0 || n >= (acc_node)g
 
 }  // namespace
 
-acc_graph::~acc_graph() { give_back_status_words(status_words); }
+acc_graph::~acc_graph() { give_back_status_words(*this); }
 
 extern "C" {
 

@@ -221,9 +221,11 @@ static void* buffer_of(const Graph& g, const Schedule& sch, char* ws, int node) 
   return ws + sch.ctrl_bytes + sch.array_off[node];
 }
 
-// Status words of the handles (see raise_status in device/eval.cuh): pinned host memory that the kernels write to, a
-// cache line for each handle that has run, in pages that stay with the process; a destroyed handle's line goes to the
-// next one.  Run numbers are unique in the process, so a kernel that outlives its handle cannot speak for another run.
+// Status words of the runs (see raise_status in device/eval.cuh): pinned host memory that the kernels write to, a cache
+// line for every workspace that a handle runs over (runs over different workspaces may be in flight together), in pages
+// that stay with the process; a destroyed handle's lines go to the next one.  Run numbers are unique in the process, so
+// a kernel that outlives its handle cannot speak for another run.  A run that is being captured into a CUDA graph will
+// be replayed under one number: its line is cleared in the stream, like the control region, and is not handed on.
 // With the words in device memory a run paid for clearing them (3 us to enqueue) and a waited-for one for a copy back
 // (7 us to enqueue, 8 us of waiting): a chain of 2^16, waited for, 29.6 -> 16.6 us with the rest of the host path.
 namespace {
@@ -231,31 +233,68 @@ std::mutex status_guard;
 std::vector<uint32_t*> free_status_words;
 std::atomic<uint32_t> last_run{0};
 constexpr int kStatusLines = 512;                          // lines of one page of status words
-}  // namespace
+constexpr size_t kMaxReports = 64;                         // lines of one handle; beyond that the one used longest ago is taken over
 
-// The handle's status words and a number for a new run.
-static int begin_run(Graph& handle) {
-  if (!handle.status_words) {
-    std::lock_guard<std::mutex> lock(status_guard);
-    if (free_status_words.empty()) {
-      void* page = nullptr;
-      if (cudaHostAlloc(&page, kStatusLines * 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
-        return set_error(ACC_ERR_CUDA, "no pinned memory for the status words: %s", cudaGetErrorString(cudaGetLastError()));
-      memset(page, 0, kStatusLines * 64);
-      for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_back(static_cast<uint32_t*>(page) + k * 16);
-    }
-    handle.status_words = free_status_words.back();
-    free_status_words.pop_back();
-  }
-  do handle.run_id = ++last_run;
-  while (handle.run_id == 0);
-  return ACC_OK;
+RunReport* report_for(Graph& handle, const void* workspace) {
+  for (RunReport& r : handle.reports)
+    if (r.workspace == workspace) return &r;
+  return nullptr;
 }
 
-void give_back_status_words(uint32_t* words) {
-  if (!words) return;
+uint32_t* take_status_words() {
   std::lock_guard<std::mutex> lock(status_guard);
-  free_status_words.push_back(words);
+  if (free_status_words.empty()) {
+    void* page = nullptr;
+    // (allocating is not allowed while a stream is being captured, unless the thread says that it does not matter)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaHostAlloc(&page, kStatusLines * 64, cudaHostAllocPortable | cudaHostAllocMapped);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      set_error(ACC_ERR_CUDA, "no pinned memory for the status words: %s", cudaGetErrorString(e));
+      return nullptr;
+    }
+    memset(page, 0, kStatusLines * 64);
+    for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_back(static_cast<uint32_t*>(page) + k * 16);
+  }
+  uint32_t* words = free_status_words.back();
+  free_status_words.pop_back();
+  return words;
+}
+
+// The report of a new run over `workspace`.
+int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunReport** out) {
+  RunReport* r = report_for(handle, workspace);
+  if (!r && handle.reports.size() >= kMaxReports) {
+    for (RunReport& c : handle.reports)
+      if (!c.captured && (!r || (int32_t)(c.run_id - r->run_id) < 0)) r = &c;
+  }
+  if (!r) {
+    uint32_t* words = take_status_words();
+    if (!words) return ACC_ERR_CUDA;
+    handle.reports.emplace_back();
+    r = &handle.reports.back();
+    r->words = words;
+  }
+  r->workspace = workspace;
+  do r->run_id = ++last_run;
+  while (r->run_id == 0);
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) cudaGetLastError();
+  r->captured = r->captured || capturing == cudaStreamCaptureStatusActive;
+  if (r->captured && cudaMemsetAsync(r->words, 0, dev::kStatusConditions * 4, stream) != cudaSuccess)
+    return set_error(ACC_ERR_CUDA, "clearing the status words failed: %s", cudaGetErrorString(cudaGetLastError()));
+  *out = r;
+  return ACC_OK;
+}
+}  // namespace
+
+void give_back_status_words(Graph& handle) {
+  std::lock_guard<std::mutex> lock(status_guard);
+  for (const RunReport& r : handle.reports)
+    if (!r.captured) free_status_words.push_back(r.words);
+  handle.reports.clear();
 }
 
 static bool mark(std::vector<cudaEvent_t>* marks, cudaStream_t stream) {
@@ -294,7 +333,8 @@ int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t
     const int rc = resolve_pointers(g, sch, ws);
     if (rc != ACC_OK) return rc;
   }
-  const int begun = begin_run(handle);
+  RunReport* report = nullptr;
+  const int begun = begin_run(handle, workspace, stream, &report);
   if (begun != ACC_OK) return begun;
   for (const auto& piece : sch.to_clear)
     if (cudaMemsetAsync(ws + piece.first, 0, piece.second, stream) != cudaSuccess)
@@ -305,8 +345,8 @@ int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t
   for (ClusterStep& st : sch.steps) {
     st.launch.stream = stream;
     st.launch.spin_limit = g.spin_limit;
-    st.launch.status = handle.status_words;
-    st.launch.run_id = handle.run_id;
+    st.launch.status = report->words;
+    st.launch.run_id = report->run_id;
     st.launch.extra_launches = 0;
     const int rc = st.kernel->launch(st.launch);
     if (rc != ACC_OK) return rc;
@@ -350,11 +390,13 @@ int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaS
 int finish(Graph& g, void* workspace, cudaStream_t stream) {
   const cudaError_t e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
-  if (!workspace || !g.run_id) return ACC_OK;
-  const volatile uint32_t* raised = g.status_words;
-  if (raised[dev::kStatusTimeout] == g.run_id) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
-  if (raised[dev::kStatusIndex] == g.run_id) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
-  if (raised[dev::kStatusEmptySegment] == g.run_id) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
+  const RunReport* r = workspace ? report_for(g, workspace) : nullptr;
+  if (!r) return ACC_OK;
+  const volatile uint32_t* words = r->words;
+  const auto raised = [&](int condition) { return r->captured ? words[condition] != 0 : words[condition] == r->run_id; };
+  if (raised(dev::kStatusTimeout)) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
+  if (raised(dev::kStatusIndex)) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
+  if (raised(dev::kStatusEmptySegment)) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
   return ACC_OK;
 }
 

@@ -28,6 +28,15 @@ struct Edge {
   bool ordered;   // the slot traverses the array in a definite order (Table 1)
 };
 
+// Where the kernels of the runs over one workspace report to: a line of pinned host words, in which a word that holds
+// the number of the last such run says that its condition arose.
+struct RunReport {
+  const void* workspace = nullptr;
+  uint32_t* words = nullptr;
+  uint32_t run_id = 0;             // unique in the process, never 0
+  bool captured = false;           // a run was enqueued on a capturing stream: the words are cleared in the stream, any non-zero word counts
+};
+
 struct Graph {
   std::vector<Node> nodes;
   std::vector<Edge> edges;
@@ -45,8 +54,7 @@ struct Graph {
   bool plan_proven = false;        // ... and whether its result is proven optimal
   int32_t launches = 0;
   std::string schedule;
-  uint32_t run_id = 0;             // number of the last run, unique in the process; 0: none yet
-  uint32_t* status_words = nullptr;   // pinned host words that this handle's kernels report to, taken with the first run
+  std::vector<RunReport> reports;  // one per workspace that runs were enqueued over
   uint32_t run_serial = 0;         // bumped by every change that invalidates a schedule
   uint32_t spin_limit = 1u << 22;  // polls a scan tile spends on a predecessor before it gives up (acc_set_spin_limit)
 };

@@ -495,6 +495,49 @@ def test_segmented_fold_where_a_window_of_offsets_ends_at_a_straddling_segment(t
     check_program(prog, [[-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2]], inputs_t=inputs)
 
 
+def test_status_belongs_to_the_run_over_its_workspace():
+    """Two runs of one handle in flight over two workspaces, and replays of a captured run: each wait reports its own."""
+    import torch
+    from paper_2407_13585_b200 import binding as B
+    prog = W.segmented_sums(1000, 4)
+    g = B.Graph(prog.nodes, prog.outputs)
+    g.set_partition([-1, -1, 0, 0, 0])
+    inputs = {k: v.cuda() for k, v in W.make_inputs(prog).items()}
+    offsets = inputs[1]
+    good, bad = offsets.clone(), torch.tensor([0, 10, 10, 500, 1000], dtype=torch.int32, device="cuda")
+    for i, t in inputs.items():
+        g.bind(i, t)
+    outs = [torch.empty(4, dtype=torch.float32, device="cuda") for _ in prog.outputs]
+    for o, t in zip(prog.outputs, outs):
+        g.bind(o, t)
+    spaces = [torch.empty(g.workspace_bytes(), dtype=torch.uint8, device="cuda") for _ in range(2)]
+
+    def status(ws):
+        g.workspace = ws
+        try:
+            g.finish()
+        except B.AccError as e:
+            return e.status
+        return "ACC_OK"
+
+    for ws, off in zip(spaces, (bad, good)):
+        offsets.copy_(off)
+        g.workspace = ws
+        g.run(finish=False)
+    assert [status(ws) for ws in spaces] == ["ACC_ERR_SHAPE", "ACC_OK"]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        g.workspace = spaces[1]
+        g.run(finish=False)
+    for off, want in ((bad, "ACC_ERR_SHAPE"), (good, "ACC_OK"), (bad, "ACC_ERR_SHAPE"), (good, "ACC_OK")):
+        offsets.copy_(off)
+        graph.replay()
+        assert status(spaces[1]) == want
+    assert status(spaces[0]) == "ACC_ERR_SHAPE"
+
+
 def test_segmented_fold_reports_bad_offsets():
     import torch
     from paper_2407_13585_b200 import binding as B
