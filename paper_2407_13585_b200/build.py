@@ -50,8 +50,33 @@ def _headers_mtime():
     return max(m, os.path.getmtime(os.path.abspath(__file__)))
 
 
-def _compile(src, obj, verbose):
+CLUSTERS_PER_PART = 10      # clusters one compiler run instantiates
+
+
+def _parts(src):
+    """How many parts a file of cluster instantiations is compiled in (see ACC_PARTS in csrc/device/launch.cuh)."""
+    with open(src) as f:
+        clusters = sum(line.startswith("ACC_CLUSTER") for line in f)
+    return max(1, -(-clusters // CLUSTERS_PER_PART))
+
+
+def _jobs(srcs, name_of, force, hdr):
+    """(objects to link, [(source, object, part, parts)] to compile), the largest files first."""
+    objs, jobs = [], []
+    for src in srcs:
+        parts = _parts(src)
+        for part in range(parts):
+            obj = os.path.join(OBJ, name_of(src) + (".%d" % part if parts > 1 else "") + ".o")
+            objs.append(obj)
+            if force or not os.path.exists(obj) or os.path.getmtime(obj) < max(hdr, os.path.getmtime(src)):
+                jobs.append((src, obj, part, parts))
+    return objs, sorted(jobs, key=lambda j: -os.path.getsize(j[0]) / j[3])
+
+
+def _compile(src, obj, part, parts, verbose):
     cmd = ["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-x", "cu", "-c", src, "-o", obj]
+    if parts > 1:
+        cmd += ["-DACC_PARTS=%d" % parts, "-DACC_PART=%d" % part]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed for %s\n%s\n%s" % (src, r.stdout, r.stderr))
@@ -62,14 +87,9 @@ def _compile(src, obj, verbose):
 def build(force=False, verbose=False):
     os.makedirs(OBJ, exist_ok=True)
     hdr = _headers_mtime()
-    jobs, objs = [], []
-    for src in _sources():
-        obj = os.path.join(OBJ, os.path.relpath(src, CSRC).replace(os.sep, "_") + ".o")
-        objs.append(obj)
-        if force or not os.path.exists(obj) or os.path.getmtime(obj) < max(hdr, os.path.getmtime(src)):
-            jobs.append((src, obj))
+    objs, jobs = _jobs(_sources(), lambda src: os.path.relpath(src, CSRC).replace(os.sep, "_"), force, hdr)
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as pool:
-        list(pool.map(lambda j: _compile(j[0], j[1], verbose), jobs))
+        list(pool.map(lambda j: _compile(*j, verbose), jobs))
     if jobs or not os.path.exists(LIB):
         cmd = ["nvcc", "-shared", "-o", LIB] + objs + ["-lcudart"]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -85,14 +105,9 @@ def build_kernel_library(src_dir, lib_path, force=False, verbose=False):
     os.makedirs(OBJ, exist_ok=True)
     hdr = _headers_mtime()
     tag = os.path.basename(lib_path).replace(".so", "")
-    jobs, objs = [], []
-    for src in _sources(src_dir):
-        obj = os.path.join(OBJ, tag + "_" + os.path.relpath(src, src_dir).replace(os.sep, "_") + ".o")
-        objs.append(obj)
-        if force or not os.path.exists(obj) or os.path.getmtime(obj) < max(hdr, os.path.getmtime(src)):
-            jobs.append((src, obj))
+    objs, jobs = _jobs(_sources(src_dir), lambda src: tag + "_" + os.path.relpath(src, src_dir).replace(os.sep, "_"), force, hdr)
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as pool:
-        list(pool.map(lambda j: _compile(j[0], j[1], verbose), jobs))
+        list(pool.map(lambda j: _compile(*j, verbose), jobs))
     if jobs or not os.path.exists(lib_path) or os.path.getmtime(lib_path) < os.path.getmtime(LIB):
         rpath = os.path.relpath(HERE, os.path.dirname(lib_path))
         cmd = ["nvcc", "-shared", "-o", lib_path] + objs + ["-L" + HERE, "-lacc", "-lcudart",

@@ -373,7 +373,7 @@ __device__ __forceinline__ val_of<IX> eval_here(const A& a, const IX& ix) {
       return acc;
     };
     if constexpr (W == 1) {
-      return row_value(ix);
+      return row_value(lane(ix, 0));
     } else if constexpr (std::is_same<IX, IxS4>::value) {
       return V4{{row_value(lane_clamped(ix, 0, a.n[I].C)), row_value(lane_clamped(ix, 1, a.n[I].C)),
                  row_value(lane_clamped(ix, 2, a.n[I].C)), row_value(lane_clamped(ix, 3, a.n[I].C))}};
@@ -393,7 +393,7 @@ __device__ __forceinline__ val_of<IX> eval_here(const A& a, const IX& ix) {
       return acc;
     };
     if constexpr (W == 1) {
-      return seg_value(ix);
+      return seg_value(lane(ix, 0));
     } else if constexpr (std::is_same<IX, IxS4>::value) {
       return V4{{seg_value(lane_clamped(ix, 0, a.n[I].C)), seg_value(lane_clamped(ix, 1, a.n[I].C)),
                  seg_value(lane_clamped(ix, 2, a.n[I].C)), seg_value(lane_clamped(ix, 3, a.n[I].C))}};

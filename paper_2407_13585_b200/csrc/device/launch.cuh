@@ -7,6 +7,7 @@
 #include "../graph.h"
 #include "../registry.h"
 #include "hist.cuh"
+#include "scanring.cuh"
 #include "segfold.cuh"
 #include "skeletons.cuh"
 #include "slabgather.cuh"
@@ -155,6 +156,80 @@ struct Launcher {
     return true;
   }
 
+  // Scans through the shared-memory ring (k_scan_ring), or a warp or block per row where rows are short (k_scan_rows);
+  // without them, where a chunk behind an index map would not be a 128-bit access, k_scan.
+  static constexpr bool kRingShape = kHasScan && dev::scan_ring_eligible<CL>();
+  static bool use_ring(const ClusterLaunch& L, int C) {
+    if constexpr (!kRingShape) return false;
+    else return !dev::has_index_map<CL>() || vec_ok(L, C);
+  }
+  // (a row of C elements may begin up to three words into its first 16-byte chunk)
+  static int ring_tiles_per_row(int R, int C) {
+    if constexpr (kRingShape) return (C + (R > 1 && C % 4 ? 3 : 0) + dev::RingTile<CL>::TILE - 1) / dev::RingTile<CL>::TILE;
+    else return 0;
+  }
+  static int64_t scan_scratch_bytes(const ClusterLaunch& L, int R, int C) {
+    if (use_ring(L, C)) {
+      int per_row = ring_tiles_per_row(R, C);
+      if constexpr (kRingShape) {
+        if constexpr (dev::can_stage<CL>()) per_row = std::max(per_row, Launcher<dev::StagedScan<CL>>::ring_tiles_per_row(R, C));
+      }
+      return 16 + (per_row > 1 ? 2 * (int64_t)dev::count_if<CL>(dev::is_scan_root) * R * per_row * 8 : 0);
+    }
+    return 16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8;
+  }
+
+  // WHOLE: the cluster whose costly members are staged first (this one is then what is left of it), or void.
+  template <class WHOLE = void>
+  static int launch_ring(const ClusterLaunch& L, dev::Args<N>& a, int R, int C, dev::StageArgs<WHOLE, N> whole = {}) {
+    if constexpr (kRingShape) {
+      constexpr int kForms = std::is_void<WHOLE>::value ? dev::ScanForms<CL>::value : 2;
+      if constexpr ((kForms & 1) != 0) {
+        if (C <= dev::kScanWarpRow) {
+          const int warps = dev::kBlock / 32;
+          dev::k_scan_rows<CL, 1, 4><<<(int)std::min<int64_t>((R + warps - 1) / warps, (int64_t)sm_count() * 8), dev::kBlock, 0, L.stream>>>(a);
+        } else if (C <= dev::kScanBlockRow) {
+          const int grid = (int)std::min<int64_t>(R, (int64_t)sm_count() * 8);
+          if (C <= 4096 - 3) dev::k_scan_rows<CL, 16, 2><<<grid, 512, 0, L.stream>>>(a);
+          else dev::k_scan_rows<CL, 16, 8><<<grid, 512, 0, L.stream>>>(a);
+        }
+      }
+      if constexpr ((kForms & 2) != 0) {
+        if (C > dev::kScanBlockRow) {
+          int per_row = ring_tiles_per_row(R, C);
+          const int64_t tiles = (int64_t)R * per_row;
+          if (tiles >= (int64_t(1) << 31)) return set_error(ACC_ERR_SHAPE, "too many rows to scan in one launch");
+          if constexpr (std::is_void<WHOLE>::value && dev::can_stage<CL>()) {
+            dev::Args<N> rest = a;
+            for (int i = 0; i < N; ++i)
+              if (dev::is_costly<CL>(i)) {
+                rest.n[i].ptr = a.n[dev::stage_target<CL>(i)].ptr;
+                rest.n[i].R = R;
+                rest.n[i].C = C;
+              }
+            return Launcher<dev::StagedScan<CL>>::template launch_ring<CL>(L, rest, R, C, dev::StageArgs<CL, N>{a});
+          } else {
+            using K = dev::Ring<CL, dev::ring_resident<CL>()>;
+            int n_tiles = (int)tiles;
+            const void* kern = reinterpret_cast<const void*>(dev::k_scan_ring<CL, WHOLE>);
+            static int granted[64];
+            if (!opt_in_shared_memory(kern, K::SMEM, granted))
+              return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
+            // (blocks read one another's totals: all of them resident)
+            if (!cooperative_launch_ok()) return set_error(ACC_ERR_UNSUPPORTED, "the device cannot launch cooperatively");
+            void* params[] = {&a, &per_row, &n_tiles, &whole};
+            cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tiles, sm_count())), dim3(K::THREADS), params, K::SMEM, L.stream);
+          }
+        }
+      }
+      const cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+      return ACC_OK;
+    } else {
+      return set_error(ACC_ERR_NO_KERNEL, "not a cluster of scans");
+    }
+  }
+
   // Whether the gather below the scan runs as slab passes: decided by shapes alone, so that the scratch
   // layout (which is fixed before any pointer is known) and the launch agree.
   static constexpr bool kSlabShape = dev::slab_gather_eligible<CL>();
@@ -195,12 +270,11 @@ struct Launcher {
       return (dev::tile_partials_off(blocks) + (int64_t)kRowFolds * blocks * R) * 4;
     }
     if (kHasScan) {
-      int64_t bytes = 16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8;
       if (slab_shapes_ok(L, R, C)) {                      // + group sizes and slab codes of the slab passes (slabgather.cuh)
-        const int64_t full = C / dev::kSlabWarpTile;
-        bytes = ((bytes + 15) & ~int64_t(15)) + full * 4 + full * 32 * 4;
+        const int64_t bytes = 16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8, full = C / dev::kSlabWarpTile;
+        return ((bytes + 15) & ~int64_t(15)) + full * 4 + full * 32 * 4;
       }
-      return bytes;
+      return scan_scratch_bytes(L, R, C);
     }
     if (kHasSegFold) return dev::seg_scratch_words(dev::count_if<CL>(dev::is_segfold_root), seg_grid(L)) * 4;
     if (kHasRowFold) return 0;
@@ -220,6 +294,7 @@ struct Launcher {
     if (!domain(L, R, C)) return 0;
     if (use_tiles(L, R, C)) return dev::tile_partials_off((R + dev::kTile - 1) / dev::kTile) * 4;
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
+    if (kHasScan && use_ring(L, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
     if (stream_slab_shapes_ok(L, R, C)) return (((int64_t)dev::stream_acc64_off(kScalarFolds, sm_count() * 8) * 4) + 15) & ~int64_t(15);
     return scratch_bytes(L);
   }
@@ -449,30 +524,31 @@ struct Launcher {
             else
               dev::k_scan_merge<CL><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles, slab);
           }
-          L.extra_launches = 2 + dev::kSlabs;
+          L.extra_launches += 2 + dev::kSlabs;
           const cudaError_t e = cudaGetLastError();
           if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
           return ACC_OK;
         }
       }
-      {
-        // all blocks resident at once where the device can promise it (then tiles need no ticket), else ticketed tiles
-        int per_row_arg = per_row, tiles_arg = (int)tiles;
-        void* params[] = {&a, &per_row_arg, &tiles_arg};
-        static int fit_on[2][64];
-        // (small tiles: with a warp of its own for the look-back, see scan_tiles_pipelined)
-        constexpr bool kPipelined = dev::scan_pipelines<CL>();
-        constexpr int kThreads = kScanBlock + (kPipelined ? 32 : 0);
-        const void* kern;
-        if constexpr (kPipelined)
-          kern = vec ? reinterpret_cast<const void*>(dev::k_scan_pipelined<CL, true>) : reinterpret_cast<const void*>(dev::k_scan_pipelined<CL, false>);
-        else
-          kern = vec ? reinterpret_cast<const void*>(dev::k_scan<CL, true, true>) : reinterpret_cast<const void*>(dev::k_scan<CL, false, true>);
-        const int resident = resident_grid(kern, kThreads, fit_on[vec ? 1 : 0]);
-        if (resident > 0)
-          cudaLaunchCooperativeKernel(const_cast<void*>(kern), dim3((unsigned)std::min<int64_t>(tiles, resident)), dim3(kThreads), params, 0, L.stream);
-        else if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
+      if constexpr (kRingShape) {
+        if constexpr (dev::can_stage<CL>()) {
+          // a gather below the scan and few elements: tiles that look back one after the other, in an ordinary launch, are
+          // quicker than staging in a cooperative one (30000 elements 8.7 against 12.4 us)
+          if (R == 1 && C > dev::kScanBlockRow && C <= dev::kScanFewElements && use_ring(L, C)) {
+            if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
+            else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+            return ACC_OK;
+          }
+        }
+      }
+      if (use_ring(L, C)) return launch_ring(L, a, R, C);
+      if constexpr (!kRingShape) {
+        if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
         else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
+      } else if constexpr (dev::has_index_map<CL>()) {
+        dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
       }
     } else if constexpr (kHasRowFold) {
       if (R == 0) return ACC_OK;
@@ -503,7 +579,7 @@ struct Launcher {
           dev::k_slab_partition<CL><<<pgrid, dev::kBlock, 0, L.stream>>>(a, codes, counts, full, mul, slab);
           for (int k = 0; k < dev::kSlabs; ++k) dev::k_slab_gather<CL><<<ggrid, dev::kBlock, 0, L.stream>>>(a, counts, full, (uint32_t)k, slab);
           dev::k_stream_merge<CL><<<pgrid, dev::kBlock, 0, L.stream>>>(a, slab);
-          L.extra_launches = 2 + dev::kSlabs;
+          L.extra_launches += 2 + dev::kSlabs;
           const cudaError_t e = cudaGetLastError();
           if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
           return ACC_OK;
@@ -564,26 +640,6 @@ constexpr bool is_accumulating_root(const CNode& n) {
   return dev::is_fold_root(n) || dev::is_scan_root(n) || dev::is_permute_root(n);
 }
 
-template <class CL> constexpr PassPlan pass_plan() {
-  PassPlan p;
-  uint64_t folds = 0, permutes = 0;
-  for (int i = 0; i < CL::c.n; ++i) {
-    const CNode& n = CL::c.nodes[i];
-    if (dev::is_scan_root(n)) p.keep[p.n++] = 1ull << i;             // a scan walks alone
-    else if (dev::is_fold_root(n)) folds |= 1ull << i;
-    else if (dev::is_permute_root(n)) permutes |= 1ull << i;
-  }
-  // whole-array folds and scatters share the streaming kernel; row folds have a kernel of their own
-  const bool together = dev::domain_rank<CL>() <= 1 || !folds || !permutes;
-  if (together) {
-    if (p.n == 0 || (folds | permutes)) p.keep[p.n++] = folds | permutes;
-  } else {
-    p.keep[p.n++] = folds;
-    p.keep[p.n++] = permutes;
-  }
-  return p;
-}
-
 // The scan whose values element-wise member i consumes inside the cluster, -1 if none.
 constexpr int scan_needed_by(const CCluster& c, int i) {
   for (int s = 0; s < c.n; ++s)
@@ -600,15 +656,12 @@ constexpr CNode unread_array(const CNode& n) {
 // root of the pass reaches any more, and the roots of other passes, become arrays nobody reads.
 constexpr CCluster pass_cluster(CCluster c, uint64_t keep, bool first) {
   const CCluster whole = c;
-  int scan = -1;
-  for (int i = 0; i < c.n; ++i)
-    if (((keep >> i) & 1) && dev::is_scan_root(whole.nodes[i])) scan = i;
   for (int i = 0; i < c.n; ++i) {
     if (is_accumulating_root(whole.nodes[i]) && !((keep >> i) & 1)) {
       c.nodes[i] = unread_array(whole.nodes[i]);
     } else if (dev::is_store_root(whole.nodes[i])) {
       const int needs = scan_needed_by(whole, i);
-      if (needs >= 0 ? needs != scan : !first) c.nodes[i].manifest = false;
+      if (needs >= 0 ? ((keep >> needs) & 1) == 0 : !first) c.nodes[i].manifest = false;
     }
   }
   bool live[kMaxCluster] = {};
@@ -624,55 +677,128 @@ constexpr CCluster pass_cluster(CCluster c, uint64_t keep, bool first) {
   return c;
 }
 
-template <class CL, int P>
+constexpr uint64_t scans_of_kind(const CCluster& c, int kind) {
+  uint64_t m = 0;
+  for (int i = 0; i < c.n; ++i)
+    if (dev::is_scan_root(c.nodes[i]) && c.nodes[i].kind == kind) m |= 1ull << i;
+  return m;
+}
+// Whether the scans of one direction can share a walk: as one pass they must be something k_scan_ring takes, whatever
+// the shapes.  (Each array is then read once for all of them.)
+template <class CL, int KIND>
+struct ScansTogether {
+  static constexpr CCluster c = pass_cluster(CL::c, scans_of_kind(CL::c, KIND), true);
+};
+template <class CL, int KIND> constexpr bool scans_share_a_pass() {
+  if constexpr (scans_of_kind(CL::c, KIND) == 0) return false;
+  else return dev::scan_ring_eligible<ScansTogether<CL, KIND>>() && !dev::has_index_map<ScansTogether<CL, KIND>>();
+}
+
+// TOGETHER: the scans of one direction share a pass where they can.
+template <class CL, bool TOGETHER> constexpr PassPlan pass_plan() {
+  PassPlan p;
+  uint64_t folds = 0, permutes = 0;
+  for (int kind : {(int)ACC_SCANL, (int)ACC_SCANR}) {
+    const uint64_t scans = scans_of_kind(CL::c, kind);
+    const bool together = TOGETHER && (kind == ACC_SCANL ? scans_share_a_pass<CL, ACC_SCANL>() : scans_share_a_pass<CL, ACC_SCANR>());
+    if (scans && together) p.keep[p.n++] = scans;                   // one walk for all scans of a direction
+    else
+      for (int i = 0; i < CL::c.n; ++i)
+        if ((scans >> i) & 1) p.keep[p.n++] = 1ull << i;             // a scan walks alone
+  }
+  for (int i = 0; i < CL::c.n; ++i) {
+    const CNode& n = CL::c.nodes[i];
+    if (dev::is_fold_root(n)) folds |= 1ull << i;
+    else if (dev::is_permute_root(n)) permutes |= 1ull << i;
+  }
+  // whole-array folds and scatters share the streaming kernel; row folds have a kernel of their own
+  const bool together = dev::domain_rank<CL>() <= 1 || !folds || !permutes;
+  if (together) {
+    if (p.n == 0 || (folds | permutes)) p.keep[p.n++] = folds | permutes;
+  } else {
+    p.keep[p.n++] = folds;
+    p.keep[p.n++] = permutes;
+  }
+  return p;
+}
+
+template <class CL, bool TOGETHER, int P>
 struct PassOf {
-  static constexpr CCluster c = pass_cluster(CL::c, pass_plan<CL>().keep[P], P == 0);
+  static constexpr int kScanForms = pass_plan<CL, false>().n == pass_plan<CL, true>().n ? 3 : TOGETHER ? 2 : 1;
+  static constexpr CCluster c = pass_cluster(CL::c, pass_plan<CL, TOGETHER>().keep[P], P == 0);
 };
 
 template <class CL>
 struct Passes {
-  static constexpr PassPlan plan = pass_plan<CL>();
+  static constexpr int kSingly = pass_plan<CL, false>().n, kTogether = pass_plan<CL, true>().n;
 
-  template <int P>
+  // Scans share a pass where they go through the ring (long rows); k_scan_rows keeps a row's operands in registers and
+  // takes one scan at a time.
+  static bool together(const ClusterLaunch& L) {
+    if constexpr (kSingly == kTogether) return false;
+    else {
+      int R, C;
+      return Launcher<CL>::domain(L, R, C) && C > dev::kScanBlockRow;
+    }
+  }
+
+  template <bool T, int P>
   static int64_t scratch_from(const ClusterLaunch& L) {
-    if constexpr (P < plan.n) {
-      const int64_t here = Launcher<PassOf<CL, P>>::scratch_bytes(L);
+    if constexpr (P < pass_plan<CL, T>().n) {
+      const int64_t here = Launcher<PassOf<CL, T, P>>::scratch_bytes(L);
       if (here < 0) return here;
-      const int64_t rest = scratch_from<P + 1>(L);
+      const int64_t rest = scratch_from<T, P + 1>(L);
       return rest < 0 ? rest : ((here + 255) & ~int64_t(255)) + rest;
     } else {
       return 0;
     }
   }
+  template <bool T> static int64_t all_scratch(const ClusterLaunch& L) {
+    if constexpr (pass_plan<CL, T>().n <= 1) return Launcher<CL>::scratch_bytes(L);
+    else return scratch_from<T, 0>(L);
+  }
   static int64_t scratch_bytes(const ClusterLaunch& L) {
-    if constexpr (plan.n <= 1) return Launcher<CL>::scratch_bytes(L);
-    else return scratch_from<0>(L);
+    if constexpr (kSingly != kTogether) {
+      if (together(L)) return all_scratch<true>(L);
+    }
+    return all_scratch<false>(L);
   }
   static int64_t zeroed_bytes(const ClusterLaunch& L) {
-    if constexpr (plan.n <= 1) return Launcher<CL>::zeroed_bytes(L);
-    else return scratch_from<0>(L);                   // the passes' regions follow one another: all of it
+    if constexpr (kSingly <= 1) return Launcher<CL>::zeroed_bytes(L);
+    else return scratch_bytes(L);                     // the passes' regions follow one another: all of it
   }
 
-  template <int P>
+  template <bool T, int P>
   static int launch_from(ClusterLaunch& L) {
-    if constexpr (P < plan.n) {
-      const int64_t here = Launcher<PassOf<CL, P>>::scratch_bytes(L);
+    if constexpr (P < pass_plan<CL, T>().n) {
+      const int64_t here = Launcher<PassOf<CL, T, P>>::scratch_bytes(L);
       if (here < 0) return (int)here;
-      const int rc = Launcher<PassOf<CL, P>>::launch(L);
+      const int rc = Launcher<PassOf<CL, T, P>>::launch(L);
       if (rc != ACC_OK) return rc;
       L.scratch += ((here + 255) & ~int64_t(255)) / 4;
-      return launch_from<P + 1>(L);
+      return launch_from<T, P + 1>(L);
     } else {
       return ACC_OK;
     }
   }
-  static int launch(const ClusterLaunch& L) {
-    if constexpr (plan.n <= 1) {
+  template <bool T> static int launch_all(const ClusterLaunch& L) {
+    if constexpr (pass_plan<CL, T>().n <= 1) {
       return Launcher<CL>::launch(L);
     } else {
       ClusterLaunch pass = L;
-      return launch_from<0>(pass);
+      const int rc = launch_from<T, 0>(pass);
+      L.extra_launches += pass.extra_launches;
+      return rc;
     }
+  }
+  static int launch(const ClusterLaunch& L) {
+    if constexpr (kSingly != kTogether) {
+      if (together(L)) {
+        L.extra_launches += kTogether - kSingly;      // (the entry counts a pass per scan)
+        return launch_all<true>(L);
+      }
+    }
+    return launch_all<false>(L);
   }
 };
 
@@ -682,15 +808,24 @@ struct Registrar {
     // (a cluster of segmented folds is a walk over the elements and a small second launch for the segments that
     // cross its blocks)
     register_kernel(KernelEntry{signature(CL::c), name, &Passes<CL>::scratch_bytes, &Passes<CL>::zeroed_bytes, &Passes<CL>::launch,
-                                Passes<CL>::plan.n > 1 ? Passes<CL>::plan.n : (dev::count_if<CL>(dev::is_segfold_root) > 0 ? 2 : 1)});
+                                Passes<CL>::kSingly > 1 ? Passes<CL>::kSingly : (dev::count_if<CL>(dev::is_segfold_root) > 0 ? 2 : 1)});
   }
 };
+
+// A file of many clusters is compiled in ACC_PARTS parts, each of which registers every ACC_PARTS-th cluster (the build sets
+// both; one part where they are not set).
+#ifndef ACC_PARTS
+#define ACC_PARTS 1
+#define ACC_PART 0
+#endif
+template <class CL, bool HERE> struct PartRegistrar : Registrar<CL> { using Registrar<CL>::Registrar; };
+template <class CL> struct PartRegistrar<CL, false> { explicit PartRegistrar(const char*) {} };
 
 #define ACC_CAT2(a, b) a##b
 #define ACC_CAT(a, b) ACC_CAT2(a, b)
 // Instantiates the kernels of cluster MASK of program PROG and registers them under NAME.
 #define ACC_CLUSTER(PROG, MASK, NAME)                                              \
   struct ACC_CAT(Cl_, NAME) { static constexpr CCluster c = extract(PROG, MASK); }; \
-  static Registrar<ACC_CAT(Cl_, NAME)> ACC_CAT(reg_, NAME)(#NAME);
+  static PartRegistrar<ACC_CAT(Cl_, NAME), __COUNTER__ % ACC_PARTS == ACC_PART> ACC_CAT(reg_, NAME)(#NAME);
 
 }  // namespace acc

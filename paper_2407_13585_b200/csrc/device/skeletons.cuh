@@ -930,16 +930,9 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
   if (round > 0) finish((int)blockIdx.x + (round - 1) * G, (round - 1) & 1);
 }
 
-template <class CL, bool VEC, bool STATIC = false>
-__global__ void __launch_bounds__(scan_block<CL>()) k_scan(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles) {
-  scan_tiles<CL, VEC, false, STATIC>(a, tiles_per_row, n_tiles, SlabIn{});
-}
-
-// (a tile's values stay in shared memory twice over: only for tiles of at most 16 KB)
-template <class CL> constexpr bool scan_pipelines() { return scan_block<CL>() * scan_rows<CL>() * 4 <= 4096; }
 template <class CL, bool VEC>
-__global__ void __launch_bounds__(scan_block<CL>() + 32) k_scan_pipelined(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles) {
-  if constexpr (scan_pipelines<CL>()) scan_tiles_pipelined<CL, VEC, false>(a, tiles_per_row, n_tiles, SlabIn{});
+__global__ void __launch_bounds__(scan_block<CL>()) k_scan(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles) {
+  scan_tiles<CL, VEC, false>(a, tiles_per_row, n_tiles, SlabIn{});
 }
 
 }  // namespace dev

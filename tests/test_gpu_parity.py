@@ -557,6 +557,33 @@ def test_row_scans_both_directions(rows, cols):
     check_program(W.row_scans(rows, cols))
 
 
+# tiles of the shared-memory ring: the largest row a block takes by itself and the smallest that goes through the ring; rows
+# that begin anywhere in a 16-byte chunk and cross tiles; a few rounds of the grid (every block adds up the totals) and many
+# (the first block does); the array's last words beyond its last whole chunk
+@pytest.mark.parametrize("rows,cols", [(3, 4093), (3, 4094), (2, 16381), (2, 16382), (5, 20001), (41, 90001), (90, 90002), (1, 148 * 8 * 5120 + 5)])
+def test_row_scans_through_the_ring(rows, cols):
+    prog = W.row_scans(rows, cols)
+    assert check_program(prog) == 3
+
+
+# two sums in one walk beside a scan in the other direction, on lengths around a round of the grid and its eighth
+@pytest.mark.parametrize("n", [16382, 3072 * 148 + 1, 3072 * 148 * 8 + 2, 3072 * 148 * 9 - 1])
+def test_scans_that_share_a_walk(n):
+    prog = W.scan_consumers(n)
+    check_program(prog, [[-1, -1, 0, 0, 0, 1, 1, 0, 0]], passes=True)
+    _, g = gpu_run(prog, W.make_inputs(prog), [-1, -1, 0, 0, 0, 1, 1, 0, 0])
+    assert g.launch_count() == 2
+
+
+# a gather below a scan: in one row of a block, behind tickets, and staged by the blocks of the ring
+@pytest.mark.parametrize("n", [16383, 131072, 131073, 700001])
+def test_gather_staged_for_a_scan(n):
+    prog = W.config3(n)
+    prog.name = "fixture"                     # generic index inputs bounded by n
+    prog.index_bound = {"idx": n, "x": 1 << 30}
+    check_program(prog, [[-1, -1, 0, 0, 0, 0], [-1, -1, 0, 1, 1, 1]])
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))
