@@ -131,13 +131,13 @@ struct Launcher {
     }
   }
 
-  // blocks of k_segfold: one per run of kSegTilesPerBlock tiles of the folds' source (its records are laid out for them)
+  // blocks of k_segfold: one per eight warps' runs of the folds' source (its records are laid out for them)
   static int seg_grid(const ClusterLaunch& L) {
     if constexpr (kHasSegFold) {
       const int src = CL::c.nodes[dev::first_segfold<CL>()].in[0];
       const int64_t n_src = (int64_t)L.nodes[src].R * L.nodes[src].C;
-      const int64_t tiles = std::max<int64_t>(1, (n_src + dev::kSegTile - 1) / dev::kSegTile);
-      return (int)((tiles + dev::kSegTilesPerBlock - 1) / dev::kSegTilesPerBlock);
+      const int64_t span = (int64_t)dev::seg_run(n_src, sm_count()) * (dev::kBlock / 32);
+      return (int)std::max<int64_t>(1, (n_src + span - 1) / span);
     } else {
       return 0;
     }
@@ -465,16 +465,12 @@ struct Launcher {
     if constexpr (kHasSegFold) {
       if constexpr (dev::segfold_eligible<CL>()) {
         if (C == 0) return ACC_OK;
-        constexpr int NFOLD = dev::count_if<CL>(dev::is_segfold_root);
         const int grid = seg_grid(L);
-        const int per_block = dev::kSegTilesPerBlock;
-        const bool v4 = seg_vec_ok(L);
-        const size_t smem = v4 ? 0 : (size_t)NFOLD * dev::kSegTile * 4;    // operands are staged only where rows are not 128-bit friendly
-        auto kern = v4 ? dev::k_segfold<CL, true> : dev::k_segfold<CL, false>;
-        static int granted[2][64];
-        if (smem > 48 * 1024 && !opt_in_shared_memory(kern, smem, granted[v4 ? 1 : 0]))
-          return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
-        kern<<<grid, dev::kBlock, smem, L.stream>>>(a, per_block);
+        // (chunks of four start on 16 bytes whatever the length; behind an index map they need 128-bit rows)
+        const int src = CL::c.nodes[dev::first_segfold<CL>()].in[0];
+        const int run = dev::seg_run((int64_t)L.nodes[src].R * L.nodes[src].C, sm_count());
+        if (!dev::has_index_map<CL>() || seg_vec_ok(L)) dev::k_segfold<CL, true><<<grid, dev::kBlock, 0, L.stream>>>(a, run);
+        else dev::k_segfold<CL, false><<<grid, dev::kBlock, 0, L.stream>>>(a, run);
         dev::k_segfold_across<CL><<<(grid + dev::kBlock / 32 - 1) / (dev::kBlock / 32), dev::kBlock, 0, L.stream>>>(a, grid);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));

@@ -5,42 +5,49 @@
 // The work is cut by elements, not by segments, so that a few very long segments among many
 // short ones (skewed lengths) cost what their elements cost:
 //
-//  * the source range is cut into tiles of kSegTile elements; a block owns a contiguous run of
-//    tiles and walks it in order.  A run of tiles that lies inside one segment is streamed;
-//  * any other tile, where the arrays have 128-bit rows: its operands stay in registers, a bit per
-//    element marks where segments begin, and a segmented scan (inside a chunk, across a warp by
-//    shuffles, across the tile through 32 partial values) gives every element the sum of its
-//    segment so far; the elements that end a segment write it.  Uniform work whatever the lengths;
-//  * without 128-bit rows the tile's operands are staged in shared memory and the pieces of
-//    segments are reduced from there: a thread per piece up to kSegShort elements, a warp per
-//    piece up to kSegMedium, the whole block beyond;
-//  * a piece that is a whole segment is written at once.  A segment that crosses tiles is carried
-//    by the block from tile to tile (a compensated running value in one thread); one that crosses
-//    blocks leaves a record per block (the part after its start: `tail`; a part that continues
-//    one begun earlier: `head`), and a second, small launch (k_segfold_across) combines the
+//  * a warp owns kSegRun consecutive elements and walks them 512 at a time, without a barrier: the
+//    warps of a block meet once, at the end;
+//  * where no segment begins among the 512, every lane adds its elements to a compensated running
+//    value of its own;
+//  * otherwise the offsets that fall among them become bits, the operands go through shared memory so
+//    that a lane holds 16 consecutive ones, and a segmented scan (inside the lane, then once across the
+//    warp by shuffles that stop at a lane holding a start) leaves the value of every prefix there; a
+//    lane per start then takes the value in front of it, which is the segment that ends;
+//  * a segment that crosses warps is put together by one thread of the block (fp32 sums in fp64); one
+//    that crosses blocks leaves a record per block (the part after its start: `tail`; a part that
+//    continues one begun earlier: `head`), and a second, small launch (k_segfold_across) combines the
 //    records in block order.
+//
+// (Before, a block walked tiles of 4096 elements with ten barriers each, about 800 instructions per
+// thread where a tile held several segments, and sources without 128-bit rows went through shared
+// memory element by element.  2^27 elements, a sum and a maximum: 2^20 segments of
+// Zipf lengths 243 -> 188 us, 2^15 segments 184 -> 150, 2^24 segments 450 -> 431; 10^6 elements in 10^4 segments 42.5 ->
+// 16.5.  What bounds it now is latency: a warp's step waits for its loads, then for the scan's shuffles, with 34 % of the issue
+// slots used.)
 //
 // Several segmented folds of one cluster (say a sum and a maximum over the same segments) share
 // the walk.  Results do not depend on timing: every order of combination is fixed by the layout.
 //
 // Offsets are data, so they are checked here, every one of them: a segment that leaves the
 // source is reported as ACC_ERR_INDEX_RANGE, an empty or descending one as ACC_ERR_SHAPE (a fold
-// has no seed, so an empty segment has no value); pieces are clamped to their tile, so bad
-// offsets cannot make the kernel read or write outside its arrays.
+// without a seed has no value for it).
 #pragma once
+#include "scanring.cuh"
 #include "skeletons.cuh"
 
 namespace acc {
 namespace dev {
 
-constexpr int kSegTile = 4096;                 // elements per tile
-constexpr int kSegShort = 32;                  // pieces up to here: one thread
-constexpr int kSegMedium = 1024;               // pieces up to here: one warp; longer ones: the block
-constexpr int kSegListCap = kSegTile / (kSegShort + 1) + 2;
-constexpr int kSegBigCap = kSegTile / (kSegMedium + 1) + 2;    // pieces of a tile the whole block reduces
+constexpr int kSegStep = 512;                  // elements of a warp's step
+constexpr int kSegMaxRun = 4096;               // consecutive elements of a warp, at most: what amortises finding its first segment
+constexpr int kSegStride = 20;                 // words a lane's 16 elements take in shared memory: an odd multiple of 16 bytes, no bank conflicts
+// Elements of a warp's run: a step where that is what it takes to have a run for 32 warps on every SM (a step takes 2 to 3 us
+// of latency), up to kSegMaxRun.
+inline int seg_run(int64_t n, int sms) {
+  const int64_t steps = n / ((int64_t)sms * 32 * kSegStep);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(steps, kSegMaxRun / kSegStep)) * kSegStep;
+}
 constexpr int kSegResident = 4;                // blocks per SM the kernel is built for
-constexpr int kSegTilesPerBlock = 8;           // a block's run of tiles: short enough for the block scheduler to even out slow and fast runs
-constexpr int kSegWindow = 1024;               // offsets kept in shared memory at a time
 
 template <class CL> constexpr int first_segfold() {
   for (int i = 0; i < CL::c.n; ++i)
@@ -81,29 +88,26 @@ __device__ __forceinline__ int seg_containing(const int32_t* off, int S, int x, 
 }
 
 template <class CL, bool VEC>
-__global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_constant__ Args<CL::c.n> a, int tiles_per_block) {
+__global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_constant__ Args<CL::c.n> a, int run_length) {
   constexpr int N = CL::c.n;
   constexpr int F = first_segfold<CL>();
   constexpr int NF = count_if<CL>(is_segfold_root);
-  constexpr int WARPS = kBlock / 32;
+  constexpr int WARPS = kBlock / 32, ROWS = 4, STEP = kSegStep;
   constexpr int REC = 2 + NF;
-  extern __shared__ __align__(16) uint32_t seg_vals[];                         // NF arrays of kSegTile operand values
-  __shared__ uint32_t red[WARPS];
-  __shared__ int off_win[kSegWindow + 1];                        // offsets of segments win_base .. win_base + kSegWindow
-  __shared__ int long_seg[kSegListCap], long_lo[kSegListCap], long_hi[kSegListCap], long_kind[kSegListCap];
-  __shared__ int big_seg[kSegBigCap], big_lo[kSegBigCap], big_hi[kSegBigCap], big_kind[kSegBigCap];
-  __shared__ uint32_t seg_bits[VEC ? kSegTile / 32 + 2 : 1];      // bit p: element p of the tile begins a segment
-  __shared__ int seg_before[VEC ? kSegTile / 32 : 1];            // starts before each 32-element word
-  __shared__ uint32_t seg_unit_flag[VEC ? 32 : 1], seg_unit_val[VEC ? NF : 1][VEC ? 32 : 1];
-  __shared__ int tile_open;
-  __shared__ int n_long, n_big, next_s, first_open, have_first, have_last, last_seg;
-  __shared__ uint32_t first_val[NF], last_val[NF];
+  __shared__ uint32_t bits[WARPS][STEP / 32];                    // bit p: element p of the warp's step begins a segment
+  __shared__ __align__(16) uint32_t staged[WARPS][32 * kSegStride];   // a step's operands, then the value of every prefix within its lane
+  // what a warp leaves for the block: the segment that is open at its end and its value there, and, where a segment begins
+  // in the warp's run, that segment and the value of the one that ends at the first start
+  __shared__ int open_seg[WARPS], first_seg[WARPS];              // first_seg: -1 if none begins; open_seg -1: no elements
+  __shared__ bool has_head[WARPS];                               // the segment that ends at the first start has elements in the run
+  __shared__ uint32_t open_val[NF][WARPS], head_val[NF][WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int S = a.C;                                             // segments
   constexpr int OFF = CL::c.nodes[F].in[1], SRC = CL::c.nodes[F].in[0];
   const int32_t* off = reinterpret_cast<const int32_t*>(a.n[OFF].ptr);
   const int n_src = a.n[SRC].R * a.n[SRC].C;
   uint32_t* rec = a.scratch + 4;
+  auto fold_slot_of = [](int i) { return count_if<CL>(is_segfold_root, i); };
 
   // every offset is looked at once, whatever the walk below does with it
   for (int s = blockIdx.x * kBlock + threadIdx.x; s < S; s += gridDim.x * kBlock) {
@@ -112,422 +116,261 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
     else if (hi <= lo) raise_status(a, kStatusEmptySegment);
   }
 
-  auto fold_slot_of = [](int i) { return count_if<CL>(is_segfold_root, i); };
-  // kind of a piece: bit 0 = it continues a segment begun before the tile, bit 1 = its segment goes on after the tile
-  auto store_piece = [&](int s, int kind, const uint32_t (&v)[N]) {
-    static_for<0, N>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      if constexpr (is_segfold_root(CL::c.nodes[i])) {
-        const int f = fold_slot_of(i);
-        if (kind & 1) first_val[f] = v[i];
-        else if (kind & 2) last_val[f] = v[i];
-        else reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr))[s] = v[i];
-      }
-    });
-    if (kind & 1) { have_first = 1; first_open = kind >> 1; }
-    else if (kind & 2) { have_last = 1; last_seg = s; }
-  };
-  // Inside a tile sums are plain: a thread adds at most 32 staged values and trees do the rest, which
-  // stays far inside the tolerance; what is compensated is the running value a segment keeps from
-  // tile to tile (thousands of steps for a long one).
-  auto reduce_strided = [&](int plo, int phi, int first, int stride, int tile_lo, uint32_t (&v)[N]) {
-    uint32_t w[4][N];
-    static_for<0, N>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      constexpr CNode nd = CL::c.nodes[i];
-      if constexpr (is_segfold_root(nd)) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) w[u][i] = identity_of<nd.fn, nd.dtype>();
-      }
-    });
-    int j = plo + first;
-    for (; j + 3 * stride < phi; j += 4 * stride) {              // four independent running values per fold
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) {
-          const uint32_t* src = seg_vals + fold_slot_of(i) * kSegTile - tile_lo;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) w[u][i] = combine<nd.fn, nd.dtype>(w[u][i], src[j + u * stride]);
-        }
-      });
-    }
-    for (; j < phi; j += stride) {
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) w[0][i] = combine<nd.fn, nd.dtype>(w[0][i], (seg_vals + fold_slot_of(i) * kSegTile - tile_lo)[j]);
-      });
-    }
-    static_for<0, N>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      constexpr CNode nd = CL::c.nodes[i];
-      if constexpr (is_segfold_root(nd))
-        v[i] = combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(w[0][i], w[1][i]), combine<nd.fn, nd.dtype>(w[2][i], w[3][i]));
-    });
-  };
-
   const int e_lo = max(__ldg(off), 0), e_hi = min(__ldg(off + S), n_src);   // elements that belong to segments
-  const int first_tile = blockIdx.x * tiles_per_block;
-  int s_cur = 0;                                                 // the segment that holds the next element to process (uniform)
-  int win_base = -1;                                             // first segment of the offsets window, -1: not filled (uniform)
-  // the block's carry: the running value of the segment that is open at the end of the last tile (thread 0)
-  int carry_seg = -1;
-  bool carry_from_here = false;
-  uint32_t carry[N];
-  float carry_comp[N] = {};
-
-  for (int t = 0; t < tiles_per_block; ++t) {                    // (a run of tiles inside one segment advances t by its length)
-    const int64_t tile_lo64 = (int64_t)(first_tile + t) * kSegTile;
-    if (tile_lo64 >= e_hi) break;
-    const int tile_lo = (int)tile_lo64;
-    const int tile_hi = (int)(tile_lo64 + kSegTile < (int64_t)e_hi ? tile_lo64 + kSegTile : (int64_t)e_hi);
-    const int lo0 = max(tile_lo, e_lo);
-    if (lo0 >= tile_hi) continue;
-    __syncthreads();                                             // the previous tile's values and flags have been read
-    if (win_base < 0) {                                          // the block's first tile: which segment holds its first element
-      if (warp == 0) {
-        const int s0 = seg_containing(off, S, lo0, lane);
-        if (lane == 0) next_s = s0;
+  const int64_t run_lo = ((int64_t)blockIdx.x * WARPS + warp) * run_length;
+  const int lo0 = (int)(run_lo > e_lo ? run_lo : e_lo), hi0 = (int)(run_lo + run_length < e_hi ? run_lo + run_length : e_hi);
+  if (lane == 0) { open_seg[warp] = -1; first_seg[warp] = -1; }
+  if (lo0 < hi0) {                                               // uniform
+    // the elements of a step; what lies outside [lo0, hi0) reads as the operator's identity
+    auto operands = [&](auto ic, int base, uint32_t (&x)[ROWS][4]) {
+      constexpr int i = decltype(ic)::value;
+      constexpr CNode nd = CL::c.nodes[i];
+      if constexpr (VEC) {
+        // (chunks outside the array read its last whole chunk instead, without a branch: a load whose value is used inside a
+        // branch is waited for before the next one is issued)
+        const int last = (n_src & ~3) - 4;
+        const bool whole = base >= lo0 && base + STEP <= hi0;     // uniform
+        if (last >= 0) {
+#pragma unroll
+          for (int j = 0; j < ROWS; ++j) {
+            const V4 v = eval<CL, nd.in[0]>(a, Ix4{0, min(base + (j * 32 + lane) * 4, last)});
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[j][e] = v.v[e];
+          }
+        }
+        if (!whole) {
+#pragma unroll
+          for (int j = 0; j < ROWS; ++j) {
+            const int c = base + (j * 32 + lane) * 4;
+            if (c > last && c < n_src) {                         // the array's last few elements
+#pragma unroll
+              for (int e = 0; e < 3; ++e)
+                if (c + e < n_src) x[j][e] = eval<CL, nd.in[0]>(a, Ix{0, c + e});
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (c + e < lo0 || c + e >= hi0) x[j][e] = identity_of<nd.fn, nd.dtype>();
+          }
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < ROWS; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int p = base + (j * 32 + lane) * 4 + e;
+            x[j][e] = p >= lo0 && p < hi0 ? eval<CL, nd.in[0]>(a, Ix{0, p}) : identity_of<nd.fn, nd.dtype>();
+          }
       }
-      __syncthreads();
-      s_cur = next_s;
-      __syncthreads();
-    }
-    // uniform: the window of offsets moves to s_cur (back to it where the walk over the last tile's segments moved the
-    // window past the segment that straddles the tile's end)
-    if (win_base < 0 || s_cur < win_base || s_cur + kBlock > win_base + kSegWindow) {
-      win_base = s_cur;
-      for (int k = threadIdx.x; k <= kSegWindow; k += kBlock) off_win[k] = s_cur + k <= S ? __ldg(off + s_cur + k) : 0x7FFFFFFF;
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) { n_long = 0; n_big = 0; have_first = 0; have_last = 0; first_open = 0; next_s = s_cur; }
-    // Tiles that lie inside one segment need no staging: the block streams through all of them that are
-    // its own, every thread keeping a compensated running value per fold, and reduces once at the end.
-    const int lo_c = off_win[s_cur - win_base], hi_c = off_win[s_cur - win_base + 1];
-    const bool whole = s_cur < S && lo_c <= lo0 && hi_c >= tile_hi && lo0 == tile_lo && tile_hi - tile_lo == kSegTile;
-    if (whole) {                                                 // uniform
-      const int own_end = first_tile + tiles_per_block;          // first tile that is not this block's
-      const int inside_end = min(hi_c, e_hi) / kSegTile;         // first tile that is not wholly inside the segment
-      const int run = max(1, min(own_end, inside_end) - (first_tile + t));
-      const int run_hi = tile_lo + run * kSegTile;               // (no overflow: run_hi <= e_hi)
-      uint32_t acc[N];
-      float comp[N] = {};
+    };
+    const int s0 = seg_containing(off, S, lo0, lane);
+    int next = __ldg(off + s0) == lo0 ? s0 : s0 + 1;             // the next segment to begin
+    const int first = next;
+    const bool starts_with_run = __ldg(off + s0) == lo0;
+    // where segments next .. next + 32 * AHEAD - 1 begin: enough for a step of short segments, loaded while the step before is
+    // worked on (a refill within the step is a wait)
+    constexpr int AHEAD = 3;
+    int o[AHEAD];
+    auto refill = [&](int from) {
+#pragma unroll
+      for (int u = 0; u < AHEAD; ++u) o[u] = from + 32 * u + lane < S ? __ldg(off + from + 32 * u + lane) : 0x7FFFFFFF;
+    };
+    refill(next);
+    uint32_t acc[N], open[N];                                    // the open segment: this lane's share of rows without a start, and the rest
+    float comp[N] = {};
+    uint32_t head[N];                                            // (in the lane that finds it)
+    bool found_head = false;
+    static_for<0, N>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      constexpr CNode nd = CL::c.nodes[i];
+      if constexpr (is_segfold_root(nd)) acc[i] = open[i] = identity_of<nd.fn, nd.dtype>();
+    });
+    for (int base = (int)run_lo; base < hi0; base += STEP) {
+      if (base + STEP <= lo0) continue;
+      uint32_t x[N][ROWS][4];
       static_for<0, N>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) acc[i] = identity_of<nd.fn, nd.dtype>();
+        if constexpr (is_segfold_root(CL::c.nodes[i])) operands(ic, base, x[i]);
       });
-      if constexpr (VEC) {
-        // a tile is four trips of the block, so the run is a whole number of these steps: four chunks in flight per fold
-        for (int c = tile_lo + (int)threadIdx.x * 4; c < run_hi; c += kSegTile) {
+      if constexpr (VEC) {                                       // the next step's lines, asked into L2
+        if (base + 2 * STEP <= hi0 && (lane & 7) == 0) {
           static_for<0, N>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
-            constexpr CNode nd = CL::c.nodes[i];
-            if constexpr (is_segfold_root(nd)) {
-              V4 x[kSegTile / (4 * kBlock)];
+            if constexpr (is_segfold_root(CL::c.nodes[i])) {
 #pragma unroll
-              for (int u = 0; u < kSegTile / (4 * kBlock); ++u) x[u] = eval<CL, nd.in[0]>(a, Ix4{0, c + u * kBlock * 4});
-#pragma unroll
-              for (int u = 0; u < kSegTile / (4 * kBlock); ++u)
-                fold_step<nd.fn, nd.dtype>(acc[i], comp[i], combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(x[u].v[0], x[u].v[1]),
-                                                                                     combine<nd.fn, nd.dtype>(x[u].v[2], x[u].v[3])));
+              for (int j = 0; j < ROWS; ++j) eval<CL, CL::c.nodes[i].in[0]>(a, IxPF4{0, base + STEP + (j * 32 + lane) * 4});
             }
           });
         }
-      } else {
-        for (int q = tile_lo + (int)threadIdx.x; q < run_hi; q += kBlock) {
-          static_for<0, N>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr CNode nd = CL::c.nodes[i];
-            if constexpr (is_segfold_root(nd)) fold_step<nd.fn, nd.dtype>(acc[i], comp[i], eval<CL, nd.in[0]>(a, Ix{0, q}));
-          });
-        }
       }
-      uint32_t v[N];
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) v[i] = block_reduce<nd.fn, nd.dtype>(acc[i], red);
-      });
-      if (threadIdx.x == 0) {
-        store_piece(s_cur, (lo_c < lo0 ? 1 : 0) | (hi_c > run_hi ? 2 : 0), v);
-        next_s = hi_c > run_hi ? s_cur : s_cur + 1;
-      }
-      t += run - 1;
-    } else if constexpr (VEC) {
-      // ---- a tile with pieces of several segments, 128-bit rows: a segmented scan over the tile in registers ----
-      // Thread t holds chunks (j * kBlock + t) * 4, j = 0..3, of the tile; in the order (j, warp, lane, element) the
-      // values form one sequence.  `bits` marks the elements that begin a segment.  Every element gets the sum of
-      // its segment up to itself: inside a chunk, across the lanes of a warp (a shuffle scan that stops at lanes
-      // holding a start), across the 32 (row, warp) units through shared memory; elements that end a segment
-      // (the next one begins one, or the tile ends) then hold that segment's sum over the tile and write it.
-      constexpr int ROWS = kSegTile / (4 * kBlock);
-      static_assert(ROWS * WARPS == 32, "the (row, warp) units of a tile are scanned by the lanes of one warp");
-      uint32_t xv[N][ROWS][4];
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) {
-#pragma unroll
-          for (int j = 0; j < ROWS; ++j) {
-            const int c = tile_lo + (j * kBlock + (int)threadIdx.x) * 4;
-            V4 v = V4{{identity_of<nd.fn, nd.dtype>(), identity_of<nd.fn, nd.dtype>(), identity_of<nd.fn, nd.dtype>(), identity_of<nd.fn, nd.dtype>()}};
-            if (c < tile_hi) v = eval<CL, nd.in[0]>(a, Ix4{0, c});
-#pragma unroll
-            for (int e = 0; e < 4; ++e) xv[i][j][e] = c + e < tile_hi ? v.v[e] : identity_of<nd.fn, nd.dtype>();
-          }
-        }
-      });
-      for (int k = threadIdx.x; k < kSegTile / 32 + 2; k += kBlock) seg_bits[k] = 0;
-      if (threadIdx.x == 0) tile_open = 0;
-      __syncthreads();
-      for (int base = s_cur;; base += kBlock) {                  // a thread per segment: where it begins, if that is in the tile
-        if (base + kBlock > win_base + kSegWindow) {             // uniform: the window moves up to `base`
-          __syncthreads();
-          win_base = base;
-          for (int k = threadIdx.x; k <= kSegWindow; k += kBlock) off_win[k] = base + k <= S ? __ldg(off + base + k) : 0x7FFFFFFF;
-          __syncthreads();
-        }
-        const int s = base + (int)threadIdx.x;
-        const int lo_s = off_win[s - win_base], hi_s = off_win[s - win_base + 1];
-        const bool beyond = s >= S || lo_s >= tile_hi;
-        if (!beyond) {
-          if (lo_s >= lo0) atomicOr(&seg_bits[(lo_s - tile_lo) >> 5], 1u << ((lo_s - tile_lo) & 31));
-          if (hi_s >= tile_hi) { next_s = hi_s > tile_hi ? s : s + 1; tile_open = hi_s > tile_hi ? 1 : 0; }
-        }
-        if (__syncthreads_or(beyond)) break;
-      }
-      if (warp == 0) {                                           // starts before each 32-element word of the tile
-        int cnt[4], sum = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) { cnt[k] = sum; sum += __popc(seg_bits[4 * lane + k]); }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-          if (lane >= o) incl += u;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) seg_before[4 * lane + k] = incl - sum + cnt[k];
-      }
-      __syncthreads();
-      const bool cont = lo_c < lo0, open = tile_open != 0;
-      const int lo_rel = lo0 - tile_lo, hi_rel = tile_hi - tile_lo;
-      uint32_t cin[N][ROWS];                                     // what precedes the chunk in its run, within the warp's row
-      uint32_t marks[ROWS];                                      // bits 0-3: starts in the chunk, 4: start right after it, 5: no start in earlier lanes
-      int before[ROWS];                                          // starts before the chunk, in the tile
-#pragma unroll
-      for (int j = 0; j < ROWS; ++j) {
-        const int p = (j * kBlock + (int)threadIdx.x) * 4, w = p >> 5, sh = p & 31;
-        const uint32_t word = seg_bits[w];
-        const uint32_t b5 = __funnelshift_r(word, seg_bits[w + 1], sh) & 31u, b = b5 & 15u;
-        before[j] = seg_before[w] + __popc(word & ((1u << sh) - 1u));
-        const unsigned H = __ballot_sync(0xFFFFFFFFu, b != 0);
-        const unsigned upto = H & (0xFFFFFFFFu >> (31 - lane));  // lanes up to this one that hold a start
-        const int lower = upto ? 31 - __clz(upto) : 0;            // the run this chunk's end belongs to begins in that lane
-        marks[j] = b5 | ((H & ((1u << lane) - 1u)) == 0 ? 32u : 0u);
+      const int step_hi = min(base + STEP, hi0);
+      if (__shfl_sync(0xFFFFFFFFu, o[0], 0) >= step_hi) {            // uniform: the step belongs to the open segment
         static_for<0, N>([&](auto ic) {
           constexpr int i = decltype(ic)::value;
           constexpr CNode nd = CL::c.nodes[i];
           if constexpr (is_segfold_root(nd)) {
 #pragma unroll
-            for (int e = 1; e < 4; ++e)
-              if (!((b >> e) & 1u)) xv[i][j][e] = combine<nd.fn, nd.dtype>(xv[i][j][e - 1], xv[i][j][e]);
-            uint32_t run = xv[i][j][3];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, run, o);
-              if (lane - o >= lower) run = combine<nd.fn, nd.dtype>(u, run);
-            }
-            const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, run, 1);
-            cin[i][j] = lane == 0 ? identity_of<nd.fn, nd.dtype>() : prev;
-            if (lane == 31) seg_unit_val[fold_slot_of(i)][j * WARPS + warp] = run;
+            for (int j = 0; j < ROWS; ++j)
+              fold_step<nd.fn, nd.dtype>(acc[i], comp[i], combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(x[i][j][0], x[i][j][1]),
+                                                                                   combine<nd.fn, nd.dtype>(x[i][j][2], x[i][j][3])));
           }
         });
-        if (lane == 31) seg_unit_flag[j * WARPS + warp] = H != 0 ? 1u : 0u;
+        continue;
       }
-      __syncthreads();
-      // the 32 (row, warp) units in sequence: what runs into each of them from the units before
-      const unsigned UH = __ballot_sync(0xFFFFFFFFu, seg_unit_flag[lane] != 0);
-      const unsigned uupto = UH & (0xFFFFFFFFu >> (31 - lane));
-      const int ulower = uupto ? 31 - __clz(uupto) : 0;
+      if (lane < STEP / 32) bits[warp][lane] = 0;
+      __syncwarp();
+      int begun = 0;                                             // segments that begin in this step
+      for (bool more = true; more;) {
 #pragma unroll
-      for (int j = 0; j < ROWS; ++j) before[j] -= cont ? 0 : 1;  // now: the chunk's first element lies in segment s_cur + before (+ starts up to it)
+        for (int u = 0; u < AHEAD; ++u) {
+          const unsigned beyond = __ballot_sync(0xFFFFFFFFu, o[u] >= step_hi);
+          const int k = !more ? 0 : beyond ? __ffs(beyond) - 1 : 32;   // (offsets behind one beyond the step do not count, whatever they are)
+          if (lane < k && o[u] >= base) atomicOr(&bits[warp][(o[u] - base) >> 5], 1u << ((o[u] - base) & 31));
+          begun += k;
+          more = more && k == 32;
+        }
+        refill(next + begun);
+      }
+      __syncwarp();
+      const uint32_t b = (bits[warp][lane >> 1] >> ((lane & 1) * 16)) & 0xFFFFu;   // starts among the lane's 16 elements
+      const unsigned H = __ballot_sync(0xFFFFFFFFu, b != 0);
+      const unsigned upto = H & (0xFFFFFFFFu >> (31 - lane));
+      const int lower = upto ? 31 - __clz(upto) : 0;             // the segment open at the lane's end began in that lane, or before the step
+      const bool led = (H & ((1u << lane) - 1u)) == 0;           // no start in earlier lanes
       static_for<0, N>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr CNode nd = CL::c.nodes[i];
         if constexpr (is_segfold_root(nd)) {
-          uint32_t run = seg_unit_val[fold_slot_of(i)][lane];
+          uint32_t t = acc[i];                                    // the lanes' shares of the open segment
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, run, o);
-            if (lane - o >= ulower) run = combine<nd.fn, nd.dtype>(u, run);
-          }
+          for (int d = 16; d > 0; d >>= 1) t = combine<nd.fn, nd.dtype>(t, __shfl_xor_sync(0xFFFFFFFFu, t, d));
+          open[i] = combine<nd.fn, nd.dtype>(open[i], t);
+          acc[i] = identity_of<nd.fn, nd.dtype>();
+          comp[i] = 0.0f;
+          uint32_t* mine = staged[warp];
 #pragma unroll
           for (int j = 0; j < ROWS; ++j) {
-            const int unit = j * WARPS + warp;
-            const uint32_t into = __shfl_sync(0xFFFFFFFFu, run, max(unit - 1, 0));
-            if ((marks[j] & 32u) && unit > 0) cin[i][j] = combine<nd.fn, nd.dtype>(into, cin[i][j]);
+            const int q = j * 32 + lane;                          // chunk of four: the (q % 4)-th of lane q / 4
+            *reinterpret_cast<uint4*>(mine + (q >> 2) * kSegStride + (q & 3) * 4) = make_uint4(x[i][j][0], x[i][j][1], x[i][j][2], x[i][j][3]);
           }
+          __syncwarp();
+          uint32_t run = identity_of<nd.fn, nd.dtype>();
+          uint32_t* own = mine + lane * kSegStride;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            uint4 v = *reinterpret_cast<const uint4*>(own + 4 * c);
+            v.x = run = ((b >> (4 * c + 0)) & 1u) ? v.x : combine<nd.fn, nd.dtype>(run, v.x);
+            v.y = run = ((b >> (4 * c + 1)) & 1u) ? v.y : combine<nd.fn, nd.dtype>(run, v.y);
+            v.z = run = ((b >> (4 * c + 2)) & 1u) ? v.z : combine<nd.fn, nd.dtype>(run, v.z);
+            v.w = run = ((b >> (4 * c + 3)) & 1u) ? v.w : combine<nd.fn, nd.dtype>(run, v.w);
+            *reinterpret_cast<uint4*>(own + 4 * c) = v;
+          }
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, run, d);
+            if (lane - d >= lower) run = combine<nd.fn, nd.dtype>(u, run);
+          }
+          uint32_t into = __shfl_up_sync(0xFFFFFFFFu, run, 1);    // what runs into the lane's elements
+          if (lane == 0) into = open[i];
+          else if (led) into = combine<nd.fn, nd.dtype>(open[i], into);
+          own[16] = into;                                         // (a word of the lane's padding)
+          open[i] = __shfl_sync(0xFFFFFFFFu, run, 31);            // (some segment begins in the step, so this began in it)
+          __syncwarp();
+          // a lane per start: the segment before it ends in front of it
+          uint32_t* out = reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr));
+          for (int k = lane; k < begun; k += 32) {
+            const int seg = next + k, pos = __ldg(off + seg) - base;
+            if (pos < 0 || pos >= STEP) continue;                 // (offsets that descend)
+            uint32_t v;
+            if (pos == 0) {
+              v = mine[16];
+            } else {
+              const int l = (pos - 1) >> 4, e = (pos - 1) & 15;
+              const uint32_t lb = (bits[warp][l >> 1] >> ((l & 1) * 16)) & ((2u << e) - 1u);   // starts in that lane up to the element
+              v = mine[l * kSegStride + e];
+              if (lb == 0) v = combine<nd.fn, nd.dtype>(mine[l * kSegStride + 16], v);
+            }
+            if (seg == first) { head[i] = v; found_head = true; }
+            else out[seg - 1] = v;
+          }
+          __syncwarp();                                           // (the next fold, or step, writes there)
         }
       });
-#pragma unroll
-      for (int j = 0; j < ROWS; ++j) {
-        const int p = (j * kBlock + (int)threadIdx.x) * 4;
-        const uint32_t b = marks[j] & 15u;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int pos = p + e;
-          const bool ends = pos >= lo_rel && pos < hi_rel && (pos == hi_rel - 1 || ((marks[j] >> (e + 1)) & 1u));
-          if (ends) {
-            const bool led = (b & ((2u << e) - 1u)) == 0;          // no start in the chunk up to here: the run comes in from before
-            const int seg = s_cur + before[j] + __popc(b & ((2u << e) - 1u));
-            uint32_t v[N];
-            static_for<0, N>([&](auto ic) {
-              constexpr int i = decltype(ic)::value;
-              constexpr CNode nd = CL::c.nodes[i];
-              if constexpr (is_segfold_root(nd)) v[i] = led ? combine<nd.fn, nd.dtype>(cin[i][j], xv[i][j][e]) : xv[i][j][e];
-            });
-            if ((uint32_t)seg < (uint32_t)S)
-              store_piece(seg, ((seg == s_cur && cont) ? 1 : 0) | ((pos == hi_rel - 1 && open) ? 2 : 0), v);
-          }
-        }
-      }
-    } else {
-    // stage the operands of the tile
+      next += begun;
+    }
     static_for<0, N>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       constexpr CNode nd = CL::c.nodes[i];
       if constexpr (is_segfold_root(nd)) {
-        uint32_t* dst = seg_vals + fold_slot_of(i) * kSegTile;
-        if constexpr (VEC) {
-          V4 v[kSegTile / (4 * kBlock)];
+        uint32_t t = acc[i];
 #pragma unroll
-          for (int j = 0; j < kSegTile / (4 * kBlock); ++j) {
-            const int c = tile_lo + (j * kBlock + (int)threadIdx.x) * 4;
-            if (c < tile_hi) v[j] = eval<CL, nd.in[0]>(a, Ix4{0, c});
-          }
-#pragma unroll
-          for (int j = 0; j < kSegTile / (4 * kBlock); ++j) {
-            const int q = (j * kBlock + (int)threadIdx.x) * 4;
-            if (tile_lo + q < tile_hi) *reinterpret_cast<uint4*>(dst + q) = make_uint4(v[j].v[0], v[j].v[1], v[j].v[2], v[j].v[3]);
-          }
-        } else {
-          for (int q = threadIdx.x; q < tile_hi - tile_lo; q += kBlock) dst[q] = eval<CL, nd.in[0]>(a, Ix{0, tile_lo + q});
-        }
+        for (int d = 16; d > 0; d >>= 1) t = combine<nd.fn, nd.dtype>(t, __shfl_xor_sync(0xFFFFFFFFu, t, d));
+        if (lane == 0) open_val[fold_slot_of(i)][warp] = combine<nd.fn, nd.dtype>(open[i], t);
       }
     });
+    if (found_head) {                                             // (one lane's)
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        if constexpr (is_segfold_root(CL::c.nodes[i])) head_val[fold_slot_of(i)][warp] = head[i];
+      });
+    }
+    if (lane == 0) {
+      open_seg[warp] = next - 1;
+      first_seg[warp] = next > first ? first : -1;
+      has_head[warp] = !starts_with_run && first > 0;
+    }
+  }
+  __syncthreads();
 
-    // the pieces of the tile, a thread per segment; those beyond kSegShort elements are set aside
-    for (int base = s_cur;; base += kBlock) {
-      if (win_base < 0 || base + kBlock > win_base + kSegWindow) {     // uniform: the window moves up to `base`
-        __syncthreads();
-        win_base = base;
-        for (int k = threadIdx.x; k <= kSegWindow; k += kBlock) off_win[k] = base + k <= S ? __ldg(off + base + k) : 0x7FFFFFFF;
-      }
-      __syncthreads();
-      const int s = base + (int)threadIdx.x;
-      const int lo_s = off_win[s - win_base], hi_s = off_win[s - win_base + 1];
-      const bool beyond = s >= S || lo_s >= tile_hi;
-      if (!beyond) {
-        const int plo = max(lo_s, lo0), phi = min(hi_s, tile_hi);
-        if (hi_s >= tile_hi) next_s = hi_s > tile_hi ? s : s + 1;      // the segment that holds the tile's last element
-        if (phi > plo) {
-          const int kind = (lo_s < lo0 ? 1 : 0) | (hi_s > tile_hi ? 2 : 0);
-          if (phi - plo <= kSegShort) {
-            uint32_t v[N];
-            reduce_strided(plo, phi, 0, 1, tile_lo, v);
-            store_piece(s, kind, v);
-          } else if (phi - plo <= kSegMedium) {
-            const int at = atomicAdd(&n_long, 1);
-            if (at < kSegListCap) { long_seg[at] = s; long_lo[at] = plo; long_hi[at] = phi; long_kind[at] = kind; }
+  // segments that cross warps: one thread per fold goes over the warps in order
+  if (threadIdx.x < NF) {
+    static_for<0, N>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      constexpr CNode nd = CL::c.nodes[i];
+      if constexpr (is_segfold_root(nd)) {
+        const int f = fold_slot_of(i);
+        if ((int)threadIdx.x != f) return;
+        using Run = Running<nd.fn, nd.dtype>;
+        uint32_t* out = reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr));
+        uint32_t* head = rec + (size_t)blockIdx.x * 2 * REC;
+        uint32_t* tail = head + REC;
+        auto value = Run::identity();
+        int seg = -1;                                             // the open segment; -1: nothing of one in this block yet
+        bool from_here = false, any = false;
+        auto close = [&]() {
+          if (seg < 0 || seg >= S || !any) return;
+          if (from_here) { out[seg] = Run::narrow(value); return; }
+          head[0] = (uint32_t)seg + 1u;
+          head[2 + f] = Run::narrow(value);
+        };
+        for (int w = 0; w < WARPS; ++w) {
+          if (open_seg[w] < 0 && first_seg[w] < 0) continue;      // (a run without elements)
+          if (first_seg[w] >= 0) {
+            if (has_head[w]) {
+              if (!any) { seg = first_seg[w] - 1; any = true; }
+              value = Run::add(value, Run::of(head_val[f][w]));
+            }
+            close();
+            seg = open_seg[w];
+            value = Run::of(open_val[f][w]);
+            from_here = any = true;
           } else {
-            const int at = atomicAdd(&n_big, 1);
-            if (at < kSegBigCap) { big_seg[at] = s; big_lo[at] = plo; big_hi[at] = phi; big_kind[at] = kind; }
+            if (!any) { seg = open_seg[w]; any = true; }
+            value = Run::add(value, Run::of(open_val[f][w]));
+          }
+        }
+        if (any) {
+          const int64_t block_hi = (int64_t)(blockIdx.x + 1) * WARPS * run_length;
+          if (e_hi <= block_hi) {
+            close();                                              // the last segment ends in this block
+          } else {
+            uint32_t* r = from_here ? tail : head;
+            if (seg >= 0 && seg < S) {
+              r[0] = (uint32_t)seg + 1u;
+              r[2 + f] = Run::narrow(value);
+            }
           }
         }
       }
-      if (__syncthreads_or(beyond)) break;
-    }
-    const int todo = min(n_long, kSegListCap);
-    // a warp per piece of medium length
-    for (int k = warp; k < todo; k += WARPS) {
-      const int plo = long_lo[k], phi = long_hi[k];
-      uint32_t v[N];
-      reduce_strided(plo, phi, lane, 32, tile_lo, v);
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) v[i] = warp_reduce<nd.fn, nd.dtype>(v[i]);
-      });
-      if (lane == 0) store_piece(long_seg[k], long_kind[k], v);
-    }
-    // the whole block per piece beyond that (at most three of them in a tile)
-    const int todo_big = min(n_big, kSegBigCap);
-    for (int k = 0; k < todo_big; ++k) {
-      const int plo = big_lo[k], phi = big_hi[k];
-      uint32_t v[N];
-      reduce_strided(plo, phi, (int)threadIdx.x, kBlock, tile_lo, v);
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        constexpr CNode nd = CL::c.nodes[i];
-        if constexpr (is_segfold_root(nd)) v[i] = block_reduce<nd.fn, nd.dtype>(v[i], red);
-      });
-      if (threadIdx.x == 0) store_piece(big_seg[k], big_kind[k], v);
-    }
-    }
-    __syncthreads();
-
-    // segments that cross the tile's ends: the block's running value
-    if (threadIdx.x == 0) {
-      if (have_first) {
-        if (carry_seg != s_cur) {                              // begun before this block: nothing carried yet
-          carry_seg = s_cur;
-          carry_from_here = false;
-          static_for<0, N>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            if constexpr (is_segfold_root(CL::c.nodes[i])) { carry[i] = first_val[fold_slot_of(i)]; carry_comp[i] = 0.0f; }
-          });
-        } else {
-          static_for<0, N>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr CNode nd = CL::c.nodes[i];
-            if constexpr (is_segfold_root(nd)) fold_step<nd.fn, nd.dtype>(carry[i], carry_comp[i], first_val[fold_slot_of(i)]);
-          });
-        }
-        if (!first_open) {                                     // the segment ends in this tile
-          uint32_t* head = rec + (size_t)blockIdx.x * 2 * REC;
-          if (!carry_from_here) head[0] = (uint32_t)carry_seg + 1u;
-          static_for<0, N>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            if constexpr (is_segfold_root(CL::c.nodes[i])) {
-              if (carry_from_here) reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr))[carry_seg] = carry[i];
-              else head[2 + fold_slot_of(i)] = carry[i];
-            }
-          });
-          carry_seg = -1;
-        }
-      }
-      if (have_last) {
-        carry_seg = last_seg;
-        carry_from_here = true;
-        static_for<0, N>([&](auto ic) {
-          constexpr int i = decltype(ic)::value;
-          if constexpr (is_segfold_root(CL::c.nodes[i])) { carry[i] = last_val[fold_slot_of(i)]; carry_comp[i] = 0.0f; }
-        });
-      }
-    }
-    s_cur = next_s;                                              // written before the barrier above, by the one thread that saw it
-  }
-
-  // what is still open where the block's run of tiles ends
-  if (threadIdx.x == 0 && carry_seg >= 0) {
-    uint32_t* r = rec + ((size_t)blockIdx.x * 2 + (carry_from_here ? 1 : 0)) * REC;
-    r[0] = (uint32_t)carry_seg + 1u;
-    static_for<0, N>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      if constexpr (is_segfold_root(CL::c.nodes[i])) r[2 + fold_slot_of(i)] = carry[i];
     });
   }
 }
