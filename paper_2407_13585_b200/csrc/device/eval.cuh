@@ -74,6 +74,9 @@ struct V4 { uint32_t v[4]; };
 struct Ix   { int r, c; };            // one element
 struct Ix4  { int r, c; };            // c, c+1, c+2, c+3  (c % 4 == 0)
 struct IxR4 { int r, c; };            // c, c-1, c-2, c-3  ((c-3) % 4 == 0)
+// the same in a rank-1 array whose length is no multiple of four: the image of a chunk under reversal lies across two chunks
+struct Ix4U : Ix4 {};
+struct IxR4U : IxR4 {};
 struct IxS4 { int r, c, dc; };        // clamp(c+dc+i, 0, C-1) for i = 0..3, row r (c % 4 == 0)
 struct IxG4 { Ix e[4]; };             // four unrelated positions
 
@@ -110,6 +113,16 @@ __device__ __forceinline__ V4 ld(const uint32_t* p, int C, const Ix4& i) {
 }
 __device__ __forceinline__ V4 ld(const uint32_t* p, int C, const IxR4& i) {
   const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + (i.r * C + i.c - 3)));
+  return V4{{t.w, t.z, t.y, t.x}};
+}
+// (two chunks, which the neighbouring lanes ask for as well; the shift is the same for every chunk of the array)
+__device__ __forceinline__ V4 ld(const uint32_t* p, int C, const IxR4U& i) {
+  const int at = i.c - 3, shift = at & 3;
+  if ((at | 3) + 4 >= C) return V4{{__ldg(p + at + 3), __ldg(p + at + 2), __ldg(p + at + 1), __ldg(p + at)}};   // the second chunk is not whole
+  const uint4 t = __ldg(reinterpret_cast<const uint4*>(p + (at & ~3))), u = __ldg(reinterpret_cast<const uint4*>(p + (at & ~3) + 4));
+  if (shift == 1) return V4{{u.x, t.w, t.z, t.y}};
+  if (shift == 2) return V4{{u.y, u.x, t.w, t.z}};
+  if (shift == 3) return V4{{u.z, u.y, u.x, t.w}};
   return V4{{t.w, t.z, t.y, t.x}};
 }
 __device__ __forceinline__ V4 ld(const uint32_t* p, int C, const IxG4& i) {
@@ -172,6 +185,16 @@ template <int F, int P0 = kRunTime, int P1 = kRunTime> __device__ __forceinline_
   if constexpr (F == ACC_IDX_IDENTITY) return i;
   else if constexpr (F == ACC_IDX_REVERSE) return Ix4{src.R - 1 - i.r, src.C - 1 - i.c};
   else return map_lanes<F>(i, self, src);
+}
+template <int F, int P0 = kRunTime, int P1 = kRunTime> __device__ __forceinline__ auto map_index(const Ix4U& i, const NodeArg& self, const NodeArg& src) {
+  if constexpr (F == ACC_IDX_IDENTITY) return i;
+  else if constexpr (F == ACC_IDX_REVERSE) return IxR4U{{src.R - 1 - i.r, src.C - 1 - i.c}};
+  else return map_lanes<F>(static_cast<const Ix4&>(i), self, src);
+}
+template <int F, int P0 = kRunTime, int P1 = kRunTime> __device__ __forceinline__ auto map_index(const IxR4U& i, const NodeArg& self, const NodeArg& src) {
+  if constexpr (F == ACC_IDX_IDENTITY) return i;
+  else if constexpr (F == ACC_IDX_REVERSE) return Ix4U{{src.R - 1 - i.r, src.C - 1 - i.c}};
+  else return map_lanes<F>(static_cast<const IxR4&>(i), self, src);
 }
 template <int F, int P0 = kRunTime, int P1 = kRunTime> __device__ __forceinline__ auto map_index(const IxG4& i, const NodeArg& self, const NodeArg& src) {
   if constexpr (F == ACC_IDX_IDENTITY) return i;

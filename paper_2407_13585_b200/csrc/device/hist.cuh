@@ -307,6 +307,22 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
     for (; q0 + reach < total; q0 += step, it += U) trip(std::true_type{}, (uint32_t)q0);
     for (; q0 < total; q0 += step, it += U) trip(std::false_type{}, (uint32_t)q0);
   }
+  if constexpr (VEC && DR <= 1) {
+    // the last elements of an array whose length is no multiple of four: every CTA of the first team takes those whose bin it owns
+    const int c = (int)(per_row * 4u + threadIdx.x);
+    if (team == 0 && c < a.C) {
+      const Ix ix{0, c};
+      if (rank == 0) {
+        static_for<0, N>([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          constexpr CNode nd = CL::c.nodes[i];
+          if constexpr (is_store_root(nd)) reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr))[c] = eval<CL, i>(a, ix);
+          else if constexpr (is_scalar_fold(nd)) fold_step<nd.fn, nd.dtype>(acc[i], comp[i], eval<CL, nd.in[0]>(a, ix));
+        });
+      }
+      scatter_one(eval<CL, pn.in[1]>(a, ix), eval<CL, pn.in[2]>(a, ix));
+    }
+  }
 
   __syncthreads();
   // every CTA starts its sweep somewhere else, so that the CTAs that finish together do not all

@@ -119,14 +119,17 @@ __device__ __forceinline__ double* acc64_of(const A& a, double* base) {
 }
 
 // =========================================================================================
+// VEC: rows and the images of chunks under reversal start on 16 bytes.  (A rank-1 domain is walked four elements at a time
+// either way, all but its last few; see Ix4U.)
 template <class CL, bool VEC>
 __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<CL::c.n> a) {
   constexpr int N = CL::c.n;
-  constexpr int W = VEC ? 4 : 1;
   constexpr int DR = domain_rank<CL>();
+  constexpr bool FOUR = VEC || DR <= 1;                  // four elements at a time: always over a rank-1 domain
+  constexpr int W = FOUR ? 4 : 1;
   constexpr int NF = count_if<CL>(is_scalar_fold);
   constexpr int NP64 = count_if<CL>(is_f32_add_permute);
-  using IX = std::conditional_t<VEC, Ix4, Ix>;
+  using IX = std::conditional_t<VEC, Ix4, std::conditional_t<FOUR, Ix4U, Ix>>;
   __shared__ uint32_t red[kBlock / 32];
   __shared__ bool last_block;
 
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
         st(reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr)), a.n[i].C, ix, eval<CL, i>(a, ix));
       } else if constexpr (is_scalar_fold(nd)) {
         const auto v = eval<CL, nd.in[0]>(a, ix);
-        if constexpr (VEC) {
+        if constexpr (FOUR) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) fold_step<nd.fn, nd.dtype>(acc[i], comp[i], v.v[j]);
         } else {
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
         uint32_t* out = reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr));
         const uint32_t bins = (uint32_t)(a.n[i].R * a.n[i].C);
         double* acc64 = acc64_of<CL, i>(a, acc64_base);
-        if constexpr (VEC) {
+        if constexpr (FOUR) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) permute_update<nd.fn, nd.dtype>(a, out, acc64, bins, k.v[j], x.v[j]);
         } else {
@@ -202,6 +205,24 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
       }
     });
    }
+  }
+
+  if constexpr (DR <= 1) {
+    // the last elements of an array whose length is no multiple of four
+    const int c = (int)(per_row * 4u + threadIdx.x);
+    if (blockIdx.x == 0 && c < a.C) {
+      const Ix ix{0, c};
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        constexpr CNode nd = CL::c.nodes[i];
+        uint32_t* out = reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr));
+        if constexpr (is_store_root(nd)) out[c] = eval<CL, i>(a, ix);
+        else if constexpr (is_scalar_fold(nd)) fold_step<nd.fn, nd.dtype>(acc[i], comp[i], eval<CL, nd.in[0]>(a, ix));
+        else if constexpr (is_permute_root(nd))
+          permute_update<nd.fn, nd.dtype>(a, out, acc64_of<CL, i>(a, acc64_base), (uint32_t)(a.n[i].R * a.n[i].C),
+                                          eval<CL, nd.in[1]>(a, ix), eval<CL, nd.in[2]>(a, ix));
+      });
+    }
   }
 
   if constexpr (NF > 0 || NP64 > 0) {

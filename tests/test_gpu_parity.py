@@ -39,6 +39,18 @@ def test_config1_all_partitions(n):
     assert check_program(W.config1(n)) == 8
 
 
+# lengths that are one, two and three more than a multiple of four: reversed chunks lie across two chunks, the last elements
+# are taken one by one; fewer than one chunk
+@pytest.mark.parametrize("n", [2, 5, 4097, 4098, 200003])
+def test_config1_any_length(n):
+    assert check_program(W.config1(n)) == 8
+
+
+@pytest.mark.parametrize("n,bins", [(4097, 256), (70001, 256), (70002, 8192), (600003, 70000)])
+def test_config5_any_length(n, bins):
+    assert check_program(W.config5(n, bins)) == 10
+
+
 # below one 64 x 64 tile: generic kernels; from 64 rows on: shared-memory tile pairs, with ragged
 # edge tiles (100, 130), without 128-bit accesses (130, 67: the threads stage the tiles; otherwise
 # tensor copies do) and on whole tiles (64, 256); 1600 and 2052 give every persistent block
