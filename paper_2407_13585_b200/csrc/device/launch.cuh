@@ -267,6 +267,10 @@ struct Launcher {
     return ((base + 15) & ~int64_t(15)) + full * 4 + full * 32 * 4;
   }
 
+  // k_hist's scratch behind `words` of counters and accumulators: private overflow bins per CTA, then (from a multiple of 16
+  // bytes) what the CTAs exchange.
+  static int64_t hist_exchange_off(int64_t words, const dev::HistPlan& plan) { return (words + (int64_t)sm_count() * plan.overflow + 3) & ~int64_t(3); }
+
   static int64_t scratch_bytes(const ClusterLaunch& L) {
     int R, C;
     if (!domain(L, R, C)) return ACC_ERR_NO_KERNEL;
@@ -287,7 +291,7 @@ struct Launcher {
     for (int i = 0; i < N; ++i)
       if (dev::is_f32_add_permute(CL::c.nodes[i])) words += 2 * (int64_t)L.nodes[i].R * L.nodes[i].C;
     dev::HistPlan plan;
-    if (use_hist(L, R, C, plan)) words += (int64_t)sm_count() * plan.overflow;   // private overflow bins per CTA
+    if (use_hist(L, R, C, plan)) words = hist_exchange_off(words, plan) + (int64_t)sm_count() * plan.exchange;
     if (stream_slab_shapes_ok(L, R, C)) return with_slab_area(words * 4, C);
     return words * 4;
   }
@@ -301,6 +305,8 @@ struct Launcher {
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
     if (kHasScan && use_ring(L, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
     if (stream_slab_shapes_ok(L, R, C)) return (((int64_t)dev::stream_acc64_off(kScalarFolds, sm_count() * 8) * 4) + 15) & ~int64_t(15);
+    dev::HistPlan plan;
+    if (use_hist(L, R, C, plan)) return scratch_bytes(L) - (int64_t)sm_count() * plan.exchange * 4;   // (what is exchanged is written first)
     return scratch_bytes(L);
   }
 
@@ -608,7 +614,7 @@ int Launcher<CL>::launch_hist(const ClusterLaunch& L, dev::Args<N>& a, int R, in
     constexpr int P = dev::the_f32_add_permute<CL>();
     const int64_t bins = (int64_t)L.nodes[P].R * L.nodes[P].C;
     auto kern = vec ? dev::k_hist<CL, true> : dev::k_hist<CL, false>;
-    const size_t smem = (size_t)plan.per_cta * 4;
+    const size_t smem = std::max<size_t>(((size_t)plan.per_cta + 3) / 4 * 16, (size_t)(sm_count() + dev::kHistBlock / 2) * 8);
     static int granted[2][64];
     if (!opt_in_shared_memory(kern, smem, granted[vec ? 1 : 0]))
       return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -618,7 +624,14 @@ int Launcher<CL>::launch_hist(const ClusterLaunch& L, dev::Args<N>& a, int R, in
     const int teams = (int)std::max<int64_t>(1, std::min<int64_t>(want, sm_count() / plan.group));
     const int grid = teams * plan.group;                  // one CTA per SM: all of them are resident together
     int* overflow = reinterpret_cast<int*>(L.scratch + dev::stream_acc64_off(kScalarFolds, a.grid) + 2 * bins);
-    kern<<<grid, dev::kHistBlock, smem, L.stream>>>(a, plan, overflow);
+    int* exchange = reinterpret_cast<int*>(L.scratch + hist_exchange_off(dev::stream_acc64_off(kScalarFolds, a.grid) + 2 * bins, plan));
+    if (plan.exchange && cooperative_launch_ok()) {
+      void* params[] = {&a, &plan, &overflow, &exchange};
+      cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3(grid), dim3(dev::kHistBlock), params, smem, L.stream);
+    } else {
+      plan.exchange = 0;
+      kern<<<grid, dev::kHistBlock, smem, L.stream>>>(a, plan, overflow, exchange);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     return ACC_OK;

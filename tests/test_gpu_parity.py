@@ -46,7 +46,7 @@ def test_config1_any_length(n):
     assert check_program(W.config1(n)) == 8
 
 
-@pytest.mark.parametrize("n,bins", [(4097, 256), (70001, 256), (70002, 8192), (600003, 70000)])
+@pytest.mark.parametrize("n,bins", [(4097, 256), (70001, 256), (70002, 8192), (600003, 70000), (540001, 65536), (170000, 20000)])
 def test_config5_any_length(n, bins):
     assert check_program(W.config5(n, bins)) == 10
 
