@@ -331,8 +331,11 @@ struct Launcher {
   // small to fill the machine with tiles.
   static int launch_stencil(const ClusterLaunch& L, dev::Args<N>& a, int R, int C, bool vec) {
     if constexpr (kStencilShape) {
-      if (!vec || R < 1 || (int64_t)R * C < (int64_t)dev::kStRows * dev::kStCols * 64) return 1;
+      if (R < 1 || (int64_t)R * C < (int64_t)dev::kStRows * dev::kStCols * 64) return 1;
       constexpr int depth = dev::max_shift_depth<CL>();
+      // (rows that do not start on 16 bytes are copied word by word, which pays where iterates are kept on chip: 4000 x 3999,
+      // four iterations in twos 360 -> 141 us, one by one 204 -> 201 us, 1000 x 1001 one by one 27 -> 35 us)
+      if (!vec && depth < 2) return 1;
       dev::StencilMaps maps;
       for (int i = 0; i < N; ++i) {
         const CNode& n = CL::c.nodes[i];
@@ -341,14 +344,18 @@ struct Launcher {
           return 1;
         if (dev::is_staged_external<CL>(i)) {
           if (L.nodes[i].R != R || L.nodes[i].C != C) return 1;
-          if (!make_tensor_map_2d(&maps.m[dev::tile_slot<CL>(i)], L.nodes[i].ptr, R, C, dev::st_box_rows(depth), dev::kStBoxCols)) return 1;
+          if (vec && !make_tensor_map_2d(&maps.m[dev::tile_slot<CL>(i)], L.nodes[i].ptr, R, C, dev::st_box_rows(depth), dev::kStBoxCols)) return 1;
         }
       }
-      auto kern = dev::k_stencil<CL>;
+      auto kern = dev::k_stencil<CL, true>;
+      if constexpr (depth >= 2) {
+        if (!vec) kern = dev::k_stencil<CL, false>;
+      }
       // two stages of every external's box, one box per member kept on chip
-      const size_t smem = (size_t)(dev::kStStages * dev::staged_externals<CL>() + dev::staged_members<CL>()) * dev::st_box_stride(depth) * 4;
-      static int granted[64];
-      if (!opt_in_shared_memory(kern, smem, granted))
+      const size_t smem = (size_t)(dev::kStStages * dev::staged_externals<CL>() + dev::staged_members<CL>()) * dev::st_box_stride(depth) * 4 +
+                          (vec ? 0 : (size_t)dev::kBlock / 32 * dev::kStCols * 4);
+      static int granted[2][64];
+      if (!opt_in_shared_memory(kern, smem, granted[vec ? 1 : 0]))
         return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
       const int64_t tiles = (int64_t)((C + dev::kStCols - 1) / dev::kStCols) * ((R + dev::kStRows - 1) / dev::kStRows);
       const int per_sm = std::max(1, std::min(3, (int)((size_t)220 * 1024 / (smem + 1024))));

@@ -21,6 +21,11 @@
 // would do.  The values are those of the plain evaluation, bit for bit: every element is
 // computed by the same expression, at positions clamped in the same way.
 //
+// Rows that do not start on 16 bytes (a width that is no multiple of four) cannot be copied as boxes: the block's threads
+// copy them word by word (cp.async, 4 bytes, to the same places in shared memory, counted by the same barriers), and a
+// warp's results go through shared memory on their way out, so that its stores are runs of words.  (4000 x 3999, four
+// iterations in twos: 360 -> 141 us; streamed, the iterate in between was evaluated 25-fold.)
+//
 // Every wait on an mbarrier is bounded: after kCopySpinLimit polls the thread records
 // ACC_ERR_DEVICE_TIMEOUT in the status words and goes on, so a lost copy cannot hang the GPU.
 #pragma once
@@ -190,7 +195,7 @@ __device__ __forceinline__ V4 ld_staged(const A& a, const IxHS4<DC>& ix) {
   return ld_box(ix.t.mem + member_slot<CL>(I) * st_box_stride(max_shift_depth<CL>()) + ix.off, ix, a.n[I].C);
 }
 
-template <class CL>
+template <class CL, bool BOXES>
 __global__ void __launch_bounds__(kBlock)
 k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ StencilMaps maps) {
   constexpr int N = CL::c.n;
@@ -200,13 +205,14 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
   extern __shared__ __align__(128) uint32_t boxes[];          // [stage][external slot][BS], then [member slot][BS]
   __shared__ __align__(8) uint64_t bar[kStStages];
   uint32_t* const members = boxes + kStStages * E * BS;
+  uint32_t* const results = members + staged_members<CL>() * BS;   // (not BOXES) a row of results per warp
   const int R = a.R, C = a.C;
   const uint32_t tiles_x = (uint32_t)(C + kStCols - 1) / kStCols;
   const uint32_t n_tiles = tiles_x * ((uint32_t)(R + kStRows - 1) / kStRows);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStStages; ++s) mbar_init(&bar[s], 1);
+    for (int s = 0; s < kStStages; ++s) mbar_init(&bar[s], BOXES ? 1 : kBlock);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -226,12 +232,44 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
     }
   };
 
+  // the same by all threads, word by word: a warp per box row, positions outside the array clamped (they are never read)
+  auto copy_words = [&](uint32_t tile, int stage) {
+    const uint32_t ty = tile / tiles_x, tx = tile - ty * tiles_x;
+    const int x = (int)(tx * kStCols) - 4, y = (int)(ty * kStRows) - D;
+    static_for<0, N>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      if constexpr (is_staged_external<CL>(i)) {
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(a.n[i].ptr);
+        const uint32_t dst = smem_addr(boxes + (stage * E + tile_slot<CL>(i)) * BS);
+        for (int br = warp; br < BR; br += kBlock / 32) {
+          const uint32_t* row = src + (size_t)min(max(y + br, 0), R - 1) * C;
+#pragma unroll
+          for (int k = 0; k < (kStBoxCols + 31) / 32; ++k) {
+            const int bc = k * 32 + lane;
+            if (bc < kStBoxCols)
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + (uint32_t)(br * kStBoxCols + bc) * 4u), "l"(row + min(max(x + bc, 0), C - 1))
+                           : "memory");
+          }
+        }
+      }
+    });
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(&bar[stage])) : "memory");
+  };
+
   uint32_t parity[kStStages] = {0u, 0u};
   int stage = 0;
-  if (threadIdx.x == 0 && blockIdx.x < n_tiles) issue(blockIdx.x, 0);
+  if constexpr (BOXES) {
+    if (threadIdx.x == 0 && blockIdx.x < n_tiles) issue(blockIdx.x, 0);
+  } else if (blockIdx.x < n_tiles) {
+    copy_words(blockIdx.x, 0);
+  }
   for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     // the other stage was last read before the barrier that ended the previous trip
-    if (threadIdx.x == 0 && tile + gridDim.x < n_tiles) issue(tile + gridDim.x, stage ^ 1);
+    if constexpr (BOXES) {
+      if (threadIdx.x == 0 && tile + gridDim.x < n_tiles) issue(tile + gridDim.x, stage ^ 1);
+    } else if (tile + gridDim.x < n_tiles) {
+      copy_words(tile + gridDim.x, stage ^ 1);
+    }
     const bool arrived = wait_phase(&bar[stage], parity[stage]);
     if (!arrived) raise_status(a, kStatusTimeout);
 
@@ -261,7 +299,13 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
             const int r = r0 - D + br, c = c0 - 4 + bc;
             const int off = br * kStBoxCols + bc;
             const int solo = ((lane == 31 || ch == kStChunks - 1) ? 1 : 0) | ((lane == 0 || ch == 0) ? 2 : 0);
-            const V4 v = eval_here<CL, i>(a, IxH4{r, c, off, solo, ctx});
+            V4 v = eval_here<CL, i>(a, IxH4{r, c, off, solo, ctx});
+            if constexpr (!BOXES) {                             // what lies beyond the last column reads as the last column
+              const int last = C - 1 - c;
+#pragma unroll
+              for (int e = 1; e < 4; ++e)
+                if (e > last) v.v[e] = last <= 0 ? v.v[0] : last == 1 ? v.v[1] : v.v[2];
+            }
             if (q0 + lane < kTotal && r >= 0 && r < R && c >= 0 && c < C)
               *reinterpret_cast<uint4*>(out + off) = make_uint4(v.v[0], v.v[1], v.v[2], v.v[3]);
           }
@@ -274,7 +318,25 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
     for (int p = 0; p < kStRows / (kBlock / 32); ++p) {
       // a warp per tile row, a lane per chunk
       const int r = r0 + warp + (kBlock / 32) * p, c = c0 + 4 * lane;
-      if constexpr (D == 1) {
+      if constexpr (!BOXES) {
+        const IxH4 ix{r, c, (r - r0 + D) * kStBoxCols + (c - c0 + 4), (lane == 31 ? 1 : 0) | (lane == 0 ? 2 : 0), ctx};
+        uint32_t* line = results + warp * kStCols;             // the warp's own
+        static_for<0, N>([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          if constexpr (is_store_root(CL::c.nodes[i])) {
+            const V4 v = eval<CL, i>(a, ix);
+            *reinterpret_cast<uint4*>(line + 4 * lane) = make_uint4(v.v[0], v.v[1], v.v[2], v.v[3]);
+            __syncwarp();
+            uint32_t* out = reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr)) + (size_t)r * C + c0;
+            if (r < R) {
+#pragma unroll
+              for (int k = 0; k < kStCols / 32; ++k)
+                if (c0 + k * 32 + lane < C) out[k * 32 + lane] = line[k * 32 + lane];
+            }
+            __syncwarp();
+          }
+        });
+      } else if constexpr (D == 1) {
         // A single iteration reads its neighbour words from the box, row by row under the bounds
         // check.  Measured back to back on 8192 x 8192: 91 us per launch; with all rows computed
         // first and stored afterwards (which is what the compiler makes of the form below) 104 us,
@@ -312,6 +374,7 @@ k_stencil(const __grid_constant__ Args<CL::c.n> a, const __grid_constant__ Stenc
     parity[stage] ^= 1u;
     stage ^= 1;
   }
+  if constexpr (!BOXES) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 }  // namespace dev

@@ -51,6 +51,18 @@ def test_config5_any_length(n, bins):
     assert check_program(W.config5(n, bins)) == 10
 
 
+# two iterations in one cluster on widths that are no multiple of four: boxes copied word by word, a last column anywhere in
+# its chunk, at a tile's edge and one past it
+@pytest.mark.parametrize("rows,cols", [(1100, 641), (1101, 642), (1090, 643), (4200, 129), (5000, 127)])
+def test_config4_stacked_iterations_of_any_width(rows, cols):
+    prog = W.config4(rows, cols, iters=2)
+    inputs = W.make_inputs(prog)
+    ref = oracle_run(prog, np_inputs(inputs))
+    got, g = gpu_run(prog, inputs, [-1] + [0] * 18, recompute=2)
+    assert g.launch_count() == 1
+    compare(prog, ref, got, "stacked iterations, %d x %d" % (rows, cols))
+
+
 # below one 64 x 64 tile: generic kernels; from 64 rows on: shared-memory tile pairs, with ragged
 # edge tiles (100, 130), without 128-bit accesses (130, 67: the threads stage the tiles; otherwise
 # tensor copies do) and on whole tiles (64, 256); 1600 and 2052 give every persistent block
