@@ -307,6 +307,10 @@ __global__ void __launch_bounds__(kBlock) k_tile_pair(const __grid_constant__ Ar
 // blocks are combined through a small shared array (fixed order) and one partial per row and
 // tile goes to scratch.
 //
+// Arrays whose rows do not start on 16 bytes (an extent that is no multiple of four) cannot be copied as boxes: four copy
+// warps then fetch the tiles word by word (cp.async, 4 bytes, to the same places, counted by the same barriers), and columns
+// beyond the array's edge are left out of the sums.  (6349 x 6349: 67 us, staged by the threads of k_tile_pair 75 us.)
+//
 // The kernel is launched cooperatively (all blocks resident).  After its walk a block
 // arrives at a grid-wide counter; once every block has arrived, each block adds up, in
 // column-tile order, the partials of its own slice of rows.  Publishing per pair instead
@@ -321,7 +325,8 @@ constexpr int kTpTileWords = kTile * kTile;          // 4096 words = 16 KB per c
 constexpr int kTpSlotWords = 2 * kTpTileWords;       // tiles [I,J] and [J,I] of one external
 constexpr int kTpMaxExternals = 3;
 constexpr int kTpConsumers = 256;                    // eight warps of 4 x 4 blocks = one 64 x 64 tile
-constexpr int kTpThreads = kTpConsumers + 32;                // + the copy warp
+constexpr int kTpCopiers = 128;                      // threads that copy word by word
+template <bool BOXES> constexpr int tp_threads() { return kTpConsumers + (BOXES ? 32 : kTpCopiers); }   // + the copy warp or warps
 constexpr int kTpRedStride = 20;                     // words per row of the row-sum exchange (16 used)
 constexpr uint32_t kCopySpinLimit = 1u << 20;
 template <int E> constexpr int tp_stages() { return E <= 2 ? 3 : 2; }
@@ -406,8 +411,8 @@ template <class CL> constexpr bool tile_tma_eligible() {
   return count_if<CL>(is_row_fold) >= 1 && count_if<CL>(is_row_fold) <= 2;
 }
 
-template <class CL>
-__global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_constant__ Args<CL::c.n> a,
+template <class CL, bool BOXES>
+__global__ void __launch_bounds__(tp_threads<BOXES>()) k_tile_pair_tma(const __grid_constant__ Args<CL::c.n> a,
                                                               const __grid_constant__ TileMaps maps) {
   constexpr int N = CL::c.n;
   constexpr int NRF = count_if<CL>(is_row_fold);
@@ -429,7 +434,7 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], BOXES ? 1 : kTpCopiers);
       mbar_init(&empty[s], kTpConsumers / 32);
     }
     abort_walk = 0;
@@ -440,7 +445,27 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
 
   if (threadIdx.x >= kTpConsumers) {
     // ---------------- copy warp: one lane keeps up to kStages pairs in flight -------------------
-    if (lane_id != 0) return;
+    if (BOXES && lane_id != 0) return;
+    // word by word: a warp per half row of a tile, positions beyond the array clamped (they are never used)
+    auto copy_words = [&](uint32_t pair, int stage) {
+      int I, J;
+      pair_of(pair, blocks, I, J);
+      const int n_tiles = I == J ? 1 : 2, copier = (int)threadIdx.x - kTpConsumers;
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        if constexpr (is_staged_external<CL>(i)) {
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(a.n[i].ptr);
+          for (int t = 0; t < n_tiles; ++t) {
+            const int y = (t == 0 ? I : J) * kTile, x = min((t == 0 ? J : I) * kTile + (copier & 63), n - 1);
+            const uint32_t dst = smem_addr(tiles + stage * kStageWords + tile_slot<CL>(i) * kTpSlotWords + t * kTpTileWords) + (uint32_t)(copier & 63) * 4u;
+#pragma unroll 8
+            for (int row = copier >> 6; row < kTile; row += kTpCopiers / kTile)
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + (uint32_t)row * (kTile * 4u)), "l"(src + (size_t)min(y + row, n - 1) * n + x) : "memory");
+          }
+        }
+      });
+      asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(&full[stage])) : "memory");
+    };
     auto issue = [&](uint32_t pair, int stage) {
       int I, J;
       pair_of(pair, blocks, I, J);
@@ -464,8 +489,10 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
       // its stage held trip - S: every consumer warp must have let go of that
       if (trip >= (uint32_t)S) ok = wait_phase(&empty[trip % S], (trip / S - 1) & 1u) && !*v_abort;
       if (!ok) break;
-      issue(pair, (int)(trip % S));
+      if constexpr (BOXES) issue(pair, (int)(trip % S));
+      else copy_words(pair, (int)(trip % S));
     }
+    if constexpr (!BOXES) asm volatile("cp.async.wait_all;" ::: "memory");
     if (!ok) {
       if (!*v_abort) { *v_abort = 1; raise_status(a, kStatusTimeout); }
       // copies still in flight must not land in the shared memory of a block that has gone
@@ -514,8 +541,9 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
         __syncwarp();
         if (lane_id == 0) mbar_arrive(&empty[stage]);
       }
-      const int r = r0 + 4 * by, c = c0 + 4 * bx;           // n is a multiple of 4: a block is inside or outside
+      const int r = r0 + 4 * by, c = c0 + 4 * bx;           // (where n is a multiple of four a block is inside or outside)
       const bool inside = r < n && c < n;
+      const int cols = BOXES ? 4 : n - c;                     // columns of the block that exist
       static_for<0, N>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr CNode nd = CL::c.nodes[i];
@@ -525,7 +553,12 @@ __global__ void __launch_bounds__(kTpThreads) k_tile_pair_tma(const __grid_const
           for (int j = 0; j < 4; ++j) {
             uint32_t s = identity_of<nd.fn, nd.dtype>();
             if (inside) {
-              const V4 v = eval<CL, nd.in[0]>(a, IxB4{r + j, c, j, &ctx});
+              V4 v = eval<CL, nd.in[0]>(a, IxB4{r + j, c, j, &ctx});
+              if constexpr (!BOXES) {
+#pragma unroll
+                for (int e = 1; e < 4; ++e)
+                  if (e >= cols) v.v[e] = identity_of<nd.fn, nd.dtype>();
+              }
               s = combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(v.v[0], v.v[1]), combine<nd.fn, nd.dtype>(v.v[2], v.v[3]));
             }
             red[tp][ord][4 * by + j][bx] = s;

@@ -51,6 +51,12 @@ def test_config5_any_length(n, bins):
     assert check_program(W.config5(n, bins)) == 10
 
 
+# tiles copied word by word: one, two and three columns in the last chunk of four, of a tile that is nearly empty or nearly full
+@pytest.mark.parametrize("rows", [2561, 2622, 2623])
+def test_config2_any_extent(rows):
+    check_program(W.config2(rows), [[-1, 0, 0, 0]])
+
+
 # two iterations in one cluster on widths that are no multiple of four: boxes copied word by word, a last column anywhere in
 # its chunk, at a tile's edge and one past it
 @pytest.mark.parametrize("rows,cols", [(1100, 641), (1101, 642), (1090, 643), (4200, 129), (5000, 127)])
