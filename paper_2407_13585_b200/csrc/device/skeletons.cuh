@@ -7,10 +7,10 @@
 //   k_rowfold  one block per row of a rank-2 domain; folds of the innermost extent end in a
 //              block reduction, no atomics.
 //   k_scan     single-pass scan with decoupled look-back; the scanned operand is evaluated in
-//              registers.  A tile's predecessors are always running or done: the grid is
-//              cooperative and block b takes tiles b, b + G, ..., or tiles are claimed from an
-//              atomic ticket.  k_scan_pipelined is the same scan with a warp that only looks
-//              back, for small tiles.
+//              registers.  Tiles are claimed from an atomic ticket, so a tile's predecessors are
+//              always running or done.  Most scans take k_scan_ring or k_scan_rows (scanring.cuh)
+//              instead; this one is left for what those do not: short arrays below a gather, index
+//              maps, devices without cooperative launches.
 //
 // Each is templated on the cluster description (what to evaluate) and on VEC (whether four
 // consecutive elements move as one 128-bit access).
@@ -511,17 +511,6 @@ struct SlabIn {
 __device__ __forceinline__ bool slab_passes_stand_back(const SlabIn& slab) { return 2u * __ldg(slab.local) > slab.sampled; }
 constexpr int kSlabWarpTile = 512;
 
-// Whether `leaf` (an array from outside the cluster) is read by member i at i's own index: through array operands
-// of maps and zipWiths only.
-constexpr bool reads_in_place(const CCluster& c, int i, int leaf) {
-  if (i == leaf) return true;
-  const CNode& n = c.nodes[i];
-  if (!n.member || (n.kind != ACC_MAP && n.kind != ACC_ZIPWITH)) return false;
-  for (int k = 0; k < n.narr; ++k)
-    if (reads_in_place(c, n.in[k], leaf)) return true;
-  return false;
-}
-
 // The gathered values of warp tile `wt` (kSlabWarpTile elements, grouped by slab where `staged` holds them) in element
 // order: lane's elements (j * 32 + lane) * 4 .. + 3 in gathered[j].  The stable counting sort of k_slab_partition is undone
 // from the slab codes and the group sizes, through `stage` (kSlabWarpTile words of shared memory that the warp owns).
@@ -759,26 +748,6 @@ struct ScanTile {
     }
   }
 
-  // The lines that the warp's part from walk position warp_base of `row` on will read in place, asked into L2
-  // (left-to-right scans; arrays from outside the cluster that the scanned operand reads at its own index).
-  static __device__ __forceinline__ void prefetch_operands(const Args<N>& a, int row, int warp_base) {
-    if constexpr (!REV) {
-      const int lane = threadIdx.x & 31;
-      const int n = a.C;
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        if constexpr (!CL::c.nodes[i].member && reads_in_place(CL::c, sn.in[0], i)) {
-          const char* base = reinterpret_cast<const char*>(a.n[i].ptr) + (size_t)row * n * 4;
-#pragma unroll
-          for (int k = 0; k < PART; k += 1024) {
-            const int at = warp_base + k + lane * 32;
-            if (at < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)at * 4));
-          }
-        }
-      });
-    }
-  }
-
   // SLAB: the staged values and codes of warp tile `wt` are asked into L2 ahead of their use
   static __device__ __forceinline__ void prefetch_part(const Args<N>& a, int wt, const SlabIn& slab) {
     const int lane = threadIdx.x & 31;
@@ -791,12 +760,8 @@ struct ScanTile {
 };
 
 // Tile after tile with the whole block in step: every warp scans its part, one warp looks back, every warp stores.
-// STATIC: block b walks tiles b, b + G, b + 2G, ... of a grid of G blocks that are all resident at once (a
-// cooperative launch): no ticket, whose atomic every warp of the block would otherwise wait for at the top of every
-// tile (measured on a streaming scan of 2^26 floats: 28 barrier-stall cycles per issued instruction, 19 % of the
-// issue slots used).  A tile's predecessors belong to the blocks before this one in the same round, or to an
-// earlier round, so they are running or done.  Without that guarantee the tiles are claimed from a ticket.
-template <class CL, bool VEC, bool SLAB, bool STATIC = false>
+// Tiles are claimed from a ticket: a tile's predecessors have been claimed by blocks that are running or done.
+template <class CL, bool VEC, bool SLAB>
 __device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per_row, int n_tiles, const SlabIn& slab) {
   using T = ScanTile<CL, VEC, SLAB>;
   constexpr int BLOCK = T::BLOCK, FN = T::FN, DT = T::DT;
@@ -806,33 +771,15 @@ __device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per
   __shared__ __align__(16) uint32_t slab_stage[SLAB ? BLOCK / 32 : 1][SLAB ? kSlabWarpTile : 1];   // read and written 128 bits at a time
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-  for (int round = 0;; ++round) {
-    int tile;
-    if constexpr (STATIC) {
-      // (no barrier here: what a round shares through shared memory is read before its second barrier or right
-      // after it, and written again only behind the next round's first barrier)
-      tile = (int)blockIdx.x + round * (int)gridDim.x;
-    } else {
-      __syncthreads();
-      if (threadIdx.x == 0) tile_id = (int)atomicAdd(a.scratch, 1u);
-      __syncthreads();
-      tile = tile_id;
-    }
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) tile_id = (int)atomicAdd(a.scratch, 1u);
+    __syncthreads();
+    const int tile = tile_id;
     if (tile >= n_tiles) return;
     const int row = tile / tiles_per_row, in_row = tile - row * tiles_per_row;
     const int warp_base = in_row * T::TILE + warp * T::PART;
 
-    if constexpr (STATIC) {
-      // this block's next tile is known: what it reads is on its way while this tile is scanned and looked back
-      // for (config-3 shape, 2^26 elements: 0.726 -> 0.704 ms for the cluster)
-      const int next = tile + (int)gridDim.x;
-      if constexpr (SLAB) {
-        T::prefetch_part(a, next * (BLOCK / 32) + warp, slab);
-      } else if (next < n_tiles) {
-        const int nrow = next / tiles_per_row;
-        T::prefetch_operands(a, nrow, (next - nrow * tiles_per_row) * T::TILE + warp * T::PART);
-      }
-    }
     uint32_t val[T::ROWS][T::W];
     const uint32_t carry = T::scan_part(a, row, warp_base, tile * (BLOCK / 32) + warp, slab, slab_stage[SLAB ? warp : 0], val);
     if (lane == 0) warp_total[warp] = carry;
@@ -865,17 +812,20 @@ template <int FIRST> __device__ __forceinline__ void bar_arrive(int half, int co
 // nothing but look back.  A scanning warp leaves its part's values in shared memory, tells the look-back warp that
 // the part's total is in, goes on to its part of the block's next tile, and only then comes back for the values,
 // which it finishes with what the look-back warp has found meanwhile.  Where the whole block waits for the look-back
-// (scan_tiles), the blocks of a cooperative grid fall into step and an SM's blocks all wait at once.
+// (scan_tiles), the blocks of a cooperative grid fall into step and an SM's blocks all wait at once.  Block b walks
+// tiles b, b + G, b + 2G, ... of a grid of G blocks that are all resident at once (a cooperative launch): a tile's
+// predecessors belong to the blocks before this one in the same round, or to an earlier round, so they are running or
+// done.  Used by the merging scan behind slab passes (config-3 shape, 2^26 elements: 0.704 ms with the block in step).
 // Round r uses half r & 1 of everything shared.  Barrier 1 + half: a part's total is in shared memory (the scanning
 // warps arrive, the look-back warp waits); barrier 3 + half: what comes before each part is in shared memory (the
 // look-back warp arrives, the scanning warps wait).  Every warp of a block walks the same rounds, so that each
-// barrier sees BLOCK + 32 threads once a round.  Only for grids whose blocks are all resident (STATIC tiles).
-template <class CL, bool VEC, bool SLAB>
+// barrier sees BLOCK + 32 threads once a round.
+template <class CL>
 __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int tiles_per_row, int n_tiles, const SlabIn& slab) {
-  using T = ScanTile<CL, VEC, SLAB>;
-  constexpr int BLOCK = T::BLOCK, WARPS = BLOCK / 32, FN = T::FN, DT = T::DT, ROWS = T::ROWS, W = T::W;
+  using T = ScanTile<CL, true, true>;
+  constexpr int BLOCK = T::BLOCK, WARPS = BLOCK / 32, FN = T::FN, DT = T::DT, ROWS = T::ROWS;
   static_assert(WARPS <= 32, "one lane of the look-back warp per scanning warp");
-  __shared__ __align__(16) uint32_t values[2][T::TILE];    // a part's scanned values between its two visits (SLAB: first the staging area of its merge)
+  __shared__ __align__(16) uint32_t values[2][T::TILE];    // a part's scanned values between its two visits, before that the staging area of its merge
   __shared__ uint32_t part_total[2][WARPS];
   __shared__ uint32_t part_before[2][WARPS];               // what of the row comes before each part
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -908,15 +858,11 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
     bar_sync<3>(half, BLOCK + 32);
     const uint32_t before = part_before[half][warp];
     const uint32_t* mine = values[half] + warp * T::PART;
-    uint32_t val[ROWS][W];
+    uint32_t val[ROWS][4];
 #pragma unroll
     for (int j = 0; j < ROWS; ++j) {
-      if constexpr (VEC) {
-        const uint4 q = *reinterpret_cast<const uint4*>(mine + (j * 32 + lane) * 4);
-        val[j][0] = q.x; val[j][1] = q.y; val[j][2] = q.z; val[j][3] = q.w;
-      } else {
-        val[j][0] = mine[j * 32 + lane];
-      }
+      const uint4 q = *reinterpret_cast<const uint4*>(mine + (j * 32 + lane) * 4);
+      val[j][0] = q.x; val[j][1] = q.y; val[j][2] = q.z; val[j][3] = q.w;
     }
     T::finish_part(a, row, in_row * T::TILE + warp * T::PART, before, val);
   };
@@ -928,21 +874,13 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
     const int half = round & 1;
     const int row = tile / tiles_per_row, in_row = tile - row * tiles_per_row;
     uint32_t* mine = values[half] + warp * T::PART;
-    if constexpr (SLAB) {
-      T::prefetch_part(a, (tile + G) * WARPS + warp, slab);
-    } else if (tile + G < n_tiles) {
-      const int nrow = (tile + G) / tiles_per_row;
-      T::prefetch_operands(a, nrow, (tile + G - nrow * tiles_per_row) * T::TILE + warp * T::PART);
-    }
+    T::prefetch_part(a, (tile + G) * WARPS + warp, slab);
     {
-      uint32_t val[ROWS][W];
+      uint32_t val[ROWS][4];
       const uint32_t total = T::scan_part(a, row, in_row * T::TILE + warp * T::PART, tile * WARPS + warp, slab, mine, val);
-      __syncwarp();                                        // (SLAB: every lane has taken its merged values out of `mine`)
+      __syncwarp();                                        // (every lane has taken its merged values out of `mine`)
 #pragma unroll
-      for (int j = 0; j < ROWS; ++j) {
-        if constexpr (VEC) *reinterpret_cast<uint4*>(mine + (j * 32 + lane) * 4) = make_uint4(val[j][0], val[j][1], val[j][2], val[j][3]);
-        else mine[j * 32 + lane] = val[j][0];
-      }
+      for (int j = 0; j < ROWS; ++j) *reinterpret_cast<uint4*>(mine + (j * 32 + lane) * 4) = make_uint4(val[j][0], val[j][1], val[j][2], val[j][3]);
       if (lane == 0) part_total[half][warp] = total;
     }
     bar_arrive<1>(half, BLOCK + 32);

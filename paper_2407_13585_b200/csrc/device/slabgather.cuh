@@ -228,12 +228,12 @@ __global__ void __launch_bounds__(kBlock) k_slab_gather(const __grid_constant__ 
 }
 
 // (five blocks per SM: the merge is issue bound, and a quarter more warps pay for a few spilled words)
-template <class CL, bool STATIC = false>
+template <class CL>
 __global__ void __launch_bounds__(scan_block<CL>(), 5) k_scan_merge(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles,
                                                                   const SlabIn slab_in) {
   SlabIn slab = slab_in;
   if (slab_passes_stand_back(slab)) slab.full_tiles = 0;     // every warp tile gathers for itself
-  scan_tiles<CL, true, true, STATIC>(a, tiles_per_row, n_tiles, slab);
+  scan_tiles<CL, true, true>(a, tiles_per_row, n_tiles, slab);
 }
 
 // Every root of a scan-less cluster stored from the gathered values of the earlier launches: a warp puts a warp tile
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(scan_block<CL>() + 32, 5) k_scan_merge_pipelin
                                                                                   const SlabIn slab_in) {
   SlabIn slab = slab_in;
   if (slab_passes_stand_back(slab)) slab.full_tiles = 0;     // every warp tile gathers for itself
-  scan_tiles_pipelined<CL, true, true>(a, tiles_per_row, n_tiles, slab);
+  scan_tiles_pipelined<CL>(a, tiles_per_row, n_tiles, slab);
 }
 
 }  // namespace dev
