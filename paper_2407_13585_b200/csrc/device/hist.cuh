@@ -86,6 +86,17 @@ __device__ __forceinline__ void red_add_bin(uint32_t k, uint32_t per_cta, uint32
       "@!p red.global.add.s32 [ga], %4;\n\t}"
       ::"r"(k), "r"(per_cta), "r"(bins_addr), "l"(rest), "r"(v) : "memory");
 }
+// Four updates of bins that may lie in either, or (rest == nullptr: all bins are in shared memory) without the choice per
+// element (10^8 keys into 4096 bins 118 -> 96 us, 13101521 keys into 47631 bins 46 -> 42 us).
+__device__ __forceinline__ void red_add_four(const uint32_t (&k)[4], uint32_t per_cta, uint32_t bins_addr, const int* rest, const int (&v)[4]) {
+  if (rest == nullptr) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(bins_addr + k[j] * 4u), "r"(v[j]) : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) red_add_bin(k[j], per_cta, bins_addr, rest, v[j]);
+  }
+}
 __device__ __forceinline__ void red_add_global(double* p, double v) {
   asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
@@ -181,6 +192,10 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
   }
   const float cap = exp2f((float)cap_log2);
   const float up = exp2f((float)S);
+  // the denormal 2^(S - 149): a value in [0, 2^23) times it has the integer value * 2^S as its bits (one product, without the
+  // conversion and the test that other values need: 2^27 keys 186.2 -> 184.5 us; used where S >= 0 and the values are known
+  // to be integers, which makes S <= 21)
+  const float up_bits = __uint_as_float(S >= 0 && S < 23 ? 1u << S : 0u);
   const double down = exp2((double)-S);
 
   auto scatter_one = [&](uint32_t k, uint32_t xbits) {
@@ -209,6 +224,7 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
   };
 
   const bool fast_ok = group == 1 && S >= 0;
+  const int* const rest = plan.overflow ? spill - per_cta : nullptr;
   const uint32_t bins_addr = (uint32_t)__cvta_generic_to_shared(bins_smem);
   uint32_t it = 0;
   // FULL: every chunk of the trip and of the trips prefetched from it lies inside the array (no test per chunk)
@@ -277,10 +293,10 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
           // integers below m, and (m - 1) * 2^S below cap / 2 by the choice of S: every product is an
           // exact integer the bins can take, so only the indices are looked at
           if (fast_ok & (kmax < n_bins)) {
+            int v[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              red_add_bin(key[u].v[j], (uint32_t)per_cta, bins_addr, spill - per_cta,
-                          __float_as_int(__fadd_rn(__fmul_rn(f_(val[u].v[j]), up), 12582912.0f)) - 0x4B400000);
+            for (int j = 0; j < 4; ++j) v[j] = __float_as_int(__fmul_rn(f_(val[u].v[j]), up_bits));
+            red_add_four(key[u].v, (uint32_t)per_cta, bins_addr, rest, v);
             continue;
           }
         }
@@ -293,12 +309,11 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
           big = fmaxf(big, fabsf(t[j]));
         }
         if (fast_ok & (kmax < n_bins) & (off == 0.0f) & (big < cap)) {
+          // (a zero is added like any other value: skipping it would cost more than it saves)
+          int v[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t k = key[u].v[j];
-            // (a zero is added like any other value: skipping it would cost more than it saves)
-            red_add_bin(k, (uint32_t)per_cta, bins_addr, spill - per_cta, __float_as_int(shifted[j]) - 0x4B400000);
-          }
+          for (int j = 0; j < 4; ++j) v[j] = __float_as_int(shifted[j]) - 0x4B400000;
+          red_add_four(key[u].v, (uint32_t)per_cta, bins_addr, rest, v);
         } else {
 #pragma unroll
           for (int j = 0; j < 4; ++j) scatter_one(key[u].v[j], val[u].v[j]);

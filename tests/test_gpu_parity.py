@@ -51,6 +51,12 @@ def test_config5_any_length(n, bins):
     assert check_program(W.config5(n, bins)) == 10
 
 
+# the most bins that a block's shared memory takes, and one more
+@pytest.mark.parametrize("n,bins", [(458761, 57344), (458766, 57345)])
+def test_config5_bins_that_just_fit(n, bins):
+    assert check_program(W.config5(n, bins)) == 10
+
+
 # tiles copied word by word: one, two and three columns in the last chunk of four, of a tile that is nearly empty or nearly full
 @pytest.mark.parametrize("rows", [2561, 2622, 2623])
 def test_config2_any_extent(rows):
