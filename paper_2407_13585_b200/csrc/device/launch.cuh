@@ -550,9 +550,10 @@ struct Launcher {
         }
       }
       if constexpr (kRingShape) {
-        if constexpr (dev::can_stage<CL>()) {
+        if constexpr (dev::can_stage<CL>() && dev::count_if<CL>(dev::is_scan_root) == 1) {
           // a gather below the scan and few elements: tiles that look back one after the other, in an ordinary launch, are
-          // quicker than staging in a cooperative one (30000 elements 8.7 against 12.4 us)
+          // quicker than staging in a cooperative one (30000 elements 8.7 against 12.4 us).  Several scans share the ring's
+          // walk at any size: k_scan takes one.
           if (R == 1 && C > dev::kScanBlockRow && C <= dev::kScanFewElements && use_ring(L, C)) {
             if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
             else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);

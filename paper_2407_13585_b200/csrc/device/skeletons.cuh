@@ -573,7 +573,7 @@ struct ScanTile {
   static constexpr int TILE = BLOCK * scan_rows<CL>() * 4;
   static constexpr int PART = TILE / (BLOCK / 32);         // elements of a tile that one warp takes
   static constexpr int S = first_scan<CL>();
-  static_assert(S >= 0, "k_scan needs a scan member");
+  static_assert(count_if<CL>(is_scan_root) == 1, "a tile is scanned for one scan: further ones would never be written");
   static constexpr CNode sn = CL::c.nodes[S];
   static constexpr int FN = sn.fn, DT = sn.dtype;
   static constexpr bool REV = sn.kind == ACC_SCANR;

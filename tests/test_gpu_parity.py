@@ -627,6 +627,14 @@ def test_gather_staged_for_a_scan(n):
     check_program(prog, [[-1, -1, 0, 0, 0, 0], [-1, -1, 0, 1, 1, 1]])
 
 
+# two scans of one cluster, both over a gather or one of them: a block to the row, the ring (with few elements too, where one
+# scan alone looks back tile by tile), around the lines between them
+@pytest.mark.parametrize("n", [16381, 16382, 20001, 131072, 131073])
+@pytest.mark.parametrize("which", [3, 5, 9])
+def test_scans_beside_one_over_a_gather(which, n):
+    check_program(W.gathered_scans(n, 1 << 12, which), [[-1, -1, 0, 0, 0, 0]], passes=True)
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))

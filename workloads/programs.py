@@ -418,6 +418,28 @@ def gather_three_roots(n_src=1 << 12, n=1 << 10):
     return Program("gather_three_roots", nodes, [2, 3, 4], index_bound={"idx": n_src, "x": 1 << 30})
 
 
+def gathered_scans(n=1 << 10, n_src=1 << 10, which=3):
+    """Several scans in one cluster, one or more of them over a gathered operand: k = idx & (n_src-1); h = x[k], and of the
+    roots those that `which` names by its bits: 1 running sum of h, 2 running maximum of h, 4 seeded exclusive sum of h,
+    8 running sum of k, 16 total of k.  n_src is a power of two."""
+    assert n_src & (n_src - 1) == 0
+    nodes = [
+        _inp("x", "i32", (n_src,)),
+        _inp("idx", "i32", (n,)),
+        Node("map", "i32", (n,), (1,), 1, fn="and_mask", iparam=(n_src - 1,), name="k"),
+        Node("gather", "i32", (n,), (2, 0), 2, name="h"),
+    ]
+    roots = [
+        Node("scanl", "i32", (n,), (3,), 1, fn="add", name="s"),
+        Node("scanl", "i32", (n,), (3,), 1, fn="max", name="m"),
+        Node("scanl", "i32", (n,), (3,), 1, fn="add", iparam=(7,), exclusive=True, name="e"),
+        Node("scanl", "i32", (n,), (2,), 1, fn="add", name="t"),
+        Node("fold", "i32", (), (2,), 1, fn="add", name="total"),
+    ]
+    nodes += [nd for b, nd in enumerate(roots) if (which >> b) & 1]
+    return Program("gathered_scans_%d" % which, nodes, list(range(4, len(nodes))), index_bound={"x": 1 << 30, "idx": 1 << 30})
+
+
 def histogram_2d(rows=64, n=4096, bins=256):
     """The scatter histogram of config 5 over a rank-2 array of keys, with per-row totals beside it: the
     scatter and the row folds share producers but no kernel walk."""
