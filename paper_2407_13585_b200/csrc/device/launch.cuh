@@ -814,6 +814,7 @@ struct Passes {
       return Launcher<CL>::launch(L);
     } else {
       ClusterLaunch pass = L;
+      pass.extra_launches = 0;                        // (L's own are counted already)
       const int rc = launch_from<T, 0>(pass);
       L.extra_launches += pass.extra_launches;
       return rc;

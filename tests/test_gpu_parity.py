@@ -635,6 +635,15 @@ def test_scans_beside_one_over_a_gather(which, n):
     check_program(W.gathered_scans(n, 1 << 12, which), [[-1, -1, 0, 0, 0, 0]], passes=True)
 
 
+# three scans and a total: four passes over short rows, over long ones a shared walk and the total's
+@pytest.mark.parametrize("n,launches", [(16381, 4), (16382, 2), (300001, 2)])
+def test_launches_of_shared_and_single_passes_are_counted_once(n, launches):
+    prog = W.gathered_scans(n, 1 << 12, 27)
+    check_program(prog, [[-1, -1] + [0] * 6], passes=True)
+    _, g = gpu_run(prog, W.make_inputs(prog), [-1, -1] + [0] * 6)
+    assert g.launch_count() == launches
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))
