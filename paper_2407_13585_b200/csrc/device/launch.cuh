@@ -750,9 +750,19 @@ template <class CL, bool TOGETHER> constexpr PassPlan pass_plan() {
   return p;
 }
 
+// How many of the scans, each in a pass of its own, gather in a way that slab passes can serve (slabgather.cuh).
+template <class CL, int P>
+struct SinglePass {
+  static constexpr CCluster c = pass_cluster(CL::c, pass_plan<CL, false>().keep[P], P == 0);
+};
+template <class CL, int P = 0> constexpr int slab_passes() {
+  if constexpr (P < pass_plan<CL, false>().n) return (dev::slab_gather_eligible<SinglePass<CL, P>>() ? 1 : 0) + slab_passes<CL, P + 1>();
+  else return 0;
+}
+
 template <class CL, bool TOGETHER, int P>
 struct PassOf {
-  static constexpr int kScanForms = pass_plan<CL, false>().n == pass_plan<CL, true>().n ? 3 : TOGETHER ? 2 : 1;
+  static constexpr int kScanForms = pass_plan<CL, false>().n == pass_plan<CL, true>().n ? 3 : TOGETHER ? 2 : slab_passes<CL>() == 1 ? 3 : 1;
   static constexpr CCluster c = pass_cluster(CL::c, pass_plan<CL, TOGETHER>().keep[P], P == 0);
 };
 
@@ -761,13 +771,19 @@ struct Passes {
   static constexpr int kSingly = pass_plan<CL, false>().n, kTogether = pass_plan<CL, true>().n;
 
   // Scans share a pass where they go through the ring (long rows); k_scan_rows keeps a row's operands in registers and
-  // takes one scan at a time.
+  // takes one scan at a time.  A scan whose gather runs as slab passes keeps a pass of its own, for a shared walk gathers
+  // from DRAM (2^26 indices into 256 MB beside a running sum: 890 us apart, 1354 shared); two such scans over one gather
+  // are no slower shared (1341 against 1347 us, with the sum 1505 against 1621).
   static bool together(const ClusterLaunch& L) {
     if constexpr (kSingly == kTogether) return false;
     else {
       int R, C;
-      return Launcher<CL>::domain(L, R, C) && C > dev::kScanBlockRow;
+      return Launcher<CL>::domain(L, R, C) && C > dev::kScanBlockRow && !(slab_passes<CL>() == 1 && slab_shapes<0>(L, R, C));
     }
+  }
+  template <int P> static bool slab_shapes(const ClusterLaunch& L, int R, int C) {
+    if constexpr (P < kSingly) return Launcher<PassOf<CL, false, P>>::slab_shapes_ok(L, R, C) || slab_shapes<P + 1>(L, R, C);
+    else return false;
   }
 
   template <bool T, int P>

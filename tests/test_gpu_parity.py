@@ -644,6 +644,17 @@ def test_launches_of_shared_and_single_passes_are_counted_once(n, launches):
     assert g.launch_count() == launches
 
 
+def test_slab_passes_beside_another_scan():
+    """A scan over a gather from 128 MB runs as slab passes (probe, partition, four slabs, merge) although a second scan of
+    its direction is in the cluster, which walks by itself; two scans over the gather share a walk."""
+    for which, launches in ((9, 7 + 1), (3, 1)):
+        prog = W.gathered_scans(1 << 22, 1 << 25, which)
+        inputs = W.make_inputs(prog)
+        got, g = gpu_run(prog, inputs, [-1, -1, 0, 0, 0, 0])
+        assert g.launch_count() == launches
+        compare(prog, oracle_run(prog, np_inputs(inputs)), got, "which = %d" % which)
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))
