@@ -162,11 +162,13 @@ struct Launcher {
   }
 
   // Scans through the shared-memory ring (k_scan_ring), or a warp or block per row where rows are short (k_scan_rows);
-  // without them, where a chunk behind an index map would not be a 128-bit access, k_scan.
+  // without them, where a chunk behind an index map would not be a 128-bit access, or where rows are long and the ring does
+  // not serve the scan's operand, k_scan.
   static constexpr bool kRingShape = kHasScan && dev::scan_ring_eligible<CL>();
+  static constexpr bool kRingServes = kHasScan && dev::ring_serves<CL>();
   static bool use_ring(const ClusterLaunch& L, int C) {
     if constexpr (!kRingShape) return false;
-    else return !dev::has_index_map<CL>() || vec_ok(L, C);
+    else return (!dev::has_index_map<CL>() || vec_ok(L, C)) && (kRingServes || C <= dev::kScanBlockRow);
   }
   // (a row of C elements may begin up to three words into its first 16-byte chunk)
   static int ring_tiles_per_row(int R, int C) {
@@ -199,7 +201,7 @@ struct Launcher {
           else dev::k_scan_rows<CL, 16, 8><<<grid, 512, 0, L.stream>>>(a);
         }
       }
-      if constexpr ((kForms & 2) != 0) {
+      if constexpr ((kForms & 2) != 0 && kRingServes) {
         if (C > dev::kScanBlockRow) {
           int per_row = ring_tiles_per_row(R, C);
           const int64_t tiles = (int64_t)R * per_row;
@@ -564,7 +566,7 @@ struct Launcher {
         }
       }
       if (use_ring(L, C)) return launch_ring(L, a, R, C);
-      if constexpr (!kRingShape) {
+      if constexpr (!kRingServes) {
         if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
         else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
       } else if constexpr (dev::has_index_map<CL>()) {
@@ -711,7 +713,7 @@ constexpr uint64_t scans_of_kind(const CCluster& c, int kind) {
     if (dev::is_scan_root(c.nodes[i]) && c.nodes[i].kind == kind) m |= 1ull << i;
   return m;
 }
-// Whether the scans of one direction can share a walk: as one pass they must be something k_scan_ring takes, whatever
+// Whether the scans of one direction can share a walk: as one pass they must be something k_scan_ring serves, whatever
 // the shapes.  (Each array is then read once for all of them.)
 template <class CL, int KIND>
 struct ScansTogether {
@@ -719,7 +721,7 @@ struct ScansTogether {
 };
 template <class CL, int KIND> constexpr bool scans_share_a_pass() {
   if constexpr (scans_of_kind(CL::c, KIND) == 0) return false;
-  else return dev::scan_ring_eligible<ScansTogether<CL, KIND>>() && !dev::has_index_map<ScansTogether<CL, KIND>>();
+  else return dev::ring_serves<ScansTogether<CL, KIND>>() && !dev::has_index_map<ScansTogether<CL, KIND>>();
 }
 
 // TOGETHER: the scans of one direction share a pass where they can.

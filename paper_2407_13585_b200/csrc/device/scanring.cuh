@@ -213,6 +213,30 @@ template <class CL> struct StagedScan { static constexpr CCluster c = with_array
 // (the staged arrays must come through the ring: they are written and read in one kernel)
 template <class CL> constexpr bool can_stage() { return has_stage_targets<CL>() && ring_wanted<StagedScan<CL>>(true) <= kRingMaxSlots; }
 
+// Whether everything the scans are computed from comes through the ring, element by element.  The ring evaluates the
+// operands in both of its visits: what it would have to read from memory at other positions, it would read twice (the sum of
+// two gathers stored nowhere, scanned: 2^24 elements 1101 us, by k_scan 222; a reversed array, 2^26 elements: 205 and 157).
+template <class CL> constexpr bool fed_by_ring(int i) {
+  const CNode& n = CL::c.nodes[i];
+  if (!n.member) return in_ring<CL>(i);
+  if (n.kind == ACC_GENERATE) return true;
+  if (n.kind != ACC_MAP && n.kind != ACC_ZIPWITH && (n.kind != ACC_BACKPERMUTE || n.idxfn != ACC_IDX_IDENTITY)) return false;
+  for (int k = 0; k < n.narr; ++k)
+    if (!fed_by_ring<CL>(n.in[k])) return false;
+  return true;
+}
+template <class CL> constexpr bool operands_fed_by_ring() {
+  for (int i = 0; i < CL::c.n; ++i)
+    if (is_scan_root(CL::c.nodes[i]) && !fed_by_ring<CL>(CL::c.nodes[i].in[0])) return false;
+  return true;
+}
+// ... as they are, or once the costly members are staged
+template <class CL> constexpr bool ring_serves() {
+  if constexpr (!scan_ring_eligible<CL>()) return false;
+  else if constexpr (can_stage<CL>()) return operands_fed_by_ring<StagedScan<CL>>();
+  else return operands_fed_by_ring<CL>();
+}
+
 constexpr int kRingDirectRounds = 8;   // rounds up to which every block adds the totals of a round up for itself
 constexpr int kRingPollPause = 50;     // ns between two looks at totals that were missing
 // Rows of up to kScanWarpRow elements get a warp each, up to kScanBlockRow a block each (a row may begin three words into its

@@ -655,6 +655,44 @@ def test_slab_passes_beside_another_scan():
         compare(prog, oracle_run(prog, np_inputs(inputs)), got, "which = %d" % which)
 
 
+# operands that the ring does not serve (two gathers and one array to stage them in; an array read backwards): a block to a
+# row up to 16381 elements, beyond that tiles that look back, with 128-bit accesses and without
+@pytest.mark.parametrize("n", [5, 16381, 16382, 70000, 70001, 1 << 20])
+def test_scans_of_operands_that_do_not_come_through_the_ring(n):
+    check_program(W.sum_of_two_gathers(n), [[-1, -1, -1, 0, 0, 0, 0]])
+    check_program(W.scan_of_reversed(n), [[-1, 0, 0]])
+
+
+def test_scan_over_two_gathers_costs_no_more_than_its_nodes():
+    """The cluster reads each gathered word once: it takes no longer than its four nodes alone (a factor of 1.5 for what else
+    runs on the device; read twice, it took three times as long)."""
+    import torch
+    from paper_2407_13585_b200 import binding as B
+    prog = W.sum_of_two_gathers(1 << 24)
+    inputs = {k: v.cuda() for k, v in W.make_inputs(prog).items()}
+    g = B.Graph(prog.nodes, prog.outputs)
+    g.set_partition([-1, -1, -1, 0, 0, 0, 0])
+    for i, t in inputs.items():
+        g.bind(i, t)
+    out = torch.empty(1 << 24, dtype=torch.int32, device="cuda")
+    g.bind(6, out)
+
+    def milliseconds(executor):
+        begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        g.run(executor)
+        times = []
+        for _ in range(5):
+            begin.record()
+            for _ in range(4):
+                g.run(executor, finish=False)
+            end.record()
+            end.synchronize()
+            times.append(begin.elapsed_time(end) / 4)
+        return min(times)
+
+    assert milliseconds(B.FUSED) <= 1.5 * milliseconds(B.UNFUSED)
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))

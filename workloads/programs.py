@@ -440,6 +440,30 @@ def gathered_scans(n=1 << 10, n_src=1 << 10, which=3):
     return Program("gathered_scans_%d" % which, nodes, list(range(4, len(nodes))), index_bound={"x": 1 << 30, "idx": 1 << 30})
 
 
+def sum_of_two_gathers(n=1 << 10):
+    """A running sum over x[i] + x[j], neither of which is stored."""
+    nodes = [
+        _inp("x", "i32", (n,)),
+        _inp("i", "i32", (n,)),
+        _inp("j", "i32", (n,)),
+        Node("gather", "i32", (n,), (1, 0), 2, name="g"),
+        Node("gather", "i32", (n,), (2, 0), 2, name="h"),
+        Node("zipwith", "i32", (n,), (3, 4), 2, fn="add", name="u"),
+        Node("scanl", "i32", (n,), (5,), 1, fn="add", name="s"),
+    ]
+    return Program("sum_of_two_gathers", nodes, [6], index_bound={"x": 1 << 30, "i": n, "j": n})
+
+
+def scan_of_reversed(n=1 << 10):
+    """The running sum of an array read backwards."""
+    nodes = [
+        _inp("x", "f32", (n,)),
+        Node("backpermute", "f32", (n,), (0,), 1, idx_fn="reverse", name="y"),
+        Node("scanl", "f32", (n,), (1,), 1, fn="add", name="s"),
+    ]
+    return Program("scan_of_reversed", nodes, [2])
+
+
 def histogram_2d(rows=64, n=4096, bins=256):
     """The scatter histogram of config 5 over a rank-2 array of keys, with per-row totals beside it: the
     scatter and the row folds share producers but no kernel walk."""
