@@ -163,12 +163,12 @@ struct Launcher {
 
   // Scans through the shared-memory ring (k_scan_ring), or a warp or block per row where rows are short (k_scan_rows);
   // without them, where a chunk behind an index map would not be a 128-bit access, or where rows are long and the ring does
-  // not serve the scan's operand, k_scan.
+  // not serve the scan's operand or the device cannot launch a grid with all blocks resident, k_scan.
   static constexpr bool kRingShape = kHasScan && dev::scan_ring_eligible<CL>();
   static constexpr bool kRingServes = kHasScan && dev::ring_serves<CL>();
   static bool use_ring(const ClusterLaunch& L, int C) {
     if constexpr (!kRingShape) return false;
-    else return (!dev::has_index_map<CL>() || vec_ok(L, C)) && (kRingServes || C <= dev::kScanBlockRow);
+    else return (!dev::has_index_map<CL>() || vec_ok(L, C)) && (C <= dev::kScanBlockRow || (kRingServes && cooperative_launch_ok()));
   }
   // (a row of C elements may begin up to three words into its first 16-byte chunk)
   static int ring_tiles_per_row(int R, int C) {
@@ -223,7 +223,6 @@ struct Launcher {
             if (!opt_in_shared_memory(kern, K::SMEM, granted))
               return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
             // (blocks read one another's totals: all of them resident)
-            if (!cooperative_launch_ok()) return set_error(ACC_ERR_UNSUPPORTED, "the device cannot launch cooperatively");
             void* params[] = {&a, &per_row, &n_tiles, &whole};
             cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tiles, sm_count())), dim3(K::THREADS), params, K::SMEM, L.stream);
           }
@@ -234,6 +233,20 @@ struct Launcher {
       return ACC_OK;
     } else {
       return set_error(ACC_ERR_NO_KERNEL, "not a cluster of scans");
+    }
+  }
+
+  // k_scan: tiles that look back one after the other, claimed from a ticket.
+  static int launch_look_back(const ClusterLaunch& L, const dev::Args<N>& a, bool vec, int tiles_per_row, int64_t tiles) {
+    if constexpr (dev::count_if<CL>(dev::is_scan_root) == 1) {
+      const int grid = (int)std::min<int64_t>(tiles, (int64_t)sm_count() * (1536 / kScanBlock));
+      if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles);
+      else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles);
+      const cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+      return ACC_OK;
+    } else {
+      return set_error(ACC_ERR_NO_KERNEL, "several scans walk together through the ring only");
     }
   }
 
@@ -556,22 +569,11 @@ struct Launcher {
           // a gather below the scan and few elements: tiles that look back one after the other, in an ordinary launch, are
           // quicker than staging in a cooperative one (30000 elements 8.7 against 12.4 us).  Several scans share the ring's
           // walk at any size: k_scan takes one.
-          if (R == 1 && C > dev::kScanBlockRow && C <= dev::kScanFewElements && use_ring(L, C)) {
-            if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
-            else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
-            return ACC_OK;
-          }
+          if (R == 1 && C > dev::kScanBlockRow && C <= dev::kScanFewElements && use_ring(L, C)) return launch_look_back(L, a, vec, per_row, tiles);
         }
       }
       if (use_ring(L, C)) return launch_ring(L, a, R, C);
-      if constexpr (!kRingServes) {
-        if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
-        else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
-      } else if constexpr (dev::has_index_map<CL>()) {
-        dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, per_row, (int)tiles);
-      }
+      return launch_look_back(L, a, vec, per_row, tiles);
     } else if constexpr (kHasRowFold) {
       if (R == 0) return ACC_OK;
       const int grid = std::min(R, sm_count() * 16);
@@ -780,7 +782,7 @@ struct Passes {
     if constexpr (kSingly == kTogether) return false;
     else {
       int R, C;
-      return Launcher<CL>::domain(L, R, C) && C > dev::kScanBlockRow && !(slab_passes<CL>() == 1 && slab_shapes<0>(L, R, C));
+      return Launcher<CL>::domain(L, R, C) && C > dev::kScanBlockRow && cooperative_launch_ok() && !(slab_passes<CL>() == 1 && slab_shapes<0>(L, R, C));
     }
   }
   template <int P> static bool slab_shapes(const ClusterLaunch& L, int R, int C) {

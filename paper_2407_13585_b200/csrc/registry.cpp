@@ -2,6 +2,7 @@
 // of the program translation units when the library is loaded.
 #include "registry.h"
 
+#include <atomic>
 #include <map>
 
 namespace acc {
@@ -35,11 +36,12 @@ int sm_count() {
 }
 
 bool cooperative_launch_ok() {
+  static std::atomic<int8_t> known[64];                    // by device: 0 not asked yet, 1 no, 2 yes
   int dev = 0, ok = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&ok, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (dev < 64 && known[dev] != 0) return known[dev] == 2;
+  if (cudaDeviceGetAttribute(&ok, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (dev < 64) known[dev] = ok ? 2 : 1;
   return ok != 0;
 }
 

@@ -693,6 +693,39 @@ def test_scan_over_two_gathers_costs_no_more_than_its_nodes():
     assert milliseconds(B.FUSED) <= 1.5 * milliseconds(B.UNFUSED)
 
 
+WITHOUT_COOPERATIVE_LAUNCHES = """
+import ctypes, sys
+ctypes.CDLL(sys.argv[1], mode=ctypes.RTLD_GLOBAL)          # its definition is found before the library's own
+sys.path[:0] = sys.argv[2:]
+import workloads as W
+from helpers import compare, gpu_run, oracle_run
+from paper_2407_13585_b200 import binding, build
+binding.load_kernel_library(build.TEST_LIB)
+for prog, pi, launches in ((W.row_scans(3, 20001), [-1, 0, 1, 1], 2), (W.scan_consumers(70001), [-1, -1, 0, 0, 0, 1, 1, 0, 0], 3),
+                           (W.gathered_scans(140000, 1 << 12, 27), [-1, -1] + [0] * 6, 4),
+                           (W.config5(1 << 19, 1 << 15), [-1, -1, 0, 0, 0, 0, 1], 2), (W.config2(2600), [-1, 0, 0, 0], 1)):
+    inputs = W.make_inputs(prog)
+    got, g = gpu_run(prog, inputs, pi)
+    assert g.launch_count() == launches, (prog.name, g.launch_count())
+    compare(prog, oracle_run(prog, {k: v.numpy() for k, v in inputs.items()}), got, prog.name)
+print("done")
+"""
+
+
+def test_scans_on_a_device_without_cooperative_launches(tmp_path):
+    """What needs a grid of resident blocks falls back: long scans to tiles claimed from a ticket, one scan to a walk.  (In a
+    process of its own, in which the library is told that the device cannot.)"""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    (tmp_path / "no.cpp").write_text("namespace acc { bool cooperative_launch_ok() { return false; } }\n")
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(tmp_path / "no.so"), str(tmp_path / "no.cpp")], check=True)
+    child = subprocess.run([sys.executable, "-c", WITHOUT_COOPERATIVE_LAUNCHES, str(tmp_path / "no.so"), os.path.dirname(here), here],
+                           capture_output=True, text=True, timeout=600)
+    assert child.returncode == 0 and child.stdout.endswith("done\n"), child.stderr[-2000:]
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))
