@@ -224,7 +224,7 @@ struct Launcher {
               return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
             // (blocks read one another's totals: all of them resident)
             void* params[] = {&a, &per_row, &n_tiles, &whole};
-            cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tiles, sm_count())), dim3(K::THREADS), params, K::SMEM, L.stream);
+            cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tiles, std::min(sm_count(), dev::kRingMaxBlocks))), dim3(K::THREADS), params, K::SMEM, L.stream);
           }
         }
       }

@@ -237,6 +237,8 @@ template <class CL> constexpr bool ring_serves() {
   else return operands_fed_by_ring<CL>();
 }
 
+constexpr int kRingPerLane = 5;        // totals of a round that a lane of a look-back warp takes
+constexpr int kRingMaxBlocks = 32 * kRingPerLane;   // and so the most blocks a round may have
 constexpr int kRingDirectRounds = 8;   // rounds up to which every block adds the totals of a round up for itself
 constexpr int kRingPollPause = 50;     // ns between two looks at totals that were missing
 // Rows of up to kScanWarpRow elements get a warp each, up to kScanBlockRow a block each (a row may begin three words into its
@@ -599,18 +601,18 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
           here[o] = Run::bits(Run::identity());
         }
       });
-      // the totals of tiles base + step * u of scan o, u = 0..4, where these lie below `limit`: waits until they are posted
-      auto totals = [&](int o, int base, int step, int limit, uint64_t (&v)[5]) {
+      // the totals of tiles base + step * u of scan o, u = 0 .. kRingPerLane - 1, where these lie below `limit`: waits until they are posted
+      auto totals = [&](int o, int base, int step, int limit, uint64_t (&v)[kRingPerLane]) {
         const uint64_t* at = states + (size_t)o * n_tiles + base;
 #pragma unroll
-        for (int u = 0; u < 5; ++u) v[u] = base + step * u < limit ? 0u : 1u;
+        for (int u = 0; u < kRingPerLane; ++u) v[u] = base + step * u < limit ? 0u : 1u;
         for (uint32_t spins = 0;;) {
           bool missing = false;
 #pragma unroll
-          for (int u = 0; u < 5; ++u)                                   // (only what is still missing is asked for again)
+          for (int u = 0; u < kRingPerLane; ++u)                                   // (only what is still missing is asked for again)
             if ((v[u] & 1u) == 0u) v[u] = ld_posted(at + step * u);
 #pragma unroll
-          for (int u = 0; u < 5; ++u) missing = missing || (v[u] & 1u) == 0u;
+          for (int u = 0; u < kRingPerLane; ++u) missing = missing || (v[u] & 1u) == 0u;
           if (!__any_sync(0xFFFFFFFFu, missing)) return true;
           if (++spins > a.spin_limit) return false;
           __nanosleep(kRingPollPause);
@@ -631,12 +633,12 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
               constexpr int o = scan_ord<CL>(sc);
               using Run = Running<CL::c.nodes[sc].fn, CL::c.nodes[sc].dtype>;
               auto h = Run::identity(), x = Run::identity();
-              for (int base = max(first, row_first); base < limit; base += 32 * 5) {
-                uint64_t v[5];
+              for (int base = max(first, row_first); base < limit; base += 32 * kRingPerLane) {
+                uint64_t v[kRingPerLane];
                 in_time = in_time && totals(o, base + lane, 32, limit, v);
                 if (!in_time) break;
 #pragma unroll
-                for (int u = 0; u < 5; ++u) {
+                for (int u = 0; u < kRingPerLane; ++u) {
                   const int j = base + 32 * u + lane;
                   const auto t = j < limit ? Run::of((uint32_t)(v[u] >> 32)) : Run::identity();
                   if (j < tile) h = Run::add(h, t);
@@ -667,11 +669,11 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
           if (lane == 0 && more) mbar_arrive(&carried[after]);
         } else if (blockIdx.x == 0) {
           // the first block scans the totals of the round (a row's first tile starts anew) and posts what precedes each tile
-          const int limit = min(first + G, n_tiles), j0 = first + 5 * lane;
-          uint64_t excl[NS][5], lane_before[NS], lane_after[NS];
-          bool resets[5], any = false;                                     // a row begins at tile j0 + u; one begins in this lane's tiles
+          const int limit = min(first + G, n_tiles), j0 = first + kRingPerLane * lane;
+          uint64_t excl[NS][kRingPerLane], lane_before[NS], lane_after[NS];
+          bool resets[kRingPerLane], any = false;                                     // a row begins at tile j0 + u; one begins in this lane's tiles
 #pragma unroll
-          for (int u = 0; u < 5; ++u) {
+          for (int u = 0; u < kRingPerLane; ++u) {
             resets[u] = j0 + u < limit && (j0 + u) % tiles_per_row == 0;
             any = any || resets[u];
           }
@@ -683,11 +685,11 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
             if constexpr (is_scan_root(CL::c.nodes[sc])) {
               constexpr int o = scan_ord<CL>(sc);
               using Run = Running<CL::c.nodes[sc].fn, CL::c.nodes[sc].dtype>;
-              uint64_t v[5];
+              uint64_t v[kRingPerLane];
               in_time = in_time && totals(o, j0, 1, limit, v);
               auto run = Run::identity();
 #pragma unroll
-              for (int u = 0; u < 5; ++u) {
+              for (int u = 0; u < kRingPerLane; ++u) {
                 if (resets[u]) run = Run::identity();
                 excl[o][u] = Run::bits(run);
                 if (in_time && j0 + u < limit) run = Run::add(run, Run::of((uint32_t)(v[u] >> 32)));
@@ -714,7 +716,7 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
               if (run_from < 0) before = Run::add(sofar, before);
               bool fresh = false;
 #pragma unroll
-              for (int u = 0; u < 5; ++u) {
+              for (int u = 0; u < kRingPerLane; ++u) {
                 fresh = fresh || resets[u];
                 const auto p = fresh ? Run::from(excl[o][u]) : Run::add(before, Run::from(excl[o][u]));
                 if (u == 0) here[o] = Run::bits(p);                         // (lane 0: this block's tile)

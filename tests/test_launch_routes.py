@@ -1,0 +1,78 @@
+"""Which kernels a run launches, with how many blocks, and what the host side makes of their status words: the library over
+a CUDA runtime that launches nothing (fake_cuda.cpp), on the CPU."""
+import ctypes as C
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+CHILD = """
+import ctypes as C, json, sys
+fake = C.CDLL(sys.argv[1], mode=C.RTLD_GLOBAL)               # before the library, which then finds these definitions
+sys.path[:0] = sys.argv[2:4]
+import workloads as W
+from paper_2407_13585_b200 import binding as B, build
+B.load_kernel_library(build.TEST_LIB)
+fake.fake_launches.restype = C.c_char_p
+fake.fake_status.restype = C.POINTER(C.c_uint32)
+lib = B.lib()
+
+
+def bound(prog, pi=None, recompute=0):
+    g = B.Graph(prog.nodes, prog.outputs)
+    g.set_partition_recompute(pi or [-1 if nd.kind == "input" else 0 for nd in prog.nodes], recompute)
+    address = 1 << 40
+    for i, nd in enumerate(prog.nodes):
+        count = 1
+        for e in nd.shape:
+            count *= e
+        assert lib.acc_bind(g._h, i, C.c_void_p(address), C.c_size_t(4 * count)) == 0
+        address += (4 * count + 255) // 256 * 256
+    return g
+
+
+def run(g, workspace=1 << 50):
+    code = lib.acc_run(g._h, C.c_void_p(workspace), C.c_size_t(1 << 44), None, B.FUSED)
+    assert code == 0, (code, lib.acc_last_error())
+
+
+def launches(prog, pi=None, recompute=0):
+    fake.fake_clear()
+    g = bound(prog, pi, recompute)
+    run(g)
+    out = []
+    for line in fake.fake_launches().decode().splitlines():
+        name, grid, block, how = line.split("|")
+        out.append([name.split("<")[0].split("::")[-1], "<" + name.split("<", 1)[1], int(grid), int(block), how == "C"])
+    return out
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    """Runs a script behind CHILD in a process of its own and returns what it leaves in `result`."""
+    fake = str(tmp_path_factory.mktemp("fake") / "fake_cuda.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-o", fake, os.path.join(HERE, "fake_cuda.cpp"), "-ldl"], check=True)
+
+    def run(script):
+        p = subprocess.run([sys.executable, "-c", CHILD + script + "\nprint('RESULT' + json.dumps(result))", fake, os.path.dirname(HERE), HERE],
+                           capture_output=True, text=True, timeout=300)
+        assert p.returncode == 0, p.stderr[-3000:]
+        return json.loads(p.stdout.rsplit("RESULT", 1)[1])
+    return run
+
+
+def test_the_ring_has_no_more_blocks_than_a_look_back_warp_adds_up(child):
+    """The first block's look-back warps cover 160 tiles a round: on a device with more SMs the grid stays at that."""
+    got = child("""
+result = []
+for sms in (100, 148, 160, 170):
+    fake.fake_device(sms, 1)
+    result.append(launches(W.row_scans(1, 1 << 24), [-1, 0, 1, 1]))
+""")
+    assert [[k[0] for k in run] for run in got] == [["k_scan_ring", "k_scan_ring"]] * 4
+    assert [{k[2] for k in run} for run in got] == [{100}, {148}, {160}, {160}]
