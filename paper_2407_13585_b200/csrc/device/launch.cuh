@@ -163,12 +163,32 @@ struct Launcher {
 
   // Scans through the shared-memory ring (k_scan_ring), or a warp or block per row where rows are short (k_scan_rows);
   // without them, where a chunk behind an index map would not be a 128-bit access, or where rows are long and the ring does
-  // not serve the scan's operand or the device cannot launch a grid with all blocks resident, k_scan.
+  // not serve the scan's operand or the device cannot launch a grid with all blocks resident, k_scan, which also takes what
+  // it is quicker at.
   static constexpr bool kRingShape = kHasScan && dev::scan_ring_eligible<CL>();
   static constexpr bool kRingServes = kHasScan && dev::ring_serves<CL>();
-  static bool use_ring(const ClusterLaunch& L, int C) {
+  static bool use_ring(const ClusterLaunch& L, int R, int C) {
     if constexpr (!kRingShape) return false;
-    else return (!dev::has_index_map<CL>() || vec_ok(L, C)) && (C <= dev::kScanBlockRow || (kRingServes && cooperative_launch_ok()));
+    else return (!dev::has_index_map<CL>() || vec_ok(L, C)) && (C <= dev::kScanBlockRow || (kRingServes && cooperative_launch_ok())) && !look_back_is_quicker(L, R, C);
+  }
+  // One scan of a size at which the ring has not got going: its tiles wait for a round's totals to be exchanged, k_scan's for
+  // their neighbours only, and most of them are there at once.  us for two scans of rows, ring against k_scan with resident
+  // blocks: 64 x 17000 23.6 / 14.4, 148 x 17000 27.1 / 18.6, 148 x 33000 36.1 / 33.3, 8 x 200000 24.7 / 18.4; 300 x 17000 equal
+  // (600 tiles), 1000 x 17000 84 / 88.  One row: 300000 15.4 / 14.5, 500000 17.7 / 15.3, 2^20 23.1 / 17.6, 2^21 25.3 / 23.1,
+  // 3 * 10^6 27.1 / 27.4 (184 tiles).  Element by element (rows without 128-bit accesses), where the ring takes more than a round:
+  // 32 x 30001 23.9 / 18.6, 3 x 500001 24.0 / 22.2, 900001 23.0 / 21.0; 757761 (149 tiles of the ring) 19.5 / 20.5, 2^21 + 1 25.3 / 26.2,
+  // 148 x 33001 36.5 / 47.1.  A staged gather below the scan: one row of few elements (30000: ticketed tiles 8.7, ring 12.4).
+  static bool look_back_is_quicker(const ClusterLaunch& L, int R, int C) {
+    if constexpr (!kRingShape || dev::count_if<CL>(dev::is_scan_root) != 1) {
+      return false;                                      // (k_scan takes one scan; several share the ring's walk)
+    } else {
+      const int64_t per_row = (C + kScanTile - 1) / kScanTile, tiles = R * per_row;
+      if (C <= dev::kScanBlockRow) return false;
+      if constexpr (dev::costly_members<CL>() > 0) return R == 1 && C <= dev::kScanFewElements;
+      if constexpr (dev::scan_gathers<CL>()) return false;   // (with what reads the scan: smaller tiles, not measured)
+      if (vec_ok(L, C)) return tiles <= 3 * sm_count() && per_row <= 160;
+      return tiles <= sm_count() && per_row <= 64 && 8 * (int64_t)R * ring_tiles_per_row(R, C) > 9 * sm_count();
+    }
   }
   // (a row of C elements may begin up to three words into its first 16-byte chunk)
   static int ring_tiles_per_row(int R, int C) {
@@ -176,7 +196,7 @@ struct Launcher {
     else return 0;
   }
   static int64_t scan_scratch_bytes(const ClusterLaunch& L, int R, int C) {
-    if (use_ring(L, C)) {
+    if (use_ring(L, R, C)) {
       int per_row = ring_tiles_per_row(R, C);
       if constexpr (kRingShape) {
         if constexpr (dev::can_stage<CL>()) per_row = std::max(per_row, Launcher<dev::StagedScan<CL>>::ring_tiles_per_row(R, C));
@@ -236,12 +256,25 @@ struct Launcher {
     }
   }
 
-  // k_scan: tiles that look back one after the other, claimed from a ticket.
-  static int launch_look_back(const ClusterLaunch& L, const dev::Args<N>& a, bool vec, int tiles_per_row, int64_t tiles) {
+  // k_scan: tiles that look back one after the other, claimed from a ticket, or walked by blocks that are all resident.
+  static int launch_look_back(const ClusterLaunch& L, dev::Args<N>& a, bool vec, int tiles_per_row, int64_t tiles, bool resident = false) {
     if constexpr (dev::count_if<CL>(dev::is_scan_root) == 1) {
+      if (resident) {
+        const void* kern = vec ? reinterpret_cast<const void*>(dev::k_scan<CL, true>) : reinterpret_cast<const void*>(dev::k_scan<CL, false>);
+        static int fit_on[2][64];
+        const int at_once = resident_grid(kern, kScanBlock, fit_on[vec ? 1 : 0]);
+        if (at_once > 0) {
+          int n_tiles = (int)tiles, yes = 1;
+          void* params[] = {&a, &tiles_per_row, &n_tiles, &yes};
+          cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tiles, at_once)), dim3(kScanBlock), params, 0, L.stream);
+          const cudaError_t e = cudaGetLastError();
+          if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+          return ACC_OK;
+        }
+      }
       const int grid = (int)std::min<int64_t>(tiles, (int64_t)sm_count() * (1536 / kScanBlock));
-      if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles);
-      else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles);
+      if (vec) dev::k_scan<CL, true><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles, 0);
+      else dev::k_scan<CL, false><<<grid, kScanBlock, 0, L.stream>>>(a, tiles_per_row, (int)tiles, 0);
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
       return ACC_OK;
@@ -318,7 +351,7 @@ struct Launcher {
     if (!domain(L, R, C)) return 0;
     if (use_tiles(L, R, C)) return dev::tile_partials_off((R + dev::kTile - 1) / dev::kTile) * 4;
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
-    if (kHasScan && use_ring(L, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
+    if (kHasScan && use_ring(L, R, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
     if (stream_slab_shapes_ok(L, R, C)) return (((int64_t)dev::stream_acc64_off(kScalarFolds, sm_count() * 8) * 4) + 15) & ~int64_t(15);
     dev::HistPlan plan;
     if (use_hist(L, R, C, plan)) return scratch_bytes(L) - (int64_t)sm_count() * plan.exchange * 4;   // (what is exchanged is written first)
@@ -564,16 +597,9 @@ struct Launcher {
           return ACC_OK;
         }
       }
-      if constexpr (kRingShape) {
-        if constexpr (dev::can_stage<CL>() && dev::count_if<CL>(dev::is_scan_root) == 1) {
-          // a gather below the scan and few elements: tiles that look back one after the other, in an ordinary launch, are
-          // quicker than staging in a cooperative one (30000 elements 8.7 against 12.4 us).  Several scans share the ring's
-          // walk at any size: k_scan takes one.
-          if (R == 1 && C > dev::kScanBlockRow && C <= dev::kScanFewElements && use_ring(L, C)) return launch_look_back(L, a, vec, per_row, tiles);
-        }
-      }
-      if (use_ring(L, C)) return launch_ring(L, a, R, C);
-      return launch_look_back(L, a, vec, per_row, tiles);
+      if (use_ring(L, R, C)) return launch_ring(L, a, R, C);
+      // (a gather's latency covers the ticket's: sums over two gathers of 2^24 elements 222 us with tickets, 330 without)
+      return launch_look_back(L, a, vec, per_row, tiles, !dev::scan_gathers<CL>() && tiles <= 3 * sm_count());
     } else if constexpr (kHasRowFold) {
       if (R == 0) return ACC_OK;
       const int grid = std::min(R, sm_count() * 16);

@@ -511,6 +511,17 @@ struct SlabIn {
 __device__ __forceinline__ bool slab_passes_stand_back(const SlabIn& slab) { return 2u * __ldg(slab.local) > slab.sampled; }
 constexpr int kSlabWarpTile = 512;
 
+// Whether `leaf` (an array from outside the cluster) is read by member i at i's own index: through array operands
+// of maps and zipWiths only.
+constexpr bool reads_in_place(const CCluster& c, int i, int leaf) {
+  if (i == leaf) return true;
+  const CNode& n = c.nodes[i];
+  if (!n.member || (n.kind != ACC_MAP && n.kind != ACC_ZIPWITH)) return false;
+  for (int k = 0; k < n.narr; ++k)
+    if (reads_in_place(c, n.in[k], leaf)) return true;
+  return false;
+}
+
 // The gathered values of warp tile `wt` (kSlabWarpTile elements, grouped by slab where `staged` holds them) in element
 // order: lane's elements (j * 32 + lane) * 4 .. + 3 in gathered[j].  The stable counting sort of k_slab_partition is undone
 // from the slab codes and the group sizes, through `stage` (kSlabWarpTile words of shared memory that the warp owns).
@@ -748,6 +759,25 @@ struct ScanTile {
     }
   }
 
+  // The lines that the warp's part from walk position warp_base of `row` on will read in place, asked into L2
+  // (left-to-right scans; arrays from outside the cluster that the scanned operand reads at its own index).
+  static __device__ __forceinline__ void prefetch_operands(const Args<N>& a, int row, int warp_base) {
+    if constexpr (!REV) {
+      const int lane = threadIdx.x & 31;
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        if constexpr (!CL::c.nodes[i].member && reads_in_place(CL::c, sn.in[0], i)) {
+          const char* base = reinterpret_cast<const char*>(a.n[i].ptr) + (size_t)row * a.C * 4;
+#pragma unroll
+          for (int k = 0; k < PART; k += 1024) {
+            const int at = warp_base + k + lane * 32;
+            if (at < a.C) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)at * 4));
+          }
+        }
+      });
+    }
+  }
+
   // SLAB: the staged values and codes of warp tile `wt` are asked into L2 ahead of their use
   static __device__ __forceinline__ void prefetch_part(const Args<N>& a, int wt, const SlabIn& slab) {
     const int lane = threadIdx.x & 31;
@@ -761,8 +791,11 @@ struct ScanTile {
 
 // Tile after tile with the whole block in step: every warp scans its part, one warp looks back, every warp stores.
 // Tiles are claimed from a ticket: a tile's predecessors have been claimed by blocks that are running or done.
+// `resident`: all blocks of the grid are resident at once (a cooperative launch) and block b walks tiles b, b + G, b + 2G, ...
+// without a ticket, whose atomic a tile would begin with; a tile's predecessors then belong to the blocks before this one in
+// the same round, or to an earlier round, so they are running or done as well.
 template <class CL, bool VEC, bool SLAB>
-__device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per_row, int n_tiles, const SlabIn& slab) {
+__device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per_row, int n_tiles, const SlabIn& slab, bool resident) {
   using T = ScanTile<CL, VEC, SLAB>;
   constexpr int BLOCK = T::BLOCK, FN = T::FN, DT = T::DT;
   __shared__ uint32_t warp_total[BLOCK / 32];
@@ -771,14 +804,27 @@ __device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per
   __shared__ __align__(16) uint32_t slab_stage[SLAB ? BLOCK / 32 : 1][SLAB ? kSlabWarpTile : 1];   // read and written 128 bits at a time
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) tile_id = (int)atomicAdd(a.scratch, 1u);
-    __syncthreads();
-    const int tile = tile_id;
-    if (tile >= n_tiles) return;
+  for (int64_t walked = blockIdx.x;; walked += gridDim.x) {
+    // (resident: no barrier here.  What a tile shares through shared memory is read before its second barrier or right after
+    // it, and written again only behind the next tile's first barrier)
+    if (!resident) {
+      __syncthreads();
+      if (threadIdx.x == 0) tile_id = (int)atomicAdd(a.scratch, 1u);
+      __syncthreads();
+    }
+    const int64_t tile_of_mine = resident ? walked : tile_id;
+    if (tile_of_mine >= n_tiles) return;
+    const int tile = (int)tile_of_mine;
     const int row = tile / tiles_per_row, in_row = tile - row * tiles_per_row;
     const int warp_base = in_row * T::TILE + warp * T::PART;
+
+    if constexpr (!SLAB) {
+      // the block's next tile is known: what it reads is on its way while this tile is scanned and looked back for
+      if (resident && walked + gridDim.x < n_tiles) {
+        const int next = tile + (int)gridDim.x, next_row = next / tiles_per_row;
+        T::prefetch_operands(a, next_row, (next - next_row * tiles_per_row) * T::TILE + warp * T::PART);
+      }
+    }
 
     uint32_t val[T::ROWS][T::W];
     const uint32_t carry = T::scan_part(a, row, warp_base, tile * (BLOCK / 32) + warp, slab, slab_stage[SLAB ? warp : 0], val);
@@ -890,8 +936,8 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
 }
 
 template <class CL, bool VEC>
-__global__ void __launch_bounds__(scan_block<CL>()) k_scan(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles) {
-  scan_tiles<CL, VEC, false>(a, tiles_per_row, n_tiles, SlabIn{});
+__global__ void __launch_bounds__(scan_block<CL>()) k_scan(const __grid_constant__ Args<CL::c.n> a, int tiles_per_row, int n_tiles, int resident) {
+  scan_tiles<CL, VEC, false>(a, tiles_per_row, n_tiles, SlabIn{}, resident != 0);
 }
 
 }  // namespace dev

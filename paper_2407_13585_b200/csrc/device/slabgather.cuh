@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(scan_block<CL>(), 5) k_scan_merge(const __grid
                                                                   const SlabIn slab_in) {
   SlabIn slab = slab_in;
   if (slab_passes_stand_back(slab)) slab.full_tiles = 0;     // every warp tile gathers for itself
-  scan_tiles<CL, true, true>(a, tiles_per_row, n_tiles, slab);
+  scan_tiles<CL, true, true>(a, tiles_per_row, n_tiles, slab, false);
 }
 
 // Every root of a scan-less cluster stored from the gathered values of the earlier launches: a warp puts a warp tile

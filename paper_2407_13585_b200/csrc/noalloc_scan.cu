@@ -106,8 +106,8 @@ extern "C" int acc_scanl_add_i32_static(const int32_t* in, int32_t* out, int64_t
   const bool vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
   const int resident = sm_count() * (1536 / kScanBlock);
   const int grid = tiles < resident ? tiles : resident;
-  if (vec) dev::k_scan<ScanCluster, true><<<grid, kScanBlock, 0, stream>>>(a, tiles, tiles);
-  else dev::k_scan<ScanCluster, false><<<grid, kScanBlock, 0, stream>>>(a, tiles, tiles);
+  if (vec) dev::k_scan<ScanCluster, true><<<grid, kScanBlock, 0, stream>>>(a, tiles, tiles, 0);
+  else dev::k_scan<ScanCluster, false><<<grid, kScanBlock, 0, stream>>>(a, tiles, tiles, 0);
   e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
   uint32_t timed_out = 0;

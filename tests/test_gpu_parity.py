@@ -693,6 +693,19 @@ def test_scan_over_two_gathers_costs_no_more_than_its_nodes():
     assert milliseconds(B.FUSED) <= 1.5 * milliseconds(B.UNFUSED)
 
 
+# one scan to a walk by tiles that look back, all their blocks resident: one tile to a row and several, two rounds of tiles
+# (148 rows of three), 128-bit accesses and single ones, both directions, exclusive
+@pytest.mark.parametrize("rows,cols", [(64, 17000), (32, 30001), (3, 500001), (148, 33000), (1, 300000)])
+def test_scans_by_resident_tiles(rows, cols):
+    check_program(W.row_scans(rows, cols), [[-1, 0, 1, 1]])
+
+
+@pytest.mark.parametrize("n", [300000, 1 << 20])
+def test_seeded_and_reversed_scans_by_resident_tiles(n):
+    check_program(W.exclusive_scans(n))
+    check_program(W.suffix_sums(n))
+
+
 WITHOUT_COOPERATIVE_LAUNCHES = """
 import ctypes, sys
 ctypes.CDLL(sys.argv[1], mode=ctypes.RTLD_GLOBAL)          # its definition is found before the library's own

@@ -76,3 +76,24 @@ for sms in (100, 148, 160, 170):
 """)
     assert [[k[0] for k in run] for run in got] == [["k_scan_ring", "k_scan_ring"]] * 4
     assert [{k[2] for k in run} for run in got] == [{100}, {148}, {160}, {160}]
+
+
+def test_which_kernel_scans(child):
+    """Rows of one scan: blocks per row, the ring, and between them k_scan where it is quicker (see look_back_is_quicker)."""
+    got = child("""
+def kinds(prog, pi):
+    return [k[0] + ("" if k[0] != "k_scan" else " resident" if k[4] else " ticket") for k in launches(prog, pi)]
+result = {}
+for rows, cols in json.loads('[[1,16381],[1,20000],[1,20001],[64,17000],[148,33000],[300,17000],[32,30001],[3,500001],[148,33001],[1,900001],'
+                             '[1,300000],[1,2097152],[1,3000000]]'):
+    result["%d x %d" % (rows, cols)] = kinds(W.row_scans(rows, cols), [-1, 0, 1, 1])
+for n in (16381, 16382, 131072, 131073):
+    result["gather %d" % n] = kinds(W.config3(n), [-1, -1, 0, 0, 0, 0])
+    result["two gathers %d" % n] = kinds(W.sum_of_two_gathers(n), None)
+""")
+    ring, back, rows = ["k_scan_ring"] * 2, ["k_scan resident"] * 2, ["k_scan_rows"] * 2
+    want = {"1 x 16381": rows, "1 x 20000": back, "1 x 20001": ring, "64 x 17000": back, "148 x 33000": back, "300 x 17000": ring,
+            "32 x 30001": back, "3 x 500001": back, "148 x 33001": ring, "1 x 900001": back, "1 x 300000": back, "1 x 2097152": back, "1 x 3000000": ring}
+    assert {k: v for k, v in got.items() if "gather" not in k} == want
+    assert [got["gather %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"], ["k_scan ticket"], ["k_scan ticket"], ["k_scan_ring"]]
+    assert [got["two gathers %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"]] + [["k_scan ticket"]] * 3
