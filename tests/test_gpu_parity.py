@@ -603,7 +603,7 @@ def test_row_scans_both_directions(rows, cols):
 # tiles of the shared-memory ring: the largest row a block takes by itself and the smallest that goes through the ring; rows
 # that begin anywhere in a 16-byte chunk and cross tiles; a few rounds of the grid (every block adds up the totals) and many
 # (the first block does); the array's last words beyond its last whole chunk
-@pytest.mark.parametrize("rows,cols", [(3, 4093), (3, 4094), (2, 16381), (2, 16382), (5, 20001), (41, 90001), (90, 90002), (1, 148 * 8 * 5120 + 5)])
+@pytest.mark.parametrize("rows,cols", [(3, 4093), (3, 4094), (2, 16381), (2, 16382), (7, 8189), (5, 8190), (5, 20001), (41, 90001), (90, 90002), (1, 148 * 8 * 5120 + 5)])
 def test_row_scans_through_the_ring(rows, cols):
     prog = W.row_scans(rows, cols)
     assert check_program(prog) == 3

@@ -97,3 +97,11 @@ for n in (16381, 16382, 131072, 131073):
     assert {k: v for k, v in got.items() if "gather" not in k} == want
     assert [got["gather %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"], ["k_scan ticket"], ["k_scan ticket"], ["k_scan_ring"]]
     assert [got["two gathers %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"]] + [["k_scan ticket"]] * 3
+
+
+def test_a_block_reads_a_row_with_as_many_chunks_as_it_has(child):
+    got = child("""
+result = [launches(W.row_scans(10, cols), [-1, 0, 1, 1])[0][:2] for cols in (1024, 1025, 4093, 4094, 8189, 8190, 16381)]
+""")
+    assert {g[0] for g in got} == {"k_scan_rows"}
+    assert [g[1].split(", ", 1)[1] for g in got] == ["1, 4>", "16, 2>", "16, 2>", "16, 4>", "16, 4>", "16, 8>", "16, 8>"]
