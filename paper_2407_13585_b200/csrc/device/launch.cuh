@@ -178,12 +178,14 @@ struct Launcher {
   // 3 * 10^6 27.1 / 27.4 (184 tiles).  Element by element (rows without 128-bit accesses), where the ring takes more than a round:
   // 32 x 30001 23.9 / 18.6, 3 x 500001 24.0 / 22.2, 900001 23.0 / 21.0; 757761 (149 tiles of the ring) 19.5 / 20.5, 2^21 + 1 25.3 / 26.2,
   // 148 x 33001 36.5 / 47.1.  A staged gather below the scan: one row of few elements (30000: ticketed tiles 8.7, ring 12.4).
+  // Few rows with a gather below the scan, which a block per row would leave to few SMs: one row of 6000 from 4 MB equal, of
+  // 8000 9.2 / 7.2, of 16000 13.3 / 7.2 (two such scans 26.6 / 14.4).
   static bool look_back_is_quicker(const ClusterLaunch& L, int R, int C) {
     if constexpr (!kRingShape || dev::count_if<CL>(dev::is_scan_root) != 1) {
       return false;                                      // (k_scan takes one scan; several share the ring's walk)
     } else {
       const int64_t per_row = (C + kScanTile - 1) / kScanTile, tiles = R * per_row;
-      if (C <= dev::kScanBlockRow) return false;
+      if (C <= dev::kScanBlockRow) return dev::costly_members<CL>() > 0 && dev::scan_gathers<CL>() && C > dev::kScanGatherRow && tiles <= sm_count();
       if constexpr (dev::costly_members<CL>() > 0) return R == 1 && C <= dev::kScanFewElements;
       if constexpr (dev::scan_gathers<CL>()) return false;   // (with what reads the scan: smaller tiles, not measured)
       if (vec_ok(L, C)) return tiles <= 3 * sm_count() && per_row <= 160;
@@ -602,7 +604,7 @@ struct Launcher {
       }
       if (use_ring(L, R, C)) return launch_ring(L, a, R, C);
       // (a gather's latency covers the ticket's: sums over two gathers of 2^24 elements 222 us with tickets, 330 without)
-      return launch_look_back(L, a, vec, per_row, tiles, !dev::scan_gathers<CL>() && tiles <= 3 * sm_count());
+      return launch_look_back(L, a, vec, per_row, tiles, dev::scan_gathers<CL>() ? C <= dev::kScanBlockRow && tiles <= sm_count() : tiles <= 3 * sm_count());
     } else if constexpr (kHasRowFold) {
       if (R == 0) return ACC_OK;
       const int grid = std::min(R, sm_count() * 16);

@@ -244,6 +244,7 @@ constexpr int kRingPollPause = 50;     // ns between two looks at totals that we
 // Rows of up to kScanWarpRow elements get a warp each, up to kScanBlockRow a block each (a row may begin three words into its
 // first 16-byte chunk).
 constexpr int kScanWarpRow = 1024, kScanBlockRow = 16384 - 3;
+constexpr int kScanGatherRow = 6144;        // ... but few rows with a gather below the scan up to so many elements only
 constexpr int kScanFewElements = 1 << 17;   // a gather below a scan of up to so many elements is not staged
 
 // ---- shape of the kernel --------------------------------------------------------------------------------

@@ -618,8 +618,8 @@ def test_scans_that_share_a_walk(n):
     assert g.launch_count() == 2
 
 
-# a gather below a scan: in one row of a block, behind tickets, and staged by the blocks of the ring
-@pytest.mark.parametrize("n", [16383, 131072, 131073, 700001])
+# a gather below a scan: in one row of a block, in tiles of several, behind tickets, and staged by the blocks of the ring
+@pytest.mark.parametrize("n", [6144, 6145, 16380, 16381, 16383, 131072, 131073, 700001])
 def test_gather_staged_for_a_scan(n):
     prog = W.config3(n)
     prog.name = "fixture"                     # generic index inputs bounded by n

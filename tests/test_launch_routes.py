@@ -87,7 +87,7 @@ result = {}
 for rows, cols in json.loads('[[1,16381],[1,20000],[1,20001],[64,17000],[148,33000],[300,17000],[32,30001],[3,500001],[148,33001],[1,900001],'
                              '[1,300000],[1,2097152],[1,3000000]]'):
     result["%d x %d" % (rows, cols)] = kinds(W.row_scans(rows, cols), [-1, 0, 1, 1])
-for n in (16381, 16382, 131072, 131073):
+for n in (6144, 6145, 16381, 16382, 131072, 131073):
     result["gather %d" % n] = kinds(W.config3(n), [-1, -1, 0, 0, 0, 0])
     result["two gathers %d" % n] = kinds(W.sum_of_two_gathers(n), None)
 """)
@@ -95,8 +95,9 @@ for n in (16381, 16382, 131072, 131073):
     want = {"1 x 16381": rows, "1 x 20000": back, "1 x 20001": ring, "64 x 17000": back, "148 x 33000": back, "300 x 17000": ring,
             "32 x 30001": back, "3 x 500001": back, "148 x 33001": ring, "1 x 900001": back, "1 x 300000": back, "1 x 2097152": back, "1 x 3000000": ring}
     assert {k: v for k, v in got.items() if "gather" not in k} == want
-    assert [got["gather %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"], ["k_scan ticket"], ["k_scan ticket"], ["k_scan_ring"]]
-    assert [got["two gathers %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan_rows"]] + [["k_scan ticket"]] * 3
+    assert [got["gather %d" % n][0] for n in (6144, 6145, 16381)] == ["k_scan_rows", "k_scan resident", "k_scan resident"]
+    assert [got["gather %d" % n][0] for n in (16382, 131072, 131073)] == ["k_scan ticket", "k_scan ticket", "k_scan_ring"]
+    assert [got["two gathers %d" % n] for n in (16381, 16382, 131072, 131073)] == [["k_scan resident"]] + [["k_scan ticket"]] * 3
 
 
 def test_a_block_reads_a_row_with_as_many_chunks_as_it_has(child):
