@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <deque>
 #include <map>
 #include <mutex>
 
@@ -223,27 +224,31 @@ static void* buffer_of(const Graph& g, const Schedule& sch, char* ws, int node) 
 
 // Status words of the runs (see raise_status in device/eval.cuh): pinned host memory that the kernels write to, a cache
 // line for every workspace that a handle runs over (runs over different workspaces may be in flight together), in pages
-// that stay with the process; a destroyed handle's lines go to the next one.  Run numbers are unique in the process, so
-// a kernel that outlives its handle cannot speak for another run.  A run that is being captured into a CUDA graph will
+// that stay with the process; a destroyed handle's lines go to other handles, those of runs that nobody has waited for last.
+// Run numbers are unique in the process, so a kernel that outlives its handle cannot speak for another run.  A run that is being captured into a CUDA graph will
 // be replayed under one number: its line is cleared in the stream, like the control region, and is not handed on.
 // With the words in device memory a run paid for clearing them (3 us to enqueue) and a waited-for one for a copy back
 // (7 us to enqueue, 8 us of waiting): a chain of 2^16, waited for, 29.6 -> 16.6 us with the rest of the host path.
 namespace {
 std::mutex status_guard;
-std::vector<uint32_t*> free_status_words;
+std::deque<uint32_t*> free_status_words;
 std::atomic<uint32_t> last_run{0};
 constexpr int kStatusLines = 512;                          // lines of one page of status words
-constexpr size_t kMaxReports = 64;                         // lines of one handle; beyond that the one used longest ago is taken over
+constexpr size_t kManyReports = 64;                        // lines of one handle beyond which it looks for one it can use again
 
+// (the one used last is looked at first)
 RunReport* report_for(Graph& handle, const void* workspace) {
   for (RunReport& r : handle.reports)
-    if (r.workspace == workspace) return &r;
+    if (r.workspace == workspace) {
+      std::swap(r, handle.reports.front());
+      return &handle.reports.front();
+    }
   return nullptr;
 }
 
 uint32_t* take_status_words() {
   std::lock_guard<std::mutex> lock(status_guard);
-  if (free_status_words.empty()) {
+  if (free_status_words.size() <= kStatusLines / 2) {      // (so many others are handed on before a line put last)
     void* page = nullptr;
     // (allocating is not allowed while a stream is being captured, unless the thread says that it does not matter)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -256,19 +261,19 @@ uint32_t* take_status_words() {
       return nullptr;
     }
     memset(page, 0, kStatusLines * 64);
-    for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_back(static_cast<uint32_t*>(page) + k * 16);
+    for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_front(static_cast<uint32_t*>(page) + k * 16);
   }
-  uint32_t* words = free_status_words.back();
-  free_status_words.pop_back();
+  uint32_t* words = free_status_words.front();
+  free_status_words.pop_front();
   return words;
 }
 
 // The report of a new run over `workspace`.
 int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunReport** out) {
   RunReport* r = report_for(handle, workspace);
-  if (!r && handle.reports.size() >= kMaxReports) {
+  if (!r && handle.reports.size() >= kManyReports) {       // the line of a run with nothing to report, waited for the longest ago
     for (RunReport& c : handle.reports)
-      if (!c.captured && (!r || (int32_t)(c.run_id - r->run_id) < 0)) r = &c;
+      if (!c.captured && c.settled && (!r || (int32_t)(c.run_id - r->run_id) < 0)) r = &c;
   }
   if (!r) {
     uint32_t* words = take_status_words();
@@ -278,6 +283,7 @@ int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunRepo
     r->words = words;
   }
   r->workspace = workspace;
+  r->settled = false;
   do r->run_id = ++last_run;
   while (r->run_id == 0);
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -292,8 +298,11 @@ int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunRepo
 
 void give_back_status_words(Graph& handle) {
   std::lock_guard<std::mutex> lock(status_guard);
-  for (const RunReport& r : handle.reports)
-    if (!r.captured) free_status_words.push_back(r.words);
+  for (const RunReport& r : handle.reports) {
+    if (r.captured) continue;
+    if (r.settled) free_status_words.push_front(r.words);
+    else free_status_words.push_back(r.words);
+  }
   handle.reports.clear();
 }
 
@@ -390,13 +399,14 @@ int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaS
 int finish(Graph& g, void* workspace, cudaStream_t stream) {
   const cudaError_t e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
-  const RunReport* r = workspace ? report_for(g, workspace) : nullptr;
+  RunReport* r = workspace ? report_for(g, workspace) : nullptr;
   if (!r) return ACC_OK;
   const volatile uint32_t* words = r->words;
   const auto raised = [&](int condition) { return r->captured ? words[condition] != 0 : words[condition] == r->run_id; };
   if (raised(dev::kStatusTimeout)) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
   if (raised(dev::kStatusIndex)) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
   if (raised(dev::kStatusEmptySegment)) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
+  r->settled = true;
   return ACC_OK;
 }
 

@@ -34,6 +34,7 @@ struct RunReport {
   const void* workspace = nullptr;
   uint32_t* words = nullptr;
   uint32_t run_id = 0;             // unique in the process, never 0
+  bool settled = false;            // the last run was waited for and had nothing to report
   bool captured = false;           // a run was enqueued on a capturing stream: the words are cleared in the stream, any non-zero word counts
 };
 

@@ -106,3 +106,59 @@ result = [launches(W.row_scans(10, cols), [-1, 0, 1, 1])[0][:2] for cols in (102
 """)
     assert {g[0] for g in got} == {"k_scan_rows"}
     assert [g[1].split(", ", 1)[1] for g in got] == ["1, 4>", "16, 2>", "16, 2>", "16, 4>", "16, 4>", "16, 8>", "16, 8>"]
+
+
+STATUS = """
+def finish(g, workspace):
+    return lib.acc_finish(g._h, C.c_void_p(workspace), None)
+
+
+def reports_to():                                            # the status words of the last launch, and its run's number
+    run_id = C.c_uint32()
+    return fake.fake_status(C.byref(run_id)), run_id.value
+
+prog = W.config1(4096)
+"""
+
+
+def test_no_run_in_flight_loses_its_report(child):
+    """Runs of one handle over more workspaces than it keeps lines for: each wait reports its own run, as often as it is asked."""
+    got = child(STATUS + """
+g = bound(prog)
+spaces = [(1 << 50) + (k << 32) for k in range(200)]
+lines = []
+for ws in spaces:
+    run(g, ws)
+    lines.append(reports_to())
+for words, run_id in (lines[0], lines[100], lines[199]):     # three kernels meet an empty segment
+    words[2] = run_id
+result = {"lines": len({C.addressof(w.contents) for w, _ in lines}), "codes": [finish(g, ws) for ws in spaces]}
+# further workspaces: lines of runs with nothing to report are used again, the others' are not
+for k in range(200, 1000):
+    run(g, (1 << 50) + (k << 32))
+    finish(g, (1 << 50) + (k << 32))
+result["again"] = [finish(g, ws) for ws in spaces]
+result["pages"] = fake.fake_pages()
+""")
+    bad = got["codes"][0]
+    want = [bad if k in (0, 100, 199) else 0 for k in range(200)]
+    assert bad < 0 and got["codes"] == want and got["again"] == want
+    assert got["lines"] == 200 and got["pages"] == 1
+
+
+def test_lines_of_runs_that_nobody_waited_for_are_handed_on_last(child):
+    got = child(STATUS + """
+def line_of(wait):
+    g = bound(prog)
+    run(g)
+    at = C.addressof(reports_to()[0].contents)
+    if wait:
+        finish(g, 1 << 50)
+    lib.acc_graph_destroy(g._h)
+    g._h = None
+    return at
+first = line_of(False)
+after = [line_of(True) for k in range(100)]
+result = {"again": first in after, "used": len(set(after)), "pages": fake.fake_pages()}
+""")
+    assert got == {"again": False, "used": 1, "pages": 1}
