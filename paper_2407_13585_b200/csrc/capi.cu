@@ -44,8 +44,6 @@ bool bad_node(const acc_graph* g, acc_node n) { return n < 0 || n >= (acc_node)g
 
 }  // namespace
 
-acc_graph::~acc_graph() { give_back_status_words(*this); }
-
 extern "C" {
 
 int acc_graph_create(acc_graph** out) {

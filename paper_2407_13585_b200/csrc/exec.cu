@@ -6,6 +6,7 @@
 #include <cstring>
 #include <deque>
 #include <map>
+#include <memory>
 #include <mutex>
 
 #include "cluster.h"
@@ -225,16 +226,44 @@ static void* buffer_of(const Graph& g, const Schedule& sch, char* ws, int node) 
 // Status words of the runs (see raise_status in device/eval.cuh): pinned host memory that the kernels write to, a cache
 // line for every workspace that a handle runs over (runs over different workspaces may be in flight together), in pages
 // that stay with the process; a destroyed handle's lines go to other handles, those of runs that nobody has waited for last.
-// Run numbers are unique in the process, so a kernel that outlives its handle cannot speak for another run.  A run that is being captured into a CUDA graph will
-// be replayed under one number: its line is cleared in the stream, like the control region, and is not handed on.
+// Run numbers are unique in the process, so a kernel that outlives its handle cannot speak for another run.  A run that is
+// being captured into a CUDA graph will be replayed under one number: its line is cleared in the stream, like the control
+// region, and stays with the graph (a user object of it) after the handle is gone.
 // With the words in device memory a run paid for clearing them (3 us to enqueue) and a waited-for one for a copy back
 // (7 us to enqueue, 8 us of waiting): a chain of 2^16, waited for, 29.6 -> 16.6 us with the rest of the host path.
 namespace {
-std::mutex status_guard;
-std::deque<uint32_t*> free_status_words;
-std::atomic<uint32_t> last_run{0};
 constexpr int kStatusLines = 512;                          // lines of one page of status words
+constexpr int kSettled = 15;                               // word of a line: its last run was waited for and had nothing to report
 constexpr size_t kManyReports = 64;                        // lines of one handle beyond which it looks for one it can use again
+std::atomic<uint32_t> last_run{0};
+struct StatusPool {
+  std::mutex guard;
+  std::deque<uint32_t*> free;
+};
+StatusPool& status_pool() {
+  static StatusPool* pool = new StatusPool();              // (never destroyed: a CUDA graph may outlive everything static)
+  return *pool;
+}
+
+void hand_back(uint32_t* words) {
+  StatusPool& pool = status_pool();
+  std::lock_guard<std::mutex> lock(pool.guard);
+  if (words[kSettled]) pool.free.push_front(words);
+  else pool.free.push_back(words);
+}
+
+// `words` stay in use as long as the graph that `stream` is being captured into, or an executable made of it (for good, if
+// the graph does not take them).
+void keep_with_captured_graph(const std::shared_ptr<uint32_t>& words, cudaStream_t stream) {
+  auto* held = new std::shared_ptr<uint32_t>(words);
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  cudaUserObject_t object = nullptr;
+  if (cudaStreamGetCaptureInfo(stream, &status, nullptr, &graph) != cudaSuccess || !graph ||
+      cudaUserObjectCreate(&object, held, [](void* p) { delete static_cast<std::shared_ptr<uint32_t>*>(p); }, 1, cudaUserObjectNoDestructorSync) != cudaSuccess ||
+      cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove) != cudaSuccess)
+    cudaGetLastError();
+}
 
 // (the one used last is looked at first)
 RunReport* report_for(Graph& handle, const void* workspace) {
@@ -246,9 +275,10 @@ RunReport* report_for(Graph& handle, const void* workspace) {
   return nullptr;
 }
 
-uint32_t* take_status_words() {
-  std::lock_guard<std::mutex> lock(status_guard);
-  if (free_status_words.size() <= kStatusLines / 2) {      // (so many others are handed on before a line put last)
+std::shared_ptr<uint32_t> take_status_words() {
+  StatusPool& pool = status_pool();
+  std::lock_guard<std::mutex> lock(pool.guard);
+  if (pool.free.size() <= kStatusLines / 2) {              // (so many others are handed on before a line put last)
     void* page = nullptr;
     // (allocating is not allowed while a stream is being captured, unless the thread says that it does not matter)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -260,12 +290,12 @@ uint32_t* take_status_words() {
       set_error(ACC_ERR_CUDA, "no pinned memory for the status words: %s", cudaGetErrorString(e));
       return nullptr;
     }
-    memset(page, 0, kStatusLines * 64);
-    for (int k = kStatusLines - 1; k >= 0; --k) free_status_words.push_front(static_cast<uint32_t*>(page) + k * 16);
+    for (int k = kStatusLines - 1; k >= 0; --k) pool.free.push_front(static_cast<uint32_t*>(page) + k * 16);
   }
-  uint32_t* words = free_status_words.front();
-  free_status_words.pop_front();
-  return words;
+  uint32_t* words = pool.free.front();
+  pool.free.pop_front();
+  memset(words, 0, 64);
+  return std::shared_ptr<uint32_t>(words, hand_back);
 }
 
 // The report of a new run over `workspace`.
@@ -273,38 +303,31 @@ int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunRepo
   RunReport* r = report_for(handle, workspace);
   if (!r && handle.reports.size() >= kManyReports) {       // the line of a run with nothing to report, waited for the longest ago
     for (RunReport& c : handle.reports)
-      if (!c.captured && c.settled && (!r || (int32_t)(c.run_id - r->run_id) < 0)) r = &c;
+      if (!c.captured && c.words.get()[kSettled] && (!r || (int32_t)(c.run_id - r->run_id) < 0)) r = &c;
   }
   if (!r) {
-    uint32_t* words = take_status_words();
+    std::shared_ptr<uint32_t> words = take_status_words();
     if (!words) return ACC_ERR_CUDA;
     handle.reports.emplace_back();
     r = &handle.reports.back();
     r->words = words;
   }
   r->workspace = workspace;
-  r->settled = false;
+  r->words.get()[kSettled] = 0;
   do r->run_id = ++last_run;
   while (r->run_id == 0);
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) cudaGetLastError();
-  r->captured = r->captured || capturing == cudaStreamCaptureStatusActive;
-  if (r->captured && cudaMemsetAsync(r->words, 0, dev::kStatusConditions * 4, stream) != cudaSuccess)
+  if (capturing == cudaStreamCaptureStatusActive) {
+    r->captured = true;
+    keep_with_captured_graph(r->words, stream);
+  }
+  if (r->captured && cudaMemsetAsync(r->words.get(), 0, dev::kStatusConditions * 4, stream) != cudaSuccess)
     return set_error(ACC_ERR_CUDA, "clearing the status words failed: %s", cudaGetErrorString(cudaGetLastError()));
   *out = r;
   return ACC_OK;
 }
 }  // namespace
-
-void give_back_status_words(Graph& handle) {
-  std::lock_guard<std::mutex> lock(status_guard);
-  for (const RunReport& r : handle.reports) {
-    if (r.captured) continue;
-    if (r.settled) free_status_words.push_front(r.words);
-    else free_status_words.push_back(r.words);
-  }
-  handle.reports.clear();
-}
 
 static bool mark(std::vector<cudaEvent_t>* marks, cudaStream_t stream) {
   if (!marks) return true;
@@ -354,7 +377,7 @@ int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t
   for (ClusterStep& st : sch.steps) {
     st.launch.stream = stream;
     st.launch.spin_limit = g.spin_limit;
-    st.launch.status = report->words;
+    st.launch.status = report->words.get();
     st.launch.run_id = report->run_id;
     st.launch.extra_launches = 0;
     const int rc = st.kernel->launch(st.launch);
@@ -401,12 +424,12 @@ int finish(Graph& g, void* workspace, cudaStream_t stream) {
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
   RunReport* r = workspace ? report_for(g, workspace) : nullptr;
   if (!r) return ACC_OK;
-  const volatile uint32_t* words = r->words;
+  volatile uint32_t* words = r->words.get();
   const auto raised = [&](int condition) { return r->captured ? words[condition] != 0 : words[condition] == r->run_id; };
   if (raised(dev::kStatusTimeout)) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
   if (raised(dev::kStatusIndex)) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
   if (raised(dev::kStatusEmptySegment)) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
-  r->settled = true;
+  words[kSettled] = 1;
   return ACC_OK;
 }
 

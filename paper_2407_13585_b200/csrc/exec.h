@@ -45,7 +45,6 @@ int refine_to_kernels(const Graph& g, std::vector<int32_t>& pi, int recompute_de
 // `marks`, if given, receives one recorded event before the first launch and one after each launch
 int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t ws_bytes, cudaStream_t stream,
                  std::vector<cudaEvent_t>* marks = nullptr);
-void give_back_status_words(Graph& handle);
 int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaStream_t stream);
 int finish(Graph& g, void* workspace, cudaStream_t stream);
 

@@ -29,12 +29,12 @@ struct Edge {
 };
 
 // Where the kernels of the runs over one workspace report to: a line of pinned host words, in which a word that holds
-// the number of the last such run says that its condition arose.
+// the number of the last such run says that its condition arose.  Shared with the CUDA graphs that runs were captured
+// into: the line is handed on when neither the handle nor such a graph is left.
 struct RunReport {
   const void* workspace = nullptr;
-  uint32_t* words = nullptr;
+  std::shared_ptr<uint32_t> words;
   uint32_t run_id = 0;             // unique in the process, never 0
-  bool settled = false;            // the last run was waited for and had nothing to report
   bool captured = false;           // a run was enqueued on a capturing stream: the words are cleared in the stream, any non-zero word counts
 };
 
@@ -95,6 +95,5 @@ struct ScheduleCache;   // exec.h
 }  // namespace acc
 
 struct acc_graph : acc::Graph {
-  ~acc_graph();
   std::shared_ptr<acc::ScheduleCache> cache[2];   // the schedule of either executor (kept with the handle: handles on several threads share nothing)
 };

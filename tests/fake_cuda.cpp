@@ -53,9 +53,16 @@ int sm_count() { return sms; }
 bool cooperative_launch_ok() { return cooperative != 0; }
 }  // namespace acc
 
+struct Held { void (*destroy)(void*); void* p; };
+static Held held_by_graph[4096];             // user objects of the graph that is being captured
+static int n_held = 0;
+
 extern "C" {
 void fake_device(int sm_count, int can_launch_cooperatively) { sms = sm_count; cooperative = can_launch_cooperatively; }
 void fake_capturing(int on) { capturing = on; }
+void fake_destroy_graph() {
+  while (n_held > 0) { --n_held; held_by_graph[n_held].destroy(held_by_graph[n_held].p); }
+}
 void fake_clear() { launches.clear(); }
 const char* fake_launches() { return launches.c_str(); }
 int fake_pages() { return n_pages; }
@@ -75,6 +82,21 @@ int cudaMemsetAsync(void* p, int v, size_t bytes, void*) {           // host mem
 int cudaMemcpyAsync(void*, const void*, size_t, int, void*) { return 0; }
 int cudaStreamSynchronize(void*) { return 0; }
 int cudaStreamIsCapturing(void*, int* status) { *status = capturing; return 0; }
+int cudaStreamGetCaptureInfo_v2(void*, int* status, unsigned long long*, void** graph, const void***, size_t*) {
+  *status = capturing;
+  *graph = capturing ? &held_by_graph : nullptr;
+  return 0;
+}
+int cudaUserObjectCreate(void** object, void* p, void (*destroy)(void*), unsigned, unsigned) {
+  *object = new Held{destroy, p};
+  return 0;
+}
+int cudaGraphRetainUserObject(void*, void* object, unsigned, unsigned) {
+  if (n_held == 4096) return 1;
+  held_by_graph[n_held++] = *static_cast<Held*>(object);
+  delete static_cast<Held*>(object);
+  return 0;
+}
 int cudaThreadExchangeStreamCaptureMode(int*) { return 0; }
 int cudaHostAlloc(void** p, size_t bytes, unsigned) {
   if (n_pages == 64) return 2;

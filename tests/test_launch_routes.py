@@ -162,3 +162,35 @@ after = [line_of(True) for k in range(100)]
 result = {"again": first in after, "used": len(set(after)), "pages": fake.fake_pages()}
 """)
     assert got == {"again": False, "used": 1, "pages": 1}
+
+
+def test_lines_of_captured_runs_come_back_when_handle_and_graph_are_gone(child):
+    """A captured run's line is the graph's too: it is no other handle's while the graph can be replayed, whether or not its
+    handle is left, and then goes to the next one."""
+    got = child(STATUS + """
+def used_after(k):
+    lines = set()
+    for _ in range(k):
+        g = bound(prog)
+        run(g)
+        lines.add(C.addressof(reports_to()[0].contents))
+        finish(g, 1 << 50)
+        lib.acc_graph_destroy(g._h)
+        g._h = None
+    return lines
+result = []
+for round in range(20):
+    fake.fake_capturing(1)
+    captured = set()
+    for _ in range(100):
+        g = bound(prog)
+        run(g)
+        captured.add(C.addressof(reports_to()[0].contents))
+        lib.acc_graph_destroy(g._h)
+        g._h = None
+    fake.fake_capturing(0)
+    result.append([len(captured), len(captured & used_after(5)), fake.fake_pages()])
+    fake.fake_destroy_graph()
+""")
+    assert [g[:2] for g in got] == [[100, 0]] * 20
+    assert max(g[2] for g in got) <= 2
