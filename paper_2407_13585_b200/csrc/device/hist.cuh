@@ -46,12 +46,20 @@ struct HistPlan {
   int shift;        // log2(per_cta) when it is a power of two and group > 1, else -1
   int overflow;     // bins per CTA kept in global memory (group == 1 only)
   int exchange;     // words per CTA of the scratch in which the CTAs exchange their bins; 0: they add them up with atomics
+  uint32_t polls;   // looks at the meeting counter (a tenth of a microsecond at the least) before a CTA gives the others up
 };
 constexpr int kHistExchangeBins = 20000;        // bins from which exchanging them is worth a meeting of all CTAs (1246656 keys: 10000 bins 25.7 against 22.5 us, 20000 bins the same, 60000 bins 33 against 46)
 
+// A CTA that has walked its share waits for the others', which may take longer: a value that the integer bins do not take is
+// an fp64 atomic on global memory, and where all such values meet in one bin a CTA's turn comes once in as many of these
+// (some nanoseconds each) as there are CTAs.  Eight polls for every element of a share cover that; a short walk gets the usual limit.
+inline uint32_t hist_polls(int64_t elements, int teams) {
+  return (uint32_t)std::min<int64_t>((int64_t)kCopySpinLimit + 8 * (elements / std::max(teams, 1)), 0xFFFFFFFFll);
+}
+
 // How the bins are laid out, or false when they do not fit eight CTAs.
 inline bool hist_plan(int64_t bins, int sms, HistPlan& p) {
-  p = HistPlan{1, 0, -1, 0, 0};
+  p = HistPlan{1, 0, -1, 0, 0, kCopySpinLimit};
   if (bins <= 0) return false;
   if (bins <= kHistMaxBinsPerCta + kHistOverflowBins) {
     p.per_cta = (int)std::min<int64_t>(bins, kHistMaxBinsPerCta);
@@ -387,7 +395,7 @@ k_hist(const __grid_constant__ Args<CL::c.n> a, const HistPlan plan, int* overfl
     if (plan.exchange) {                                       // all CTAs are resident: wait until each has written its bins
       uint32_t spins = 0;
       while (*reinterpret_cast<volatile uint32_t*>(a.scratch) < gridDim.x) {
-        if (++spins > kCopySpinLimit) { raise_status(a, kStatusTimeout); break; }
+        if (++spins > plan.polls) { raise_status(a, kStatusTimeout); break; }
         __nanosleep(100);
       }
     }

@@ -671,6 +671,7 @@ int Launcher<CL>::launch_hist(const ClusterLaunch& L, dev::Args<N>& a, int R, in
     const int64_t want = (chunks + per_team - 1) / per_team;
     const int teams = (int)std::max<int64_t>(1, std::min<int64_t>(want, sm_count() / plan.group));
     const int grid = teams * plan.group;                  // one CTA per SM: all of them are resident together
+    plan.polls = dev::hist_polls((int64_t)R * C, teams);
     int* overflow = reinterpret_cast<int*>(L.scratch + dev::stream_acc64_off(kScalarFolds, a.grid) + 2 * bins);
     int* exchange = reinterpret_cast<int*>(L.scratch + hist_exchange_off(dev::stream_acc64_off(kScalarFolds, a.grid) + 2 * bins, plan));
     if (plan.exchange && cooperative_launch_ok()) {

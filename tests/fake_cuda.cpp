@@ -19,6 +19,7 @@ static size_t page_bytes[64];
 static int n_pages = 0;
 static uint32_t* status_words = nullptr;     // of the last launch: where its arguments say that it reports, and as which run
 static uint32_t status_run = 0;
+static int32_t second[8];                    // of the last launch of k_hist: its second argument's first words
 
 static int note(const void* kernel, dim3 grid, dim3 block, void** args, bool coop) {
   Dl_info info;
@@ -33,6 +34,7 @@ static int note(const void* kernel, dim3 grid, dim3 block, void** args, bool coo
   char rest[64];
   snprintf(rest, sizeof rest, "|%u|%u|%s\n", grid.x, block.x, coop ? "C" : "");
   launches += name + rest;
+  if (name.find("k_hist<") != std::string::npos) memcpy(second, args[1], 6 * sizeof second[0]);
   // the first argument of a cluster's kernel holds a pointer to status words, the run's number behind it
   const char* a = static_cast<const char*>(args[0]);
   status_words = nullptr;
@@ -65,6 +67,7 @@ void fake_destroy_graph() {
 }
 void fake_clear() { launches.clear(); }
 const char* fake_launches() { return launches.c_str(); }
+const int32_t* fake_second_argument() { return second; }
 int fake_pages() { return n_pages; }
 uint32_t* fake_status(uint32_t* run) { *run = status_run; return status_words; }
 

@@ -194,3 +194,18 @@ for round in range(20):
 """)
     assert [g[:2] for g in got] == [[100, 0]] * 20
     assert max(g[2] for g in got) <= 2
+
+
+def test_a_histogram_waits_for_its_slowest_cta_as_long_as_a_walk_may_take(child):
+    """Eight polls per element of a CTA's share on top of the usual limit, whatever else the plan holds."""
+    got = child("""
+fake.fake_second_argument.restype = C.POINTER(C.c_int32)
+result = []
+for n in (1 << 18, 1 << 27, 1 << 30):
+    names = [k[0] for k in launches(W.config5(n, 1 << 15), [-1, -1, 0, 0, 0, 0, 1])]
+    plan = fake.fake_second_argument()
+    result.append([names[0], plan[4] > 0, plan[5]])
+""")
+    shares = [(1 << 18) // 32, (1 << 27) // 148, (1 << 30) // 148]
+    assert [g[:2] for g in got] == [["k_hist", True]] * 3
+    assert [g[2] for g in got] == [(1 << 20) + 8 * s for s in shares]
