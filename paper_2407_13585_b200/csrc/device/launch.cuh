@@ -428,9 +428,10 @@ struct Launcher {
   static int launch_tiles_tma(const ClusterLaunch& L, dev::Args<N>& a, int n, bool vec) {
     if constexpr (dev::tile_tma_eligible<CL>()) {
       if (!cooperative_launch_ok()) return 1;
-      // (word-by-word copies and the meeting at the end pay from here on: 1999^2 18.7 against 14.2 us, 2999^2 19.0 against 23.6,
-      // 6349^2 67 against 75)
-      if (!vec && n < 2560) return 1;
+      // (word-by-word copies and the meeting at the end pay from here on; us staged by threads against copied, one array and
+      // two: 2561 rows 18.7 / 20.5 and 23.3 / 28.7, 2701 20.0 / 22.5 and 27.3 / 28.7, 2749 20.1 / 18.4 and 28.5 / 22.6, 2851 22.4 / 20.5
+      // and 30.6 / 26.6, 4001 32.0 / 26.8 and 71.8 / 52.2)
+      if (!vec && n < 2720) return 1;
       dev::TileMaps maps;
       for (int i = 0; i < N; ++i)
         if (vec && dev::is_staged_external<CL>(i) &&

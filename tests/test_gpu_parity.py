@@ -58,7 +58,7 @@ def test_config5_bins_that_just_fit(n, bins):
 
 
 # tiles copied word by word: one, two and three columns in the last chunk of four, of a tile that is nearly empty or nearly full
-@pytest.mark.parametrize("rows", [2561, 2622, 2623])
+@pytest.mark.parametrize("rows", [2561, 2622, 2623, 2719, 2721, 2753, 2814, 2815])
 def test_config2_any_extent(rows):
     check_program(W.config2(rows), [[-1, 0, 0, 0]])
 

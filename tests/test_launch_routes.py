@@ -209,3 +209,10 @@ for n in (1 << 18, 1 << 27, 1 << 30):
     shares = [(1 << 18) // 32, (1 << 27) // 148, (1 << 30) // 148]
     assert [g[:2] for g in got] == [["k_hist", True]] * 3
     assert [g[2] for g in got] == [(1 << 20) + 8 * s for s in shares]
+
+
+def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
+    got = child("""
+result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
+""")
+    assert got == ["k_tile_pair", "k_tile_pair", "k_tile_pair_tma", "k_tile_pair_tma", "k_tile_pair_tma"]
