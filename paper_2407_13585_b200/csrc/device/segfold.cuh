@@ -194,6 +194,35 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
     });
     for (int base = (int)run_lo; base < hi0; base += STEP) {
       if (base + STEP <= lo0) continue;
+      if constexpr (VEC) {
+        // steps far inside a long segment, two at a time: twice the loads under way (2^24 elements in one segment 24.6 -> 20.6 us,
+        // 2^27 Zipf lengths 189 -> 178)
+        while (base + 2 * STEP <= hi0 && base >= lo0 && __shfl_sync(0xFFFFFFFFu, o[0], 0) >= base + 2 * STEP) {
+          uint32_t q[N][2 * ROWS];                                // a chunk of four each
+          static_for<0, N>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            constexpr CNode nd = CL::c.nodes[i];
+            if constexpr (is_segfold_root(nd)) {
+              V4 v[2 * ROWS];
+#pragma unroll
+              for (int j = 0; j < 2 * ROWS; ++j) v[j] = eval<CL, nd.in[0]>(a, Ix4{0, base + (j * 32 + lane) * 4});
+#pragma unroll
+              for (int j = 0; j < 2 * ROWS; ++j)
+                q[i][j] = combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(v[j].v[0], v[j].v[1]), combine<nd.fn, nd.dtype>(v[j].v[2], v[j].v[3]));
+            }
+          });
+          static_for<0, N>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            constexpr CNode nd = CL::c.nodes[i];
+            if constexpr (is_segfold_root(nd)) {
+#pragma unroll
+              for (int j = 0; j < 2 * ROWS; ++j) fold_step<nd.fn, nd.dtype>(acc[i], comp[i], q[i][j]);
+            }
+          });
+          base += 2 * STEP;
+        }
+        if (base >= hi0) break;
+      }
       uint32_t x[N][ROWS][4];
       static_for<0, N>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
@@ -404,21 +433,40 @@ __global__ void __launch_bounds__(kBlock) k_segfold_across(const __grid_constant
     constexpr int i = decltype(ic)::value;
     if constexpr (is_segfold_root(CL::c.nodes[i])) v[i] = tail[2 + fold_slot_of(i)];
   });
-  for (int base = b + 1; base < n_blocks; base += 32) {
-    const int b2 = base + lane;
-    const uint32_t* head = rec + (size_t)min(b2, n_blocks - 1) * 2 * REC;
-    const bool same = b2 < n_blocks && head[0] == key;
-    const unsigned others = ~__ballot_sync(0xFFFFFFFFu, same);
-    const int n = others ? __ffs(others) - 1 : 32;               // blocks of this round that continue the segment
-    static_for<0, N>([&](auto ic) {
-      constexpr int i = decltype(ic)::value;
-      constexpr CNode nd = CL::c.nodes[i];
-      if constexpr (is_segfold_root(nd)) {
-        const uint32_t x = lane < n ? head[2 + fold_slot_of(i)] : identity_of<nd.fn, nd.dtype>();
-        v[i] = combine<nd.fn, nd.dtype>(v[i], warp_reduce<nd.fn, nd.dtype>(x));
-      }
-    });
-    if (n < 32) break;
+  // G times 32 blocks from `base` on, all of whose records are asked for together; whether the segment goes on behind them
+  auto go_on = [&](auto groups_c, int base) {
+    constexpr int G = decltype(groups_c)::value;
+    bool same[G];
+    uint32_t x[N][G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int b2 = base + 32 * g + lane;
+      const uint32_t* head = rec + (size_t)min(b2, n_blocks - 1) * 2 * REC;
+      same[g] = b2 < n_blocks && head[0] == key;
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        if constexpr (is_segfold_root(CL::c.nodes[i])) x[i][g] = head[2 + fold_slot_of(i)];
+      });
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const unsigned others = ~__ballot_sync(0xFFFFFFFFu, same[g]);
+      const int n = others ? __ffs(others) - 1 : 32;             // blocks of these 32 that continue the segment
+      static_for<0, N>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        constexpr CNode nd = CL::c.nodes[i];
+        if constexpr (is_segfold_root(nd))
+          v[i] = combine<nd.fn, nd.dtype>(v[i], warp_reduce<nd.fn, nd.dtype>(lane < n ? x[i][g] : identity_of<nd.fn, nd.dtype>()));
+      });
+      if (n < 32) return false;
+    }
+    return base + 32 * G < n_blocks;
+  };
+  // (few segments cross more than 33 blocks; those that do may cross all of them: 2^27 elements in one segment, 4096 records,
+  // 156 -> 133 us)
+  if (b + 1 < n_blocks && go_on(std::integral_constant<int, 1>{}, b + 1)) {
+    int base = b + 33;
+    while (go_on(std::integral_constant<int, 8>{}, base)) base += 8 * 32;
   }
   if (lane == 0) {
     static_for<0, N>([&](auto ic) {

@@ -511,10 +511,11 @@ def test_segmented_fold_with_skewed_and_awkward_segments():
     compare(prog, ref, got, "skewed segments, equal addends")
 
 
-@pytest.mark.parametrize("n,segments", [(511, 3), (513, 100), (4095, 4095), (148 * 32 * 512 * 2 + 7, 5000), (148 * 32 * 512 * 3 - 1, 2000000)])
+@pytest.mark.parametrize("n,segments", [(511, 3), (513, 100), (4095, 4095), (148 * 32 * 512 * 2 + 7, 5000), (148 * 32 * 512 * 3 - 1, 2000000),
+                                        (1 << 22, 1), ((1 << 22) + 1029, 2), (148 * 32 * 512 * 4 + 3, 40)])
 def test_segmented_fold_by_warps(n, segments):
     """A warp's run is one step of 512 elements, or several; segments of one element, more than a step's worth of offsets at
-    a time, lengths whose last chunk of four is not whole."""
+    a time, lengths whose last chunk of four is not whole; segments of many steps, two at a time, and across hundreds of blocks."""
     assert check_program(W.segmented_sums(n, segments), [[-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2]]) == 2
 
 
