@@ -831,8 +831,8 @@ def test_diagonal_of_a_product(rows):
 
 
 def test_lookback_wait_that_runs_out_is_reported():
-    """The one device-side wait that polls plain memory (a scan tile looking back at its predecessors) is given
-    no patience at all: tiles that find a predecessor unfinished give up at once, the kernel ends normally, and
+    """A wait that polls plain memory (the ring's look-back warps, which want the totals of their round) is given
+    no patience at all: warps that find a total missing give up at once, the kernel ends normally, and
     the run reports ACC_ERR_DEVICE_TIMEOUT; with the default bound the same graph then gives the oracle's result."""
     import torch
     from oracle import interp
@@ -858,9 +858,9 @@ def test_lookback_wait_that_runs_out_is_reported():
 
 
 def test_lookback_wait_that_runs_out_where_a_warp_of_its_own_looks_back():
-    """The same wait in the scan that parks a tile's values and leaves the look-back to a ninth warp (scans with a
-    gather in their cluster): that warp gives up at once, still hands the other warps a prefix at their barrier, the
-    kernel ends normally and the run reports the time-out; with the default bound the graph gives the oracle's result."""
+    """The same wait in a ring whose blocks have staged a gather first: the look-back warps give up at once, still hand the
+    scanning warps something to go on with, the kernel ends normally and the run reports the time-out; with the default
+    bound the graph gives the oracle's result."""
     import torch
     from paper_2407_13585_b200 import binding as B
     prog = W.config3(1 << 22)
@@ -880,6 +880,36 @@ def test_lookback_wait_that_runs_out_where_a_warp_of_its_own_looks_back():
     g.run(B.FUSED)
     assert g.launch_count() == 1
     compare(prog, ref, {5: out.cpu().numpy().view(np.uint32)}, "config3 after a look-back that ran out")
+
+
+# every other form of the wait: tiles behind tickets, tiles of resident blocks, the ring with totals that the first block adds
+# up and posts (more than eight rounds), the merging scan behind slab passes (a warp of its own looks back)
+@pytest.mark.parametrize("form", ["tickets", "resident", "posted", "merge"])
+def test_each_look_back_that_runs_out_is_reported(form):
+    import torch
+    from paper_2407_13585_b200 import binding as B
+    prog, pi, launches = {"tickets": (W.sum_of_two_gathers(1 << 20), [-1, -1, -1, 0, 0, 0, 0], 1),
+                          "resident": (W.row_scans(1, 1 << 20), [-1, 0, 1, 1], 2),
+                          "posted": (W.row_scans(1, 1 << 23), [-1, 0, 1, 1], 2),
+                          "merge": (W.config3(1 << 25), [-1, -1, 0, 0, 0, 0], 7)}[form]
+    inputs = W.make_inputs(prog, device="cuda")
+    ref = oracle_run(prog, {k: v.cpu().numpy() for k, v in inputs.items()})
+    g = B.Graph(prog.nodes, prog.outputs)
+    g.set_partition(pi)
+    for i, t in inputs.items():
+        g.bind(i, t)
+    outs = {o: torch.zeros(prog.nodes[o].shape, dtype=torch.int32, device="cuda") for o in prog.outputs}
+    for o, t in outs.items():
+        g.bind(o, t)
+    g.set_spin_limit(0)
+    with pytest.raises(B.AccError) as e:
+        g.run(B.FUSED)
+    assert e.value.status == "ACC_ERR_DEVICE_TIMEOUT"
+    g.set_spin_limit(1 << 22)
+    g.run(B.FUSED)
+    assert g.launch_count() == launches
+    got = {o: t.cpu().numpy().view(np.float32 if prog.nodes[o].dtype == "f32" else np.uint32) for o, t in outs.items()}
+    compare(prog, ref, got, form)
 
 
 def test_runs_do_not_depend_on_what_the_workspace_held():

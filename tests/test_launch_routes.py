@@ -216,3 +216,12 @@ def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
 result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
 """)
     assert got == ["k_tile_pair", "k_tile_pair", "k_tile_pair_tma", "k_tile_pair_tma", "k_tile_pair_tma"]
+
+
+def test_the_forms_of_a_look_back_that_the_gpu_tests_let_run_out(child):
+    """The programs of test_each_look_back_that_runs_out_is_reported take the kernels that it names."""
+    got = child("""
+result = [[k[0], k[4]] for k in launches(W.sum_of_two_gathers(1 << 20)) + launches(W.row_scans(1, 1 << 20), [-1, 0, 1, 1]) +
+          launches(W.row_scans(1, 1 << 23), [-1, 0, 1, 1]) + launches(W.config3(1 << 25))[-1:]]
+""")
+    assert got == [["k_scan", False]] + [["k_scan", True]] * 2 + [["k_scan_ring", True]] * 2 + [["k_scan_merge_pipelined", True]]
