@@ -7,10 +7,11 @@
 //   k_rowfold  one block per row of a rank-2 domain; folds of the innermost extent end in a
 //              block reduction, no atomics.
 //   k_scan     single-pass scan with decoupled look-back; the scanned operand is evaluated in
-//              registers.  Tiles are claimed from an atomic ticket, so a tile's predecessors are
-//              always running or done.  Most scans take k_scan_ring or k_scan_rows (scanring.cuh)
-//              instead; this one is left for what those do not: short arrays below a gather, index
-//              maps, devices without cooperative launches.
+//              registers.  Tiles are claimed from an atomic ticket or walked by resident blocks, so
+//              a tile's predecessors are always running or done.  Long scans and short rows take
+//              k_scan_ring or k_scan_rows (scanring.cuh) instead; this one is for what those do not
+//              serve or are slower at: operands that the ring would read twice, single scans of some
+//              10^5 to 10^6 elements, devices without cooperative launches (see launch.cuh).
 //
 // Each is templated on the cluster description (what to evaluate) and on VEC (whether four
 // consecutive elements move as one 128-bit access).
