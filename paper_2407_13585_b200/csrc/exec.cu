@@ -298,8 +298,9 @@ std::shared_ptr<uint32_t> take_status_words() {
   return std::shared_ptr<uint32_t>(words, hand_back);
 }
 
-// The report of a new run over `workspace`.
-int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunReport** out) {
+// The report of a new run over `workspace`, as it is now.
+int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunReport& out) {
+  std::lock_guard<std::mutex> lock(handle.reports_guard);
   RunReport* r = report_for(handle, workspace);
   if (!r && handle.reports.size() >= kManyReports) {       // the line of a run with nothing to report, waited for the longest ago
     for (RunReport& c : handle.reports)
@@ -324,7 +325,7 @@ int begin_run(Graph& handle, const void* workspace, cudaStream_t stream, RunRepo
   }
   if (r->captured && cudaMemsetAsync(r->words.get(), 0, dev::kStatusConditions * 4, stream) != cudaSuccess)
     return set_error(ACC_ERR_CUDA, "clearing the status words failed: %s", cudaGetErrorString(cudaGetLastError()));
-  *out = r;
+  out = *r;
   return ACC_OK;
 }
 }  // namespace
@@ -365,8 +366,8 @@ int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t
     const int rc = resolve_pointers(g, sch, ws);
     if (rc != ACC_OK) return rc;
   }
-  RunReport* report = nullptr;
-  const int begun = begin_run(handle, workspace, stream, &report);
+  RunReport report;
+  const int begun = begin_run(handle, workspace, stream, report);
   if (begun != ACC_OK) return begun;
   for (const auto& piece : sch.to_clear)
     if (cudaMemsetAsync(ws + piece.first, 0, piece.second, stream) != cudaSuccess)
@@ -377,8 +378,8 @@ int run_schedule(Graph& handle, Graph& g, Schedule& sch, void* workspace, size_t
   for (ClusterStep& st : sch.steps) {
     st.launch.stream = stream;
     st.launch.spin_limit = g.spin_limit;
-    st.launch.status = report->words.get();
-    st.launch.run_id = report->run_id;
+    st.launch.status = report.words.get();
+    st.launch.run_id = report.run_id;
     st.launch.extra_launches = 0;
     const int rc = st.kernel->launch(st.launch);
     if (rc != ACC_OK) return rc;
@@ -420,16 +421,22 @@ int check_gather_indices(const Graph& g, void* workspace, size_t ws_bytes, cudaS
 }
 
 int finish(Graph& g, void* workspace, cudaStream_t stream) {
+  RunReport r;                                             // the run to wait for; another thread may begin others meanwhile
+  {
+    std::lock_guard<std::mutex> lock(g.reports_guard);
+    if (const RunReport* known = workspace ? report_for(g, workspace) : nullptr) r = *known;
+  }
   const cudaError_t e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "stream failed: %s", cudaGetErrorString(e));
-  RunReport* r = workspace ? report_for(g, workspace) : nullptr;
-  if (!r) return ACC_OK;
-  volatile uint32_t* words = r->words.get();
-  const auto raised = [&](int condition) { return r->captured ? words[condition] != 0 : words[condition] == r->run_id; };
+  if (!r.words) return ACC_OK;
+  const volatile uint32_t* words = r.words.get();
+  const auto raised = [&](int condition) { return r.captured ? words[condition] != 0 : words[condition] == r.run_id; };
   if (raised(dev::kStatusTimeout)) return set_error(ACC_ERR_DEVICE_TIMEOUT, "a device-side wait ran out of iterations");
   if (raised(dev::kStatusIndex)) return set_error(ACC_ERR_INDEX_RANGE, "a scatter index or a segment offset fell outside its array");
   if (raised(dev::kStatusEmptySegment)) return set_error(ACC_ERR_SHAPE, "an empty segment has no value: segment offsets must increase");
-  words[kSettled] = 1;
+  std::lock_guard<std::mutex> lock(g.reports_guard);
+  const RunReport* now = report_for(g, workspace);
+  if (now && now->run_id == r.run_id) r.words.get()[kSettled] = 1;
   return ACC_OK;
 }
 

@@ -4,6 +4,7 @@
 #include <cstdarg>
 #include <cstdint>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -56,6 +57,7 @@ struct Graph {
   int32_t launches = 0;
   std::string schedule;
   std::vector<RunReport> reports;  // one per workspace that runs were enqueued over
+  std::mutex reports_guard;        // (one thread may wait for a run while another enqueues the next)
   uint32_t run_serial = 0;         // bumped by every change that invalidates a schedule
   uint32_t spin_limit = 1u << 22;  // polls a scan tile spends on a predecessor before it gives up (acc_set_spin_limit)
 };

@@ -4,11 +4,13 @@
 #include <cxxabi.h>
 #include <dlfcn.h>
 
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <thread>
 
 struct dim3 { unsigned x, y, z; };
 
@@ -22,6 +24,7 @@ static uint32_t status_run = 0;
 static int32_t second[8];                    // of the last launch of k_hist: its second argument's first words
 
 static int note(const void* kernel, dim3 grid, dim3 block, void** args, bool coop) {
+  if (launches.size() > (1u << 20)) launches.clear();
   Dl_info info;
   std::string name = "?";
   if (dladdr(kernel, &info) && info.dli_sname) {
@@ -70,6 +73,26 @@ const char* fake_launches() { return launches.c_str(); }
 const int32_t* fake_second_argument() { return second; }
 int fake_pages() { return n_pages; }
 uint32_t* fake_status(uint32_t* run) { *run = status_run; return status_words; }
+
+// Two threads over one handle: one enqueues `runs` runs over workspaces of their own, the other waits for those before it;
+// how many calls failed.
+int fake_run_and_wait(int (*run)(void*, void*, size_t, void*, int), int (*finish)(void*, void*, void*), void* handle, int executor, int runs) {
+  std::atomic<int> begun{0}, failed{0};
+  const auto workspace = [](int k) { return reinterpret_cast<void*>((uintptr_t(1) << 50) + (uintptr_t(k) << 20)); };
+  std::thread waits([&] {
+    for (int k = 0; k < runs; ++k) {
+      while (begun.load() <= k) {}
+      if (finish(handle, workspace(k), nullptr) != 0) ++failed;
+      if (finish(handle, workspace(k / 2), nullptr) != 0) ++failed;
+    }
+  });
+  for (int k = 0; k < runs; ++k) {
+    if (run(handle, workspace(k), size_t(1) << 40, nullptr, executor) != 0) ++failed;
+    begun = k + 1;
+  }
+  waits.join();
+  return failed;
+}
 
 int cudaGetDevice(int* d) { *d = 0; return 0; }
 int cudaDeviceGetAttribute(int* v, int, int) { *v = 1; return 0; }

@@ -56,7 +56,7 @@ def launches(prog, pi=None, recompute=0):
 def child(tmp_path_factory):
     """Runs a script behind CHILD in a process of its own and returns what it leaves in `result`."""
     fake = str(tmp_path_factory.mktemp("fake") / "fake_cuda.so")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-o", fake, os.path.join(HERE, "fake_cuda.cpp"), "-ldl"], check=True)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-o", fake, os.path.join(HERE, "fake_cuda.cpp"), "-ldl", "-pthread"], check=True)
 
     def run(script):
         p = subprocess.run([sys.executable, "-c", CHILD + script + "\nprint('RESULT' + json.dumps(result))", fake, os.path.dirname(HERE), HERE],
@@ -225,3 +225,11 @@ result = [[k[0], k[4]] for k in launches(W.sum_of_two_gathers(1 << 20)) + launch
           launches(W.row_scans(1, 1 << 23), [-1, 0, 1, 1]) + launches(W.config3(1 << 25))[-1:]]
 """)
     assert got == [["k_scan", False]] + [["k_scan", True]] * 2 + [["k_scan_ring", True]] * 2 + [["k_scan_merge_pipelined", True]]
+
+
+def test_one_thread_waits_while_another_enqueues(child):
+    got = child(STATUS + """
+g = bound(prog)
+result = fake.fake_run_and_wait(C.cast(lib.acc_run, C.c_void_p), C.cast(lib.acc_finish, C.c_void_p), g._h, B.FUSED, 3000)
+""")
+    assert got == 0
