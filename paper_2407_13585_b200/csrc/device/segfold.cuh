@@ -21,8 +21,8 @@
 // (Before, a block walked tiles of 4096 elements with ten barriers each, about 800 instructions per
 // thread where a tile held several segments, and sources without 128-bit rows went through shared
 // memory element by element.  2^27 elements, a sum and a maximum: 2^20 segments of
-// Zipf lengths 243 -> 188 us, 2^15 segments 184 -> 150, 2^24 segments 450 -> 431; 10^6 elements in 10^4 segments 42.5 ->
-// 16.5.  What bounds it now is latency: a warp's step waits for its loads, then for the scan's shuffles, with 46 % of the issue
+// Zipf lengths 243 -> 178 us, 2^15 segments 184 -> 143, 2^24 segments 450 -> 413; 10^6 elements in 10^4 segments 42.5 ->
+// 16.5.  What bounds it now is latency: a warp's step waits for its loads, then for the scan's shuffles, with 42 % of the issue
 // slots used.)
 //
 // Several segmented folds of one cluster (say a sum and a maximum over the same segments) share
