@@ -1,5 +1,5 @@
-// Generated by `python -m paper_2407_13585_b200.instantiate` from workloads:sum_of_two_gathers and workloads:scan_of_reversed;
-// of each program only the cluster of all its nodes is kept (its nodes alone are among those of csrc/programs).
+// Clusters of workloads:sum_of_two_gathers and workloads:scan_of_reversed, as `python -m paper_2407_13585_b200.instantiate` prints
+// them, of each program only the one of all its nodes (its nodes alone are among those of csrc/programs).
 #include "device/launch.cuh"
 
 namespace acc {

@@ -1,5 +1,5 @@
-// Generated by `python -m paper_2407_13585_b200.instantiate` from workloads:gathered_scans, for the roots that the tests ask for;
-// of each program only the cluster of all its nodes is kept (its nodes alone are among those of csrc/programs).
+// Clusters of workloads:gathered_scans for the roots that the tests ask for, as `python -m paper_2407_13585_b200.instantiate`
+// prints them, of each program only the one of all its nodes (its nodes alone are among those of csrc/programs).
 #include "device/launch.cuh"
 
 namespace acc {
