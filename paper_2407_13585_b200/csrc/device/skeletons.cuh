@@ -459,14 +459,14 @@ __device__ __forceinline__ void st_state(uint64_t* p, uint32_t flag, uint32_t v,
 }
 __device__ __forceinline__ uint32_t flag_of(uint64_t s) { return (uint32_t)s & 3u; }
 __device__ __forceinline__ uint32_t value_of(uint64_t s) { return (uint32_t)(s >> 32); }
-// hi + lo of a state of an fp32 sum (lo is zero for a tile's own total)
+// hi + lo of a state of an fp32 sum
 __device__ __forceinline__ double wide_of(uint64_t s) {
   return (double)__uint_as_float(value_of(s)) + (double)__uint_as_float((uint32_t)s & ~3u);
 }
-__device__ __forceinline__ void st_wide(uint64_t* p, double prefix) {
+__device__ __forceinline__ void st_wide(uint64_t* p, uint32_t flag, double prefix) {
   const float hi = (float)prefix;
   const float lo = isfinite(hi) ? (float)(prefix - (double)hi) : 0.0f;     // an overflowed sum stays infinite
-  st_state(p, kFlagPrefix, __float_as_uint(hi), __float_as_uint(lo));
+  st_state(p, flag, __float_as_uint(hi), __float_as_uint(lo));
 }
 
 // stores at a descending chunk: the lanes go back into ascending memory order
@@ -590,7 +590,14 @@ struct ScanTile {
   static constexpr int FN = sn.fn, DT = sn.dtype;
   static constexpr bool REV = sn.kind == ACC_SCANR;
   static constexpr bool EXCL = sn.p0 == 1;                 // seeded and exclusive: element k leaves itself out
+  // fp32 sums: the totals of a warp's rows of 128, of the warps and of the tiles are added up in fp64, and what precedes a
+  // row is rounded once
   static constexpr bool WIDE = FN == ACC_FN_ADD && DT == ACC_F32;
+  using Prefix = std::conditional_t<WIDE, double, uint32_t>;
+  static __device__ __forceinline__ Prefix none() { if constexpr (WIDE) return 0.0; else return identity_of<FN, DT>(); }
+  static __device__ __forceinline__ Prefix wide(uint32_t v) { if constexpr (WIDE) return (double)f_(v); else return v; }
+  static __device__ __forceinline__ Prefix sum(Prefix before, Prefix v) { if constexpr (WIDE) return before + v; else return combine<FN, DT>(before, v); }
+  static __device__ __forceinline__ uint32_t rounded(Prefix p) { if constexpr (WIDE) return u_((float)p); else return p; }
   using IX = std::conditional_t<VEC, std::conditional_t<REV, IxR4, Ix4>, Ix>;
   static_assert(!SLAB || (VEC && PART == kSlabWarpTile && !REV), "the merging scan walks rank-1 tiles of 512-element warp tiles");
 
@@ -605,7 +612,7 @@ struct ScanTile {
   // the scan, and scanned within the warp (val: each element's scan over the warp's part).  Returns the part's total.
   // SLAB: the gathered values of warp tile `wt` lie, grouped by slab, where the scan's results will go; they are put
   // back into element order through `stage` (kSlabWarpTile words of shared memory that this warp owns).
-  static __device__ __forceinline__ uint32_t scan_part(const Args<N>& a, int row, int warp_base, int wt, const SlabIn& slab,
+  static __device__ __forceinline__ Prefix scan_part(const Args<N>& a, int row, int warp_base, int wt, const SlabIn& slab,
                                                        uint32_t* stage, uint32_t (&val)[ROWS][W]) {
     const int lane = threadIdx.x & 31;
     const int n = a.C;                                     // length of a row
@@ -617,7 +624,7 @@ struct ScanTile {
         unpermute_warp_tile<ROWS>(reinterpret_cast<const uint32_t*>(a.n[S].ptr), slab, wt, stage, gathered);
       }
     }
-    uint32_t carry = identity_of<FN, DT>();                // running total of this warp's earlier rows
+    Prefix carry = none();                                 // running total of this warp's earlier rows
 #pragma unroll
     for (int j = 0; j < ROWS; ++j) {
       const int c = warp_base + (j * 32 + lane) * W;
@@ -663,7 +670,7 @@ struct ScanTile {
       }
       uint32_t excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
       if (lane == 0) excl = identity_of<FN, DT>();
-      excl = combine<FN, DT>(carry, excl);
+      excl = combine<FN, DT>(rounded(carry), excl);
       if constexpr (EXCL) {
         // what came before each element: the thread's own earlier elements on top of `excl`
 #pragma unroll
@@ -673,26 +680,29 @@ struct ScanTile {
 #pragma unroll
         for (int e = 0; e < W; ++e) val[j][e] = combine<FN, DT>(excl, val[j][e]);
       }
-      carry = combine<FN, DT>(carry, __shfl_sync(0xFFFFFFFFu, incl, 31));
+      carry = sum(carry, wide(__shfl_sync(0xFFFFFFFFu, incl, 31)));
     }
     return carry;
   }
 
   // One warp publishes the tile's total, looks back over the tiles of its row before it and publishes the tile's
   // inclusive prefix.  Returns (in every lane) what came before the tile.  A wait that runs out sets the status flag.
-  static __device__ __forceinline__ uint32_t look_back(const Args<N>& a, int tile, int in_row, uint32_t tile_total) {
+  static __device__ __forceinline__ Prefix look_back(const Args<N>& a, int tile, int in_row, Prefix tile_total) {
     const int lane = threadIdx.x & 31;
     uint64_t* states = reinterpret_cast<uint64_t*>(a.scratch + 4);
-    uint32_t exclusive = identity_of<FN, DT>();
+    Prefix exclusive = none();
+    auto publish = [&](uint32_t flag, Prefix v) {
+      if constexpr (WIDE) st_wide(states + tile, flag, v);
+      else st_state(states + tile, flag, v);
+    };
     if (in_row == 0) {
-      if (lane == 0) st_state(states + tile, kFlagPrefix, tile_total);
+      if (lane == 0) publish(kFlagPrefix, tile_total);
       return exclusive;
     }
-    if (lane == 0) st_state(states + tile, kFlagAggregate, tile_total);
+    if (lane == 0) publish(kFlagAggregate, tile_total);
     int look = in_row - 1;                                 // tiles of this row before this one
     uint32_t spins = 0;
     bool gave_up = false;
-    double wide = 0.0;                                     // WIDE: the sum of the tiles before this one
     for (;;) {
       const int idx = look - lane;
       const uint64_t* at = states + (tile - in_row) + idx;
@@ -709,7 +719,7 @@ struct ScanTile {
         double part = lane <= stop ? wide_of(s) : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
-        wide += part;
+        exclusive += part;
       } else {
         uint32_t part = lane <= stop ? value_of(s) : identity_of<FN, DT>();
 #pragma unroll
@@ -720,12 +730,7 @@ struct ScanTile {
       look -= 32;
     }
     if (gave_up && lane == 0) raise_status(a, kStatusTimeout);
-    if constexpr (WIDE) {
-      exclusive = u_((float)wide);
-      if (lane == 0) st_wide(states + tile, wide + (double)f_(tile_total));
-    } else {
-      if (lane == 0) st_state(states + tile, kFlagPrefix, combine<FN, DT>(exclusive, tile_total));
-    }
+    if (lane == 0) publish(kFlagPrefix, sum(exclusive, tile_total));
     return exclusive;
   }
 
@@ -799,8 +804,8 @@ template <class CL, bool VEC, bool SLAB>
 __device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per_row, int n_tiles, const SlabIn& slab, bool resident) {
   using T = ScanTile<CL, VEC, SLAB>;
   constexpr int BLOCK = T::BLOCK, FN = T::FN, DT = T::DT;
-  __shared__ uint32_t warp_total[BLOCK / 32];
-  __shared__ uint32_t tile_prefix;
+  __shared__ typename T::Prefix warp_total[BLOCK / 32];
+  __shared__ typename T::Prefix tile_prefix;
   __shared__ int tile_id;
   __shared__ __align__(16) uint32_t slab_stage[SLAB ? BLOCK / 32 : 1][SLAB ? kSlabWarpTile : 1];   // read and written 128 bits at a time
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -828,23 +833,23 @@ __device__ __forceinline__ void scan_tiles(const Args<CL::c.n>& a, int tiles_per
     }
 
     uint32_t val[T::ROWS][T::W];
-    const uint32_t carry = T::scan_part(a, row, warp_base, tile * (BLOCK / 32) + warp, slab, slab_stage[SLAB ? warp : 0], val);
+    const auto carry = T::scan_part(a, row, warp_base, tile * (BLOCK / 32) + warp, slab, slab_stage[SLAB ? warp : 0], val);
     if (lane == 0) warp_total[warp] = carry;
     __syncthreads();
-    uint32_t offset = identity_of<FN, DT>();               // total of the warps before this one
-    uint32_t tile_total = identity_of<FN, DT>();
+    typename T::Prefix offset = T::none();                 // total of the warps before this one
+    typename T::Prefix tile_total = T::none();
 #pragma unroll
     for (int w = 0; w < BLOCK / 32; ++w) {
-      const uint32_t t = warp_total[w];
-      if (w < warp) offset = combine<FN, DT>(offset, t);
-      tile_total = combine<FN, DT>(tile_total, t);
+      const auto t = warp_total[w];
+      if (w < warp) offset = T::sum(offset, t);
+      tile_total = T::sum(tile_total, t);
     }
     if (warp == 0) {
-      const uint32_t exclusive = T::look_back(a, tile, in_row, tile_total);
+      const auto exclusive = T::look_back(a, tile, in_row, tile_total);
       if (lane == 0) tile_prefix = exclusive;
     }
     __syncthreads();
-    T::finish_part(a, row, warp_base, combine<FN, DT>(tile_prefix, offset), val);
+    T::finish_part(a, row, warp_base, T::rounded(T::sum(tile_prefix, offset)), val);
   }
 }
 
@@ -894,8 +899,8 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
       uint32_t earlier = __shfl_up_sync(0xFFFFFFFFu, incl, 1);                 // total of the parts before lane's
       if (lane == 0) earlier = identity_of<FN, DT>();
       const uint32_t tile_total = __shfl_sync(0xFFFFFFFFu, incl, WARPS - 1);
-      const uint32_t exclusive = T::look_back(a, tile, in_row, tile_total);
-      if (lane < WARPS) part_before[half][lane] = combine<FN, DT>(exclusive, earlier);
+      const auto exclusive = T::look_back(a, tile, in_row, T::wide(tile_total));
+      if (lane < WARPS) part_before[half][lane] = T::rounded(T::sum(exclusive, T::wide(earlier)));
       bar_arrive<3>(half, BLOCK + 32);
     }
   }
@@ -924,7 +929,7 @@ __device__ __forceinline__ void scan_tiles_pipelined(const Args<CL::c.n>& a, int
     T::prefetch_part(a, (tile + G) * WARPS + warp, slab);
     {
       uint32_t val[ROWS][4];
-      const uint32_t total = T::scan_part(a, row, in_row * T::TILE + warp * T::PART, tile * WARPS + warp, slab, mine, val);
+      const uint32_t total = T::rounded(T::scan_part(a, row, in_row * T::TILE + warp * T::PART, tile * WARPS + warp, slab, mine, val));
       __syncwarp();                                        // (every lane has taken its merged values out of `mine`)
 #pragma unroll
       for (int j = 0; j < ROWS; ++j) *reinterpret_cast<uint4*>(mine + (j * 32 + lane) * 4) = make_uint4(val[j][0], val[j][1], val[j][2], val[j][3]);

@@ -701,6 +701,18 @@ def test_scans_by_resident_tiles(rows, cols):
     check_program(W.row_scans(rows, cols), [[-1, 0, 1, 1]])
 
 
+@pytest.mark.parametrize("rows,cols", [(64, 17000), (148, 33000), (32, 30001)])
+def test_tiles_that_look_back_round_what_precedes_a_row_of_128_once(rows, cols):
+    """Running sums of positive addends against fp64.  An element is what precedes its 128, rounded to fp32, plus its place
+    among them: two roundings of about its own size, each 2^-24 / sqrt(3) of it at the most in the mean square (together
+    4.9e-8), and those inside the 128, a hundredth of that size.  (With fp32 carries inside a tile 5.5e-8 to 6.3e-8.)"""
+    prog = W.row_scans(rows, cols)
+    inputs = {k: v.abs() for k, v in W.make_inputs(prog).items()}
+    got, _ = gpu_run(prog, inputs, [-1, 0, 1, 1])
+    exact = np.cumsum(inputs[0].numpy().astype(np.float64).reshape(rows, cols), axis=1)
+    assert np.linalg.norm(got[1].astype(np.float64) - exact) <= 4.9e-8 * np.linalg.norm(exact)
+
+
 @pytest.mark.parametrize("n", [300000, 1 << 20])
 def test_seeded_and_reversed_scans_by_resident_tiles(n):
     check_program(W.exclusive_scans(n))
