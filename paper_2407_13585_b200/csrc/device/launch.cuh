@@ -355,6 +355,7 @@ struct Launcher {
     int R, C;
     if (!domain(L, R, C)) return 0;
     if (use_tiles(L, R, C)) return dev::tile_partials_off((R + dev::kTile - 1) / dev::kTile) * 4;
+    if (kHasSegFold) return 0;
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
     if (kHasScan && use_ring(L, R, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
     if (stream_slab_shapes_ok(L, R, C)) return (((int64_t)dev::stream_acc64_off(kScalarFolds, sm_count() * 8) * 4) + 15) & ~int64_t(15);
@@ -546,8 +547,13 @@ struct Launcher {
         // (chunks of four start on 16 bytes whatever the length; behind an index map they need 128-bit rows)
         const int src = CL::c.nodes[dev::first_segfold<CL>()].in[0];
         const int run = dev::seg_run((int64_t)L.nodes[src].R * L.nodes[src].C, sm_count());
-        if (!dev::has_index_map<CL>() || seg_vec_ok(L)) dev::k_segfold<CL, true><<<grid, dev::kBlock, 0, L.stream>>>(a, run);
-        else dev::k_segfold<CL, false><<<grid, dev::kBlock, 0, L.stream>>>(a, run);
+        if (!dev::has_index_map<CL>() || seg_vec_ok(L)) {
+          constexpr size_t smem = dev::seg_landing_bytes<CL, true>();
+          static int granted[64];
+          if (!opt_in_shared_memory(dev::k_segfold<CL, true>, smem, granted))
+            return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
+          dev::k_segfold<CL, true><<<grid, dev::kBlock, smem, L.stream>>>(a, run);
+        } else dev::k_segfold<CL, false><<<grid, dev::kBlock, 0, L.stream>>>(a, run);
         dev::k_segfold_across<CL><<<(grid + dev::kBlock / 32 - 1) / (dev::kBlock / 32), dev::kBlock, 0, L.stream>>>(a, grid);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));

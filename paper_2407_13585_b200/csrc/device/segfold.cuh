@@ -18,12 +18,11 @@
 //    continues one begun earlier: `head`), and a second, small launch (k_segfold_across) combines the
 //    records in block order.
 //
-// (Before, a block walked tiles of 4096 elements with ten barriers each, about 800 instructions per
-// thread where a tile held several segments, and sources without 128-bit rows went through shared
-// memory element by element.  2^27 elements, a sum and a maximum: 2^20 segments of
-// Zipf lengths 243 -> 178 us, 2^15 segments 184 -> 143, 2^24 segments 450 -> 413; 10^6 elements in 10^4 segments 42.5 ->
-// 16.5.  What bounds it now is latency: a warp's step waits for its loads, then for the scan's shuffles, with 42 % of the issue
-// slots used.)
+// (A block that walked tiles of 4096 elements with ten barriers each took 243 us for a sum and a maximum of 2^27 elements in 2^20
+// segments of Zipf lengths, 184 in 2^15 segments, 450 in 2^24, 42.5 for 10^6 in 10^4.  Warps on their own, with loads into
+// registers ahead of a step's work, 176, 144, 407 and 17.1; with operands that land in shared memory two steps ahead, below, and
+// without records cleared beforehand, 156, 130, 405 and 13.7: 54 % of the issue slots, the rest mostly a warp's waits for offsets
+// and for the shuffles of its scan.)
 //
 // Several segmented folds of one cluster (say a sum and a maximum over the same segments) share
 // the walk.  Results do not depend on timing: every order of combination is fixed by the layout.
@@ -41,6 +40,9 @@ namespace dev {
 constexpr int kSegStep = 512;                  // elements of a warp's step
 constexpr int kSegMaxRun = 4096;               // consecutive elements of a warp, at most: what amortises finding its first segment
 constexpr int kSegStride = 20;                 // words a lane's 16 elements take in shared memory: an odd multiple of 16 bytes, no bank conflicts
+// ... without room to spare, where operands land: a lane's 16 elements side by side, chunks of four swapped so that eight lanes
+// that read theirs 128 bits at a time meet no bank twice.  Word of chunk c of lane l:
+__device__ __forceinline__ int seg_chunk(int l, int c) { return l * 16 + ((c ^ ((l >> 1) & 3)) << 2); }
 constexpr int kSegResident = 4;                // blocks per SM the kernel is built for (5: 191 -> 257 us for 2^27 elements)
 // Elements of a warp's run: what leaves the fewest steps (2 to 3 us each, mostly latency) to the blocks that an SM's places see
 // one after another, counting one for finding a run's first segment.  As many steps as fit the first time round, which leaves
@@ -76,7 +78,7 @@ template <class CL> constexpr bool segfold_eligible() {
 }
 
 // Scratch of k_segfold (32-bit words): from word 4 two records per block, `head`
-// then `tail`, of 2 + NF words each: segment id + 1 (0: no record), unused, one value per fold.
+// then `tail`, of 2 + NF words each: segment id + 1 (0: no record), unused, one value per fold.  Every block writes its own.
 __host__ __device__ inline int seg_record_words(int n_folds) { return 2 + n_folds; }
 __host__ __device__ inline int64_t seg_scratch_words(int n_folds, int grid) { return 4 + (int64_t)grid * 2 * seg_record_words(n_folds); }
 
@@ -95,6 +97,42 @@ __device__ __forceinline__ int seg_containing(const int32_t* off, int S, int x, 
   return lo;
 }
 
+// ---- operands that land in shared memory before they are wanted ------------------------------------------------
+// Folds whose operands are computed from one array, element by element, have a warp's next two steps of that array under way
+// in asynchronous copies, straight to where a lane finds its 16 consecutive elements: no step waits for memory, no operand is
+// written to shared memory to be read again in another order, and no registers hold what another fold will need.  Two steps of
+// 2 KB a warp are what four blocks per SM have room for; three steps and three blocks 174 against 156 us (2^27 elements,
+// Zipf lengths).  The search for a run's first segment comes before the first copies: behind them its loads wait (164 -> 172 us).
+struct IxLd4 { int r, c; const uint32_t* landed; };                 // four consecutive elements, and where their array's lie
+__device__ __forceinline__ Ix lane(const IxLd4& i, int j) { return Ix{i.r, i.c + j}; }
+template <int F, int P0 = kRunTime, int P1 = kRunTime>
+__device__ __forceinline__ auto map_index(const IxLd4& i, const NodeArg&, const NodeArg&) {
+  static_assert(F == ACC_IDX_IDENTITY, "operands that land ahead are read in place");
+  return i;
+}
+template <class CL, int I, class A> __device__ __forceinline__ V4 ld_ext(const A&, const IxLd4& ix) {
+  const uint4 v = *reinterpret_cast<const uint4*>(ix.landed);
+  return V4{{v.x, v.y, v.z, v.w}};
+}
+// the one array that member i is computed from, element by element; -1: none yet, -2: anything else
+template <class CL> constexpr int seg_array_below(int i, int so_far) {
+  const CNode& n = CL::c.nodes[i];
+  if (so_far == -2) return -2;
+  if (!n.member) return n.rank == 1 && (so_far == -1 || so_far == i) ? i : -2;
+  if (n.kind == ACC_GENERATE) return so_far;
+  if (n.kind != ACC_MAP && n.kind != ACC_ZIPWITH && (n.kind != ACC_BACKPERMUTE || n.idxfn != ACC_IDX_IDENTITY)) return -2;
+  for (int k = 0; k < n.narr; ++k) so_far = seg_array_below<CL>(n.in[k], so_far);
+  return so_far;
+}
+template <class CL> constexpr int seg_landing_array() {
+  int x = -1;
+  for (int i = 0; i < CL::c.n; ++i)
+    if (is_segfold_root(CL::c.nodes[i])) x = seg_array_below<CL>(CL::c.nodes[i].in[0], x);
+  return x;
+}
+constexpr int kSegAhead = 2;                   // steps whose copies are under way
+template <class CL, bool VEC> constexpr size_t seg_landing_bytes() { return VEC && seg_landing_array<CL>() >= 0 ? (size_t)kSegAhead * kSegStep * 4 * (kBlock / 32) : 0; }
+
 template <class CL, bool VEC>
 __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_constant__ Args<CL::c.n> a, int run_length) {
   constexpr int N = CL::c.n;
@@ -103,12 +141,14 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
   constexpr int WARPS = kBlock / 32, ROWS = 4, STEP = kSegStep;
   constexpr int REC = 2 + NF;
   __shared__ uint32_t bits[WARPS][STEP / 32];                    // bit p: element p of the warp's step begins a segment
-  __shared__ __align__(16) uint32_t staged[WARPS][32 * kSegStride];   // a step's operands, then the value of every prefix within its lane
+  __shared__ __align__(16) uint32_t staged[WARPS][32 * kSegStride];   // the value of every prefix within its lane (before that a step's operands, if they do not land ahead)
   // what a warp leaves for the block: the segment that is open at its end and its value there, and, where a segment begins
   // in the warp's run, that segment and the value of the one that ends at the first start
   __shared__ int open_seg[WARPS], first_seg[WARPS];              // first_seg: -1 if none begins; open_seg -1: no elements
   __shared__ bool has_head[WARPS];                               // the segment that ends at the first start has elements in the run
   __shared__ uint32_t open_val[NF][WARPS], head_val[NF][WARPS];
+  constexpr int LAND = VEC ? seg_landing_array<CL>() : -2;         // the array that lands ahead
+  extern __shared__ __align__(16) uint32_t landing_smem[];       // [warp][step % kSegAhead][STEP]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int S = a.C;                                             // segments
   constexpr int OFF = CL::c.nodes[F].in[1], SRC = CL::c.nodes[F].in[0];
@@ -128,8 +168,28 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
   const int64_t run_lo = ((int64_t)blockIdx.x * WARPS + warp) * run_length;
   const int lo0 = (int)(run_lo > e_lo ? run_lo : e_lo), hi0 = (int)(run_lo + run_length < e_hi ? run_lo + run_length : e_hi);
   if (lane == 0) { open_seg[warp] = -1; first_seg[warp] = -1; }
+  if (threadIdx.x < 2) rec[((size_t)blockIdx.x * 2 + threadIdx.x) * REC] = 0;    // no record yet (nobody clears them beforehand)
   if (lo0 < hi0) {                                               // uniform
-    // the elements of a step; what lies outside [lo0, hi0) reads as the operator's identity
+    uint32_t* const landing = landing_smem + (size_t)warp * kSegAhead * STEP;
+    int slot = 0;                                                // of the step that is worked on
+    auto land = [&](int base) {                                  // (a group is closed for every step, so that they can be counted)
+      if constexpr (LAND >= 0) {
+        const int last = (n_src & ~3) - 4;
+        if (base < hi0 && last >= 0) {
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(a.n[LAND].ptr);
+          const uint32_t to = (uint32_t)__cvta_generic_to_shared(landing + slot * STEP);
+#pragma unroll
+          for (int j = 0; j < ROWS; ++j) {
+            const int q = j * 32 + lane;                         // chunk of the step
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + seg_chunk(q >> 2, q & 3) * 4), "l"(src + min(base + q * 4, last)) : "memory");
+          }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+    };
+    // the elements of a step; what lies outside [lo0, hi0) reads as the operator's identity.  A lane takes chunks of four:
+    // those of its 16 consecutive elements where they have landed, else every 32nd.
+    auto chunk_begin = [&](int base, int j) { return base + (LAND >= 0 ? lane * 16 + j * 4 : (j * 32 + lane) * 4); };
     auto operands = [&](auto ic, int base, uint32_t (&x)[ROWS][4]) {
       constexpr int i = decltype(ic)::value;
       constexpr CNode nd = CL::c.nodes[i];
@@ -141,7 +201,10 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
         if (last >= 0) {
 #pragma unroll
           for (int j = 0; j < ROWS; ++j) {
-            const V4 v = eval<CL, nd.in[0]>(a, Ix4{0, min(base + (j * 32 + lane) * 4, last)});
+            const int c = chunk_begin(base, j);
+            V4 v;
+            if constexpr (LAND >= 0) v = eval<CL, nd.in[0]>(a, IxLd4{0, c, landing + slot * STEP + seg_chunk(lane, j)});
+            else v = eval<CL, nd.in[0]>(a, Ix4{0, min(c, last)});
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[j][e] = v.v[e];
           }
@@ -149,7 +212,7 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
         if (!whole) {
 #pragma unroll
           for (int j = 0; j < ROWS; ++j) {
-            const int c = base + (j * 32 + lane) * 4;
+            const int c = chunk_begin(base, j);
             if (c > last && c < n_src) {                         // the array's last few elements
 #pragma unroll
               for (int e = 0; e < 3; ++e)
@@ -165,11 +228,17 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
         for (int j = 0; j < ROWS; ++j)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const int p = base + (j * 32 + lane) * 4 + e;
+            const int p = chunk_begin(base, j) + e;
             x[j][e] = p >= lo0 && p < hi0 ? eval<CL, nd.in[0]>(a, Ix{0, p}) : identity_of<nd.fn, nd.dtype>();
           }
       }
     };
+    const int base0 = (int)run_lo + (lo0 - (int)run_lo) / STEP * STEP;   // the first step with elements of a segment
+    if constexpr (LAND >= 0) {
+#pragma unroll
+      for (slot = 0; slot < kSegAhead; ++slot) land(base0 + slot * STEP);
+      slot = 0;
+    }
     const int s0 = seg_containing(off, S, lo0, lane);
     int next = __ldg(off + s0) == lo0 ? s0 : s0 + 1;             // the next segment to begin
     const int first = next;
@@ -192,9 +261,8 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
       constexpr CNode nd = CL::c.nodes[i];
       if constexpr (is_segfold_root(nd)) acc[i] = open[i] = identity_of<nd.fn, nd.dtype>();
     });
-    for (int base = (int)run_lo; base < hi0; base += STEP) {
-      if (base + STEP <= lo0) continue;
-      if constexpr (VEC) {
+    for (int base = base0; base < hi0; base += STEP) {
+      if constexpr (VEC && LAND < 0) {
         // steps far inside a long segment, two at a time: twice the loads under way (2^24 elements in one segment 24.6 -> 20.6 us,
         // 2^27 Zipf lengths 189 -> 178)
         while (base + 2 * STEP <= hi0 && base >= lo0 && __shfl_sync(0xFFFFFFFFu, o[0], 0) >= base + 2 * STEP) {
@@ -223,12 +291,24 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
         }
         if (base >= hi0) break;
       }
-      uint32_t x[N][ROWS][4];
-      static_for<0, N>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        if constexpr (is_segfold_root(CL::c.nodes[i])) operands(ic, base, x[i]);
-      });
-      if constexpr (VEC) {                                       // the next step's lines, asked into L2
+      uint32_t x[LAND >= 0 ? 1 : N][ROWS][4];                     // (of one fold after another where they have landed)
+      auto ahead = [&]() {                                        // every lane has its last values of the step: its room goes to a later one
+        if constexpr (LAND >= 0) {
+          __syncwarp();
+          land(base + kSegAhead * STEP);
+          slot = slot + 1 == kSegAhead ? 0 : slot + 1;
+        }
+      };
+      if constexpr (LAND >= 0) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSegAhead - 1) : "memory");
+        __syncwarp();
+      } else {
+        static_for<0, N>([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          if constexpr (is_segfold_root(CL::c.nodes[i])) operands(ic, base, x[i]);
+        });
+      }
+      if constexpr (VEC && LAND < 0) {                                       // the next step's lines, asked into L2
         if (base + 2 * STEP <= hi0 && (lane & 7) == 0) {
           static_for<0, N>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
@@ -245,12 +325,15 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
           constexpr int i = decltype(ic)::value;
           constexpr CNode nd = CL::c.nodes[i];
           if constexpr (is_segfold_root(nd)) {
+            constexpr int at = LAND >= 0 ? 0 : i;
+            if constexpr (LAND >= 0) operands(ic, base, x[at]);
 #pragma unroll
             for (int j = 0; j < ROWS; ++j)
-              fold_step<nd.fn, nd.dtype>(acc[i], comp[i], combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(x[i][j][0], x[i][j][1]),
-                                                                                   combine<nd.fn, nd.dtype>(x[i][j][2], x[i][j][3])));
+              fold_step<nd.fn, nd.dtype>(acc[i], comp[i], combine<nd.fn, nd.dtype>(combine<nd.fn, nd.dtype>(x[at][j][0], x[at][j][1]),
+                                                                                   combine<nd.fn, nd.dtype>(x[at][j][2], x[at][j][3])));
           }
         });
+        ahead();
         continue;
       }
       if (lane < STEP / 32) bits[warp][lane] = 0;
@@ -284,22 +367,32 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
           acc[i] = identity_of<nd.fn, nd.dtype>();
           comp[i] = 0.0f;
           uint32_t* mine = staged[warp];
+          constexpr int at = LAND >= 0 ? 0 : i;
+          if constexpr (LAND >= 0) {
+            operands(ic, base, x[at]);
+            if constexpr (count_if<CL>(is_segfold_root, i + 1) == NF) ahead();   // (the last fold)
+          } else {
 #pragma unroll
-          for (int j = 0; j < ROWS; ++j) {
-            const int q = j * 32 + lane;                          // chunk of four: the (q % 4)-th of lane q / 4
-            *reinterpret_cast<uint4*>(mine + (q >> 2) * kSegStride + (q & 3) * 4) = make_uint4(x[i][j][0], x[i][j][1], x[i][j][2], x[i][j][3]);
+            for (int j = 0; j < ROWS; ++j) {
+              const int q = j * 32 + lane;                        // chunk of four: the (q % 4)-th of lane q / 4
+              *reinterpret_cast<uint4*>(mine + (q >> 2) * kSegStride + (q & 3) * 4) = make_uint4(x[at][j][0], x[at][j][1], x[at][j][2], x[at][j][3]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < ROWS; ++j) {
+              const uint4 v = *reinterpret_cast<const uint4*>(mine + lane * kSegStride + j * 4);
+              x[at][j][0] = v.x; x[at][j][1] = v.y; x[at][j][2] = v.z; x[at][j][3] = v.w;
+            }
           }
-          __syncwarp();
           uint32_t run = identity_of<nd.fn, nd.dtype>();
-          uint32_t* own = mine + lane * kSegStride;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            uint4 v = *reinterpret_cast<const uint4*>(own + 4 * c);
-            v.x = run = ((b >> (4 * c + 0)) & 1u) ? v.x : combine<nd.fn, nd.dtype>(run, v.x);
-            v.y = run = ((b >> (4 * c + 1)) & 1u) ? v.y : combine<nd.fn, nd.dtype>(run, v.y);
-            v.z = run = ((b >> (4 * c + 2)) & 1u) ? v.z : combine<nd.fn, nd.dtype>(run, v.z);
-            v.w = run = ((b >> (4 * c + 3)) & 1u) ? v.w : combine<nd.fn, nd.dtype>(run, v.w);
-            *reinterpret_cast<uint4*>(own + 4 * c) = v;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const uint32_t v = x[at][c][e];
+              x[at][c][e] = run = ((b >> (4 * c + e)) & 1u) ? v : combine<nd.fn, nd.dtype>(run, v);
+            }
+            *reinterpret_cast<uint4*>(mine + lane * kSegStride + c * 4) = make_uint4(x[at][c][0], x[at][c][1], x[at][c][2], x[at][c][3]);
           }
 #pragma unroll
           for (int d = 1; d < 32; d <<= 1) {
@@ -309,7 +402,7 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
           uint32_t into = __shfl_up_sync(0xFFFFFFFFu, run, 1);    // what runs into the lane's elements
           if (lane == 0) into = open[i];
           else if (led) into = combine<nd.fn, nd.dtype>(open[i], into);
-          own[16] = into;                                         // (a word of the lane's padding)
+          mine[lane * kSegStride + 16] = into;                    // (a word of the lane's padding)
           open[i] = __shfl_sync(0xFFFFFFFFu, run, 31);            // (some segment begins in the step, so this began in it)
           __syncwarp();
           // a lane per start: the segment before it ends in front of it
@@ -334,6 +427,7 @@ __global__ void __launch_bounds__(kBlock, kSegResident) k_segfold(const __grid_c
       });
       next += begun;
     }
+    if constexpr (LAND >= 0) asm volatile("cp.async.wait_all;" ::: "memory");
     static_for<0, N>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       constexpr CNode nd = CL::c.nodes[i];

@@ -519,6 +519,19 @@ def test_segmented_fold_by_warps(n, segments):
     assert check_program(W.segmented_sums(n, segments), [[-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2]]) == 2
 
 
+# the segments cover part of the source only: steps of a run before the first segment, a first segment that begins with a step,
+# at its end or inside it, a last one that ends with the array's last, incomplete chunk or long before; no records from before
+@pytest.mark.parametrize("n,lo,hi", [(70003, 0, 70003), (70003, 512, 70001), (70002, 1535, 70002), (70001, 5000, 5001), (4099, 4096, 4099), (3, 1, 3),
+                                     (300000, 299000, 299999), (300000, 1, 262145)])
+def test_segmented_fold_of_part_of_the_source(n, lo, hi):
+    import torch
+    segments = max(1, (hi - lo) // 37)
+    prog = W.segmented_sums(n, segments)
+    inputs = W.make_inputs(prog)
+    inputs[1] = torch.from_numpy(np.linspace(lo, hi, segments + 1).astype(np.int32))
+    check_program(prog, [[-1, -1, 0, 0, 0], [-1, -1, 0, 0, 1]], inputs_t=inputs, runs=2)
+
+
 @pytest.mark.parametrize("tail", [0, 3])
 def test_segmented_fold_where_a_window_of_offsets_ends_at_a_straddling_segment(tail):
     """Tiles whose last segment, one that goes on into the next tile, is the last of a chunk of 256 offsets, so that the
