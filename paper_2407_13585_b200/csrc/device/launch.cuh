@@ -119,6 +119,11 @@ struct Launcher {
     return (int)std::max<int64_t>(1, std::min<int64_t>(trips, (int64_t)sm_count() * 8));
   }
 
+  // folds of few elements, over all arrays that are read or stored: one cluster of blocks (k_stream_few, where both sides' times are)
+  static constexpr bool kFewShape = dev::few_eligible<CL>();
+  static constexpr int kFewElements = 1 << 17;
+  static bool use_few(const ClusterLaunch&, int R, int C) { return kFewShape && (int64_t)R * C * dev::few_arrays<CL>() <= kFewElements; }
+
   // transposes staged through shared-memory tile pairs (k_tile_pair)
   static constexpr bool kTileShape = dev::tile_eligible<CL>();
   static constexpr int kRowFolds = dev::count_if<CL>(dev::is_row_fold);
@@ -359,6 +364,7 @@ struct Launcher {
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
     if (kHasScan && use_ring(L, R, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
     if (stream_slab_shapes_ok(L, R, C)) return (((int64_t)dev::stream_acc64_off(kScalarFolds, sm_count() * 8) * 4) + 15) & ~int64_t(15);
+    if (use_few(L, R, C)) return 0;
     dev::HistPlan plan;
     if (use_hist(L, R, C, plan)) return scratch_bytes(L) - (int64_t)sm_count() * plan.exchange * 4;   // (what is exchanged is written first)
     return scratch_bytes(L);
@@ -642,6 +648,15 @@ struct Launcher {
           for (int k = 0; k < dev::kSlabs; ++k) dev::k_slab_gather<CL><<<ggrid, dev::kBlock, 0, L.stream>>>(a, counts, full, (uint32_t)k, slab);
           dev::k_stream_merge<CL><<<pgrid, dev::kBlock, 0, L.stream>>>(a, slab);
           L.extra_launches += 2 + dev::kSlabs;
+          const cudaError_t e = cudaGetLastError();
+          if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+          return ACC_OK;
+        }
+      }
+      if constexpr (kFewShape) {
+        if (use_few(L, R, C)) {
+          if (stream_vec_ok(L, vec)) dev::k_stream_few<CL, true><<<dev::kFewBlocks, dev::kFewThreads, 0, L.stream>>>(a);
+          else dev::k_stream_few<CL, false><<<dev::kFewBlocks, dev::kFewThreads, 0, L.stream>>>(a);
           const cudaError_t e = cudaGetLastError();
           if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
           return ACC_OK;

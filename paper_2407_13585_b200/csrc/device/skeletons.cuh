@@ -120,28 +120,17 @@ __device__ __forceinline__ double* acc64_of(const A& a, double* base) {
 }
 
 // =========================================================================================
+// The walk of a block of BLOCK threads over its share of the domain: roots are stored, folds added up per thread, scatters made.
 // VEC: rows and the images of chunks under reversal start on 16 bytes.  (A rank-1 domain is walked four elements at a time
 // either way, all but its last few; see Ix4U.)
-template <class CL, bool VEC>
-__global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<CL::c.n> a) {
+template <class CL, bool VEC, int BLOCK>
+__device__ __forceinline__ void stream_walk(const Args<CL::c.n>& a, uint32_t (&acc)[CL::c.n], float (&comp)[CL::c.n], double* acc64_base) {
   constexpr int N = CL::c.n;
   constexpr int DR = domain_rank<CL>();
   constexpr bool FOUR = VEC || DR <= 1;                  // four elements at a time: always over a rank-1 domain
   constexpr int W = FOUR ? 4 : 1;
-  constexpr int NF = count_if<CL>(is_scalar_fold);
-  constexpr int NP64 = count_if<CL>(is_f32_add_permute);
   using IX = std::conditional_t<VEC, Ix4, std::conditional_t<FOUR, Ix4U, Ix>>;
-  __shared__ uint32_t red[kBlock / 32];
-  __shared__ bool last_block;
-
-  uint32_t acc[N];
-  float comp[N] = {};                                    // see fold_step
-  static_for<0, N>([&](auto ic) {
-    constexpr int i = decltype(ic)::value;
-    constexpr CNode nd = CL::c.nodes[i];
-    if constexpr (is_scalar_fold(nd)) acc[i] = identity_of<nd.fn, nd.dtype>();
-  });
-  double* acc64_base = reinterpret_cast<double*>(a.scratch + stream_acc64_off(NF, a.grid));
+  static_assert(DR <= 1 || BLOCK == kBlock, "a warp per row of a tile");
 
   // Rank 1: a grid-stride walk over chunks.  Rank 2: a grid-stride walk over tiles of
   // kStreamTileRows rows x 32 chunks, one warp per row segment (512 contiguous bytes), so that
@@ -155,14 +144,14 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
   // evaluation finds them in L1: an array longer than the L2 crosses DRAM once instead of twice.
   constexpr bool MIRROR = DR <= 1 && has_reversal<CL>();
   const uint32_t half = (per_row + 1) / 2;
-  const uint32_t trips = DR <= 1 ? ((MIRROR ? half : per_row) + kBlock - 1) / kBlock
+  const uint32_t trips = DR <= 1 ? ((MIRROR ? half : per_row) + BLOCK - 1) / BLOCK
                                  : tiles_x * (((uint32_t)a.R + kStreamTileRows - 1) / kStreamTileRows);
   for (uint32_t t = blockIdx.x; t < trips; t += gridDim.x) {
    for (int side = 0; side < (MIRROR ? 2 : 1); ++side) {
     IX ix;
     bool live;
     if constexpr (DR <= 1) {
-      uint32_t q = t * kBlock + threadIdx.x;
+      uint32_t q = t * BLOCK + threadIdx.x;
       live = q < (MIRROR ? half : per_row);
       if (MIRROR && side == 1) {
         live = live && per_row - 1 - q != q;               // the middle chunk of an odd count has no partner
@@ -225,6 +214,25 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
       });
     }
   }
+}
+
+template <class CL, bool VEC>
+__global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<CL::c.n> a) {
+  constexpr int N = CL::c.n;
+  constexpr int NF = count_if<CL>(is_scalar_fold);
+  constexpr int NP64 = count_if<CL>(is_f32_add_permute);
+  __shared__ uint32_t red[kBlock / 32];
+  __shared__ bool last_block;
+
+  uint32_t acc[N];
+  float comp[N] = {};                                    // see fold_step
+  static_for<0, N>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr CNode nd = CL::c.nodes[i];
+    if constexpr (is_scalar_fold(nd)) acc[i] = identity_of<nd.fn, nd.dtype>();
+  });
+  double* acc64_base = reinterpret_cast<double*>(a.scratch + stream_acc64_off(NF, a.grid));
+  stream_walk<CL, VEC, kBlock>(a, acc, comp, acc64_base);
 
   if constexpr (NF > 0 || NP64 > 0) {
     // partial of every scalar fold, then the block that arrives last finishes the job
@@ -259,6 +267,66 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
         float* out = reinterpret_cast<float*>(const_cast<void*>(a.n[i].ptr));
         const int bins = a.n[i].R * a.n[i].C;
         for (int b = threadIdx.x; b < bins; b += kBlock) out[b] = (float)((double)defaults[b] + acc64[b]);
+      }
+    });
+  }
+}
+
+// Folds of few elements: one cluster of blocks, which leave their partial sums in the shared memory of the first, so that there
+// is no counter to clear beforehand (a second thing to launch) and none to go round.  What bounds such calls is how often
+// something is launched and waited for: the chain of 2^16 elements, one run after another, 8.2 -> 4.8 us, waited for 16.5 -> 13.1;
+// of 2^17 (the most that is measured: two mirrored pairs of chunks a thread) 8.1 -> 4.8 and 16.6 -> 13.7.  From there on the grid's
+// many SMs are worth the clearing.
+constexpr int kFewBlocks = 8, kFewThreads = 1024;
+template <class CL> constexpr bool few_eligible() {
+  if (domain_rank<CL>() > 1 || count_if<CL>(is_scalar_fold) == 0) return false;
+  for (int i = 0; i < CL::c.n; ++i) {
+    const CNode& n = CL::c.nodes[i];
+    if (n.member && !is_scalar_fold(n) && (!is_elementwise(n.kind) || n.kind == ACC_GATHER)) return false;   // (random reads and inner loops want all SMs)
+  }
+  return true;
+}
+template <class CL> constexpr int few_arrays() {         // read or written element by element
+  int k = 0;
+  for (int i = 0; i < CL::c.n; ++i) k += CL::c.nodes[i].member ? (is_store_root(CL::c.nodes[i]) ? 1 : 0) : (CL::c.nodes[i].rank > 0 ? 1 : 0);
+  return k > 0 ? k : 1;
+}
+template <class CL, bool VEC>
+__global__ void __cluster_dims__(kFewBlocks, 1, 1) __launch_bounds__(kFewThreads) k_stream_few(const __grid_constant__ Args<CL::c.n> a) {
+  constexpr int N = CL::c.n;
+  constexpr int NF = count_if<CL>(is_scalar_fold);
+  __shared__ uint32_t red[kFewThreads / 32];
+  __shared__ uint32_t part[NF][kFewBlocks];              // the first block's is used
+  uint32_t acc[N];
+  float comp[N] = {};                                    // see fold_step
+  static_for<0, N>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr CNode nd = CL::c.nodes[i];
+    if constexpr (is_scalar_fold(nd)) acc[i] = identity_of<nd.fn, nd.dtype>();
+  });
+  stream_walk<CL, VEC, kFewThreads>(a, acc, comp, nullptr);
+  static_for<0, N>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr CNode nd = CL::c.nodes[i];
+    if constexpr (is_scalar_fold(nd)) {
+      const uint32_t v = block_reduce_n<nd.fn, nd.dtype, kFewThreads>(acc[i], red);
+      if (threadIdx.x == 0) {
+        uint32_t first;                                  // the word in the first block's shared memory
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(first) : "r"((uint32_t)__cvta_generic_to_shared(&part[count_if<CL>(is_scalar_fold, i)][blockIdx.x])));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(first), "r"(v) : "memory");
+      }
+    }
+  });
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    static_for<0, N>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      constexpr CNode nd = CL::c.nodes[i];
+      if constexpr (is_scalar_fold(nd)) {
+        uint32_t v = identity_of<nd.fn, nd.dtype>();
+#pragma unroll
+        for (int b = 0; b < kFewBlocks; ++b) v = combine<nd.fn, nd.dtype>(v, part[count_if<CL>(is_scalar_fold, i)][b]);
+        *reinterpret_cast<uint32_t*>(const_cast<void*>(a.n[i].ptr)) = v;
       }
     });
   }

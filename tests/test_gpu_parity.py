@@ -46,6 +46,13 @@ def test_config1_any_length(n):
     assert check_program(W.config1(n)) == 8
 
 
+# one cluster of blocks: a chunk per thread and one more, the most elements that it takes and one more, in each of the clusters
+# that end in the fold
+@pytest.mark.parametrize("n", [32767, 65533, 65540, 131071, 131072, 131073])
+def test_folds_of_few_elements(n):
+    assert check_program(W.config1(n), runs=2) == 8
+
+
 @pytest.mark.parametrize("n,bins", [(4097, 256), (70001, 256), (70002, 8192), (600003, 70000), (540001, 65536), (170000, 20000)])
 def test_config5_any_length(n, bins):
     assert check_program(W.config5(n, bins)) == 10

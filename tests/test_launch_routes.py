@@ -211,6 +211,16 @@ for n in (1 << 18, 1 << 27, 1 << 30):
     assert [g[2] for g in got] == [(1 << 20) + 8 * s for s in shares]
 
 
+def test_few_elements_are_folded_by_one_cluster_of_blocks(child):
+    """... counted over all arrays that are read or stored (the third cluster reads two); a gather below the fold keeps the grid."""
+    got = child("""
+result = [[k[0], k[2]] for n in (131072, 131073) for k in launches(W.config1(n))]
+result += [launches(W.config1(n), [-1, 0, 0, 0, 1])[1][0] for n in (131072, 131073)]
+result += [launches(W.config1(n), [-1, 0, 0, 1, 1])[1][0] for n in (65536, 65537)]
+""")
+    assert got == [["k_stream_few", 8], ["k_stream", 128]] + ["k_stream_few", "k_stream"] * 2
+
+
 def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
     got = child("""
 result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
