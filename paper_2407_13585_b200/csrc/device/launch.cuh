@@ -128,6 +128,13 @@ struct Launcher {
   static constexpr bool kTileShape = dev::tile_eligible<CL>();
   static constexpr int kRowFolds = dev::count_if<CL>(dev::is_row_fold);
 
+  // ... or, where there are few (and more than one), by a cluster of blocks to every block of rows (k_tile_rows, where both sides'
+  // times are; ahead up to 3000 rows at least, but from 2560 on the array is 26 MB and more, and what a program's other arrays leave of
+  // the L2 decides)
+  static constexpr bool kTileRowsShape = dev::tile_rows_eligible<CL>();
+  static constexpr int kTileRowsMost = 2559;
+  static bool use_tile_rows(int n) { return kTileRowsShape && n > dev::kTile && n <= kTileRowsMost; }
+
   // The tile-pair kernel wants a square domain of at least one tile, and every staged
   // external of that same shape.
   static bool use_tiles(const ClusterLaunch& L, int R, int C) {
@@ -359,7 +366,7 @@ struct Launcher {
   static int64_t zeroed_bytes(const ClusterLaunch& L) {
     int R, C;
     if (!domain(L, R, C)) return 0;
-    if (use_tiles(L, R, C)) return dev::tile_partials_off((R + dev::kTile - 1) / dev::kTile) * 4;
+    if (use_tiles(L, R, C)) return use_tile_rows(R) ? 0 : dev::tile_partials_off((R + dev::kTile - 1) / dev::kTile) * 4;
     if (kHasSegFold) return 0;
     if (kHasScan && slab_shapes_ok(L, R, C)) return ((16 + (int64_t)R * ((C + kScanTile - 1) / kScanTile) * 8) + 15) & ~int64_t(15);
     if (kHasScan && use_ring(L, R, C) && (scan_scratch_bytes(L, R, C) == 16 || C <= dev::kScanBlockRow)) return 0;
@@ -532,6 +539,19 @@ struct Launcher {
     }
     if (use_tiles(L, R, C)) {
       if constexpr (kTileShape) {
+        if constexpr (kTileRowsShape) {
+          if (use_tile_rows(R)) {
+            auto kern = vec ? dev::k_tile_rows<CL, true> : dev::k_tile_rows<CL, false>;
+            const size_t smem = (size_t)dev::staged_externals<CL>() * 2 * dev::kTileWords * 4;
+            static int granted[2][64];
+            if (!opt_in_shared_memory(kern, smem, granted[vec ? 1 : 0]))
+              return set_error(ACC_ERR_CUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(cudaGetLastError()));
+            kern<<<(R + dev::kTile - 1) / dev::kTile * dev::kTrBlocks, dev::kBlock, smem, L.stream>>>(a);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return set_error(ACC_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+            return ACC_OK;
+          }
+        }
         const int rc = launch_tiles_tma(L, a, R, vec);
         if (rc != 1) return rc;                          // 1 = no tensor copies here: the threads stage the tiles
         auto kern = vec ? dev::k_tile_pair<CL, true> : dev::k_tile_pair<CL, false>;

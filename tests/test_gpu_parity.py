@@ -70,6 +70,25 @@ def test_config2_any_extent(rows):
     check_program(W.config2(rows), [[-1, 0, 0, 0]])
 
 
+# a cluster of blocks to a block of rows: two tiles, a last tile of one row, more column tiles than blocks, the most rows; one
+# array and two
+@pytest.mark.parametrize("rows", [65, 128, 513, 520, 577, 2557, 2559])
+def test_row_folds_by_clusters_of_blocks(rows):
+    check_program(W.config2(rows), [[-1, 0, 0, 0]], runs=2)
+    check_program(W.diagonal_of_product(rows), [[-1, -1, 0, 0, 0]], runs=2)
+
+
+# iterates kept on chip, tiles inside the array beside tiles at its edges: box rows that are a multiple of three and not (two, three
+# and four iterations), copied as boxes and word by word
+@pytest.mark.parametrize("rows,cols,iters", [(1026, 640, 2), (1026, 641, 2), (4300, 392, 2), (900, 1028, 3), (900, 1027, 3), (900, 1028, 4), (901, 1030, 4)])
+def test_config4_stacked_iterations_inside_the_array(rows, cols, iters):
+    prog = W.config4(rows, cols, iters=iters)
+    inputs = W.make_inputs(prog)
+    got, g = gpu_run(prog, inputs, [-1] + [0] * (9 * iters), recompute=iters)
+    assert g.launch_count() == 1
+    compare(prog, oracle_run(prog, np_inputs(inputs)), got, "%d iterations, %d x %d" % (iters, rows, cols))
+
+
 # two iterations in one cluster on widths that are no multiple of four: boxes copied word by word, a last column anywhere in
 # its chunk, at a tile's edge and one past it
 @pytest.mark.parametrize("rows,cols", [(1100, 641), (1101, 642), (1090, 643), (4200, 129), (5000, 127)])

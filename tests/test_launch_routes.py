@@ -221,6 +221,13 @@ result += [launches(W.config1(n), [-1, 0, 0, 1, 1])[1][0] for n in (65536, 65537
     assert got == [["k_stream_few", 8], ["k_stream", 128]] + ["k_stream_few", "k_stream"] * 2
 
 
+def test_few_tiles_are_folded_by_clusters_of_blocks(child):
+    got = child("""
+result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][:3:2] for rows in (63, 64, 65, 128, 129, 2559)]
+""")
+    assert got == [["k_rowfold", 63], ["k_tile_pair_tma", 1], ["k_tile_rows", 16], ["k_tile_rows", 16], ["k_tile_rows", 24], ["k_tile_rows", 320]]
+
+
 def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
     got = child("""
 result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
