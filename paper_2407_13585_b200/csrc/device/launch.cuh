@@ -121,7 +121,7 @@ struct Launcher {
 
   // folds of few elements, over all arrays that are read or stored: one cluster of blocks (k_stream_few, where both sides' times are)
   static constexpr bool kFewShape = dev::few_eligible<CL>();
-  static constexpr int kFewElements = 1 << 17;
+  static constexpr int kFewElements = 1 << 18;
   static bool use_few(const ClusterLaunch&, int R, int C) { return kFewShape && (int64_t)R * C * dev::few_arrays<CL>() <= kFewElements; }
 
   // transposes staged through shared-memory tile pairs (k_tile_pair)

@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
 // Folds of few elements: one cluster of blocks, which leave their partial sums in the shared memory of the first, so that there
 // is no counter to clear beforehand (a second thing to launch) and none to go round.  What bounds such calls is how often
 // something is launched and waited for: the chain of 2^16 elements, one run after another, 8.2 -> 4.8 us, waited for 16.5 -> 13.1;
-// of 2^17 (the most that is measured: two mirrored pairs of chunks a thread) 8.1 -> 4.8 and 16.6 -> 13.7.  From there on the grid's
-// many SMs are worth the clearing.
+// of 2^18, the most that it is used for, 8.2 -> 6.2 and 15.6 -> 14.0.  400001 elements take 9.6 against 8.2 us, 2^20 12.3 against 8.2:
+// there the grid's many SMs are worth the clearing.
 constexpr int kFewBlocks = 8, kFewThreads = 1024;
 template <class CL> constexpr bool few_eligible() {
   if (domain_rank<CL>() > 1 || count_if<CL>(is_scalar_fold) == 0) return false;

@@ -48,7 +48,7 @@ def test_config1_any_length(n):
 
 # one cluster of blocks: a chunk per thread and one more, the most elements that it takes and one more, in each of the clusters
 # that end in the fold
-@pytest.mark.parametrize("n", [32767, 65533, 65540, 131071, 131072, 131073])
+@pytest.mark.parametrize("n", [32767, 65533, 65540, 131073, 262143, 262144, 262145])
 def test_folds_of_few_elements(n):
     assert check_program(W.config1(n), runs=2) == 8
 

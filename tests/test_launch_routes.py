@@ -214,11 +214,11 @@ for n in (1 << 18, 1 << 27, 1 << 30):
 def test_few_elements_are_folded_by_one_cluster_of_blocks(child):
     """... counted over all arrays that are read or stored (the third cluster reads two); a gather below the fold keeps the grid."""
     got = child("""
-result = [[k[0], k[2]] for n in (131072, 131073) for k in launches(W.config1(n))]
-result += [launches(W.config1(n), [-1, 0, 0, 0, 1])[1][0] for n in (131072, 131073)]
-result += [launches(W.config1(n), [-1, 0, 0, 1, 1])[1][0] for n in (65536, 65537)]
+result = [[k[0], k[2]] for n in (262144, 262145) for k in launches(W.config1(n))]
+result += [launches(W.config1(n), [-1, 0, 0, 0, 1])[1][0] for n in (262144, 262145)]
+result += [launches(W.config1(n), [-1, 0, 0, 1, 1])[1][0] for n in (131072, 131073)]
 """)
-    assert got == [["k_stream_few", 8], ["k_stream", 128]] + ["k_stream_few", "k_stream"] * 2
+    assert got == [["k_stream_few", 8], ["k_stream", 256]] + ["k_stream_few", "k_stream"] * 2
 
 
 def test_few_tiles_are_folded_by_clusters_of_blocks(child):
