@@ -230,12 +230,16 @@ struct Launcher {
           const int warps = dev::kBlock / 32;
           dev::k_scan_rows<CL, 1, 4><<<(int)std::min<int64_t>((R + warps - 1) / warps, (int64_t)sm_count() * 8), dev::kBlock, 0, L.stream>>>(a);
         } else if (C <= dev::kScanBlockRow) {
-          const int grid = (int)std::min<int64_t>(R, (int64_t)sm_count() * 8);
           // (a thread's chunks are all under way together, those beyond the row's end for nothing: rows of 5000 in sixteen warps
-          // of four chunks 19.5 us for 2000 of them, of eight 29.7)
-          if (C <= 4096 - 3) dev::k_scan_rows<CL, 16, 2><<<grid, 512, 0, L.stream>>>(a);
-          else if (C <= 8192 - 3) dev::k_scan_rows<CL, 16, 4><<<grid, 512, 0, L.stream>>>(a);
-          else dev::k_scan_rows<CL, 16, 8><<<grid, 512, 0, L.stream>>>(a);
+          // of four chunks 19.5 us for 2000 of them, of eight 29.7; and a warp beyond the row's end takes another block's place: as
+          // many warps as have chunks instead of sixteen, two scans of 4099 x 3001 45.1 -> 39.0 us, 8000 x 1200 66.9 -> 28.7, 2443 x 5825 53.3 ->
+          // 45.1, 3000 x 9000 92.1 -> 71.5)
+          const int chunks = C <= 4096 - 3 ? 2 : C <= 8192 - 3 ? 4 : 8;
+          const int warps = (C + (R > 1 && C % 4 ? 3 : 0) + chunks * 128 - 1) / (chunks * 128);
+          const int grid = (int)std::min<int64_t>(R, (int64_t)sm_count() * 16);
+          if (chunks == 2) dev::k_scan_rows<CL, 16, 2><<<grid, warps * 32, 0, L.stream>>>(a);
+          else if (chunks == 4) dev::k_scan_rows<CL, 16, 4><<<grid, warps * 32, 0, L.stream>>>(a);
+          else dev::k_scan_rows<CL, 16, 8><<<grid, warps * 32, 0, L.stream>>>(a);
         }
       }
       if constexpr ((kForms & 2) != 0 && kRingServes) {

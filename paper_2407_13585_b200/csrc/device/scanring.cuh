@@ -950,8 +950,8 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
 }
 
 // =========================================================================================
-// WARPS warps per row (one: kBlock / 32 rows to a block), CH chunks of four per lane at a time: all of a row's loads are
-// under way together, which is what bounds these rows.  Rows longer than WARPS * CH * 128 elements take several such spans
+// A warp per row (WARPS = 1: kBlock / 32 rows to a block), or a block per row with as many warps as the row has work for, up to WARPS;
+// CH chunks of four per lane at a time: all of a row's loads are under way together, which is what bounds these rows.  Rows longer than WARPS * CH * 128 elements take several such spans
 // (one warp only).
 template <class CL, int WARPS, int CH>
 __global__ void __launch_bounds__(WARPS == 1 ? kBlock : WARPS * 32, WARPS == 1 ? 1 : CH == 2 ? 3 : 2) k_scan_rows(const __grid_constant__ Args<CL::c.n> a) {
@@ -959,7 +959,7 @@ __global__ void __launch_bounds__(WARPS == 1 ? kBlock : WARPS * 32, WARPS == 1 ?
   constexpr bool REV = CL::c.nodes[first_scan<CL>()].kind == ACC_SCANR;
   __shared__ uint32_t warp_total[2][NS][WARPS];
   const int lane = threadIdx.x & 31, mem_lane = REV ? 31 - lane : lane;
-  const int warp = WARPS == 1 ? 0 : (int)threadIdx.x >> 5, mem_warp = REV ? WARPS - 1 - warp : warp;
+  const int warp = WARPS == 1 ? 0 : (int)threadIdx.x >> 5, mem_warp = WARPS > 1 && REV ? (int)blockDim.x / 32 - 1 - warp : warp;
   const int n = a.C;
   int half = 0;                                                       // which half of warp_total this row uses
   for (int row = blockIdx.x * ROWS + (WARPS == 1 ? (int)threadIdx.x >> 5 : 0); row < a.R; row += gridDim.x * ROWS, half ^= 1) {

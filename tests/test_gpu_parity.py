@@ -791,6 +791,13 @@ def test_scans_on_a_device_without_cooperative_launches(tmp_path):
     assert child.returncode == 0 and child.stdout.endswith("done\n"), child.stderr[-2000:]
 
 
+# a block per row with as many warps as the row has chunks for: the last warp full, with one element, one warp more; rows that begin
+# up to three words into a chunk, and rows that do not; in both directions
+@pytest.mark.parametrize("cols", [1025, 1277, 1278, 1280, 1281, 3069, 3070, 4094, 4605, 4606, 8190, 9213, 9214, 9216])
+def test_rows_by_as_many_warps_as_they_have_chunks_for(cols):
+    check_program(W.row_scans(5, cols), [[-1, 0, 1, 1]])
+
+
 @pytest.mark.parametrize("n", [1, 6, 4096, 100001, 1 << 18])
 def test_right_to_left_scan_int32(n):
     check_program(W.suffix_sums(n))

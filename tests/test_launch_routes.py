@@ -108,6 +108,13 @@ result = [launches(W.row_scans(10, cols), [-1, 0, 1, 1])[0][:2] for cols in (102
     assert [g[1].split(", ", 1)[1] for g in got] == ["1, 4>", "16, 2>", "16, 2>", "16, 4>", "16, 4>", "16, 8>", "16, 8>"]
 
 
+def test_a_block_has_as_many_warps_as_a_row_has_chunks_for(child):
+    got = child("""
+result = [launches(W.row_scans(10, cols), [-1, 0, 1, 1])[0][3] // 32 for cols in (1025, 1277, 1278, 1280, 4093, 4094, 4605, 4606, 8189, 8190, 9213, 9214, 16381)]
+""")
+    assert got == [5, 5, 6, 5, 16, 9, 9, 10, 16, 9, 9, 10, 16]
+
+
 STATUS = """
 def finish(g, workspace):
     return lib.acc_finish(g._h, C.c_void_p(workspace), None)
