@@ -50,6 +50,11 @@ def _headers_mtime():
     return max(m, os.path.getmtime(os.path.abspath(__file__)))
 
 
+# Device code of the test suite's own kernels is stored compressed: they outnumber the library's four to one (353 MB as they are, 47 MB
+# compressed), and a tree that is copied to another machine with its built files has to stay small.  The library itself is not:
+# what is compressed has to be unpacked by the process that first launches it.
+TEST_FLAGS = ["--compress-mode=size"]
+
 CLUSTERS_PER_PART = 10      # clusters one compiler run instantiates
 
 
@@ -73,8 +78,8 @@ def _jobs(srcs, name_of, force, hdr):
     return objs, sorted(jobs, key=lambda j: -os.path.getsize(j[0]) / j[3])
 
 
-def _compile(src, obj, part, parts, verbose):
-    cmd = ["nvcc"] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-x", "cu", "-c", src, "-o", obj]
+def _compile(src, obj, part, parts, flags, verbose):
+    cmd = ["nvcc"] + NVCC_FLAGS + list(flags) + (["-Xptxas", "-v"] if verbose else []) + ["-x", "cu", "-c", src, "-o", obj]
     if parts > 1:
         cmd += ["-DACC_PARTS=%d" % parts, "-DACC_PART=%d" % part]
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -89,7 +94,7 @@ def build(force=False, verbose=False):
     hdr = _headers_mtime()
     objs, jobs = _jobs(_sources(), lambda src: os.path.relpath(src, CSRC).replace(os.sep, "_"), force, hdr)
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as pool:
-        list(pool.map(lambda j: _compile(*j, verbose), jobs))
+        list(pool.map(lambda j: _compile(*j, (), verbose), jobs))
     if jobs or not os.path.exists(LIB):
         cmd = ["nvcc", "-shared", "-o", LIB] + objs + ["-lcudart"]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -98,16 +103,17 @@ def build(force=False, verbose=False):
     return LIB
 
 
-def build_kernel_library(src_dir, lib_path, force=False, verbose=False):
+def build_kernel_library(src_dir, lib_path, force=False, verbose=False, flags=()):
     """Compiles every .cu under src_dir into lib_path, a shared object of further kernel instantiations
-    that resolves the registry and the launch helpers from libacc.so (found next to this file at run time)."""
+    that resolves the registry and the launch helpers from libacc.so (found next to this file at run time).
+    flags: further arguments of the compiler."""
     build(force=False, verbose=verbose)
     os.makedirs(OBJ, exist_ok=True)
     hdr = _headers_mtime()
     tag = os.path.basename(lib_path).replace(".so", "")
     objs, jobs = _jobs(_sources(src_dir), lambda src: tag + "_" + os.path.relpath(src, src_dir).replace(os.sep, "_"), force, hdr)
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as pool:
-        list(pool.map(lambda j: _compile(*j, verbose), jobs))
+        list(pool.map(lambda j: _compile(*j, flags, verbose), jobs))
     if jobs or not os.path.exists(lib_path) or os.path.getmtime(lib_path) < os.path.getmtime(LIB):
         rpath = os.path.relpath(HERE, os.path.dirname(lib_path))
         cmd = ["nvcc", "-shared", "-o", lib_path] + objs + ["-L" + HERE, "-lacc", "-lcudart",
@@ -119,7 +125,7 @@ def build_kernel_library(src_dir, lib_path, force=False, verbose=False):
 
 
 def build_test_kernels(force=False, verbose=False):
-    return build_kernel_library(TEST_SRC, TEST_LIB, force, verbose)
+    return build_kernel_library(TEST_SRC, TEST_LIB, force, verbose, TEST_FLAGS)
 
 
 if __name__ == "__main__":

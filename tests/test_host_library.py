@@ -457,3 +457,10 @@ def test_spin_limit_is_a_property_of_the_graph():
     g.set_spin_limit(0)
     g.set_spin_limit(1 << 22)
     assert B.lib().acc_set_spin_limit(None, 5) == B.lib().acc_launch_count(None)      # both refuse a null graph with ACC_ERR_ARG
+
+
+def test_built_libraries_stay_small():
+    # a copy of the tree takes them along to the machine with the GPU, where copies of more than 512 MB are refused; half of that
+    # is left to what lies beside them (353 + 101 MB before the test kernels were compressed)
+    from paper_2407_13585_b200 import build
+    assert os.path.getsize(build.LIB) + os.path.getsize(build.TEST_LIB) < 256 << 20
