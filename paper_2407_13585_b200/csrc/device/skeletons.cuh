@@ -272,6 +272,36 @@ __global__ void __launch_bounds__(kBlock) k_stream(const __grid_constant__ Args<
   }
 }
 
+// Partial sums that the blocks of a thread-block cluster leave in the shared memory of its first.  That memory may be written to
+// once the block that owns it is known to have started (that all are scheduled together does not say so), and read once all have
+// written.  A kernel arrives with its first statement and waits in front of its first write, so that the walk lies between the two;
+// writing takes what that wait returns.  All threads of all blocks take every step.
+class FirstBlock {
+ public:
+  class Open {
+   public:
+    // `word`: this block's address of a word that lies at the same place in the first block
+    __device__ __forceinline__ void put(uint32_t* word, uint32_t v) const {
+      uint32_t there;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(there) : "r"((uint32_t)__cvta_generic_to_shared(word)));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(there), "r"(v) : "memory");
+    }
+    __device__ __forceinline__ void all_have_written() const {
+      __syncwarp();                                      // (an aligned barrier is for the whole warp together)
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+   private:
+    friend class FirstBlock;
+    __device__ __forceinline__ Open() {}
+  };
+  __device__ __forceinline__ FirstBlock() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+  __device__ __forceinline__ Open all_have_started() const {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return Open();
+  }
+};
+
 // Folds of few elements: one cluster of blocks, which leave their partial sums in the shared memory of the first, so that there
 // is no counter to clear beforehand (a second thing to launch) and none to go round.  What bounds such calls is how often
 // something is launched and waited for: the chain of 2^16 elements, one run after another, 8.2 -> 4.8 us, waited for 16.5 -> 13.1;
@@ -293,6 +323,7 @@ template <class CL> constexpr int few_arrays() {         // read or written elem
 }
 template <class CL, bool VEC>
 __global__ void __cluster_dims__(kFewBlocks, 1, 1) __launch_bounds__(kFewThreads) k_stream_few(const __grid_constant__ Args<CL::c.n> a) {
+  const FirstBlock first;
   constexpr int N = CL::c.n;
   constexpr int NF = count_if<CL>(is_scalar_fold);
   __shared__ uint32_t red[kFewThreads / 32];
@@ -305,19 +336,16 @@ __global__ void __cluster_dims__(kFewBlocks, 1, 1) __launch_bounds__(kFewThreads
     if constexpr (is_scalar_fold(nd)) acc[i] = identity_of<nd.fn, nd.dtype>();
   });
   stream_walk<CL, VEC, kFewThreads>(a, acc, comp, nullptr);
+  const FirstBlock::Open open = first.all_have_started();
   static_for<0, N>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     constexpr CNode nd = CL::c.nodes[i];
     if constexpr (is_scalar_fold(nd)) {
       const uint32_t v = block_reduce_n<nd.fn, nd.dtype, kFewThreads>(acc[i], red);
-      if (threadIdx.x == 0) {
-        uint32_t first;                                  // the word in the first block's shared memory
-        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(first) : "r"((uint32_t)__cvta_generic_to_shared(&part[count_if<CL>(is_scalar_fold, i)][blockIdx.x])));
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(first), "r"(v) : "memory");
-      }
+      if (threadIdx.x == 0) open.put(&part[count_if<CL>(is_scalar_fold, i)][blockIdx.x], v);
     }
   });
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  open.all_have_written();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     static_for<0, N>([&](auto ic) {
       constexpr int i = decltype(ic)::value;

@@ -299,6 +299,7 @@ template <class CL> constexpr bool tile_rows_eligible() {
 }
 template <class CL, bool VEC>
 __global__ void __cluster_dims__(kTrBlocks, 1, 1) __launch_bounds__(kBlock) k_tile_rows(const __grid_constant__ Args<CL::c.n> a) {
+  const FirstBlock first;
   constexpr int N = CL::c.n;
   constexpr int NRF = count_if<CL>(is_row_fold), E = staged_externals<CL>();
   extern __shared__ __align__(16) uint32_t tiles[];
@@ -361,6 +362,7 @@ __global__ void __cluster_dims__(kTrBlocks, 1, 1) __launch_bounds__(kBlock) k_ti
     }
     __syncthreads();                                        // (the next tile takes this one's place)
   }
+  const FirstBlock::Open open = first.all_have_started();
   static_for<0, N>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     constexpr CNode nd = CL::c.nodes[i];
@@ -371,15 +373,11 @@ __global__ void __cluster_dims__(kTrBlocks, 1, 1) __launch_bounds__(kBlock) k_ti
         uint32_t s = row_part[i][j];
 #pragma unroll
         for (int w = 8; w > 0; w >>= 1) s = combine<nd.fn, nd.dtype>(s, __shfl_xor_sync(0xFFFFFFFFu, s, w));
-        if (cx == 0) {
-          uint32_t first;                                   // the word in the first block's shared memory
-          asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(first) : "r"((uint32_t)__cvta_generic_to_shared(&part[ord][rank][4 * rg + j])));
-          asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(first), "r"(s) : "memory");
-        }
+        if (cx == 0) open.put(&part[ord][rank][4 * rg + j], s);
       }
     }
   });
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  open.all_have_written();
   if (rank == 0 && threadIdx.x < kTile && I * kTile + (int)threadIdx.x < n) {
     static_for<0, N>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
