@@ -129,10 +129,12 @@ struct Launcher {
   static constexpr int kRowFolds = dev::count_if<CL>(dev::is_row_fold);
 
   // ... or, where there are few (and more than one), by a cluster of blocks to every block of rows (k_tile_rows, where both sides'
-  // times are; ahead up to 3000 rows at least, but from 2560 on the array is 26 MB and more, and what a program's other arrays leave of
-  // the L2 decides)
+  // times are).  Two arrays, up to 33 blocks of rows: with two blocks per SM 33 clusters run at once, a 34th afterwards (us, the pair kernels /
+  // this one: 2048 rows 14.4 / 11.4, 2111 21.9 / 16.4, 2112 14.3 / 13.0; 2176 14.3 / 18.4, 2177 21.5 / 23.6, 2559 20.5 / 28.3).  One array,
+  // up to 2559 rows: it stays ahead to about 3100 (2624 rows 16.4 / 12.3, 3000 16.4 / 14.2, 3100 18.3 / 16.4, 3300 17.6 / 18.5), measured
+  // with nothing else in the L2; where other arrays go through it between two runs is not measured there.
   static constexpr bool kTileRowsShape = dev::tile_rows_eligible<CL>();
-  static constexpr int kTileRowsMost = 2559;
+  static constexpr int kTileRowsMost = dev::staged_externals<CL>() == 1 ? 2559 : 33 * dev::kTile;
   static bool use_tile_rows(int n) { return kTileRowsShape && n > dev::kTile && n <= kTileRowsMost; }
 
   // The tile-pair kernel wants a square domain of at least one tile, and every staged

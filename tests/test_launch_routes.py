@@ -235,6 +235,14 @@ result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][:3:2] for rows in (63, 64,
     assert got == [["k_rowfold", 63], ["k_tile_pair_tma", 1], ["k_tile_rows", 16], ["k_tile_rows", 16], ["k_tile_rows", 24], ["k_tile_rows", 320]]
 
 
+def test_two_arrays_are_folded_by_clusters_of_blocks_while_these_run_all_at_once(child):
+    """... which 34 blocks of rows with two arrays' tiles do not (2176 rows: 18.4 us, by pairs of tiles 14.3)."""
+    got = child("""
+result = [launches(W.diagonal_of_product(rows), [-1, -1, 0, 0, 0])[0][0] for rows in (65, 2111, 2112, 2113, 2176, 2559)]
+""")
+    assert got == ["k_tile_rows"] * 3 + ["k_tile_pair", "k_tile_pair_tma", "k_tile_pair"]
+
+
 def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
     got = child("""
 result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
