@@ -98,11 +98,16 @@ __device__ __forceinline__ int seg_containing(const int32_t* off, int S, int x, 
 }
 
 // ---- operands that land in shared memory before they are wanted ------------------------------------------------
-// Folds whose operands are computed from one array, element by element, have a warp's next two steps of that array under way
+// Several folds whose operands are computed from one array, element by element, have a warp's next two steps of that array under way
 // in asynchronous copies, straight to where a lane finds its 16 consecutive elements: no step waits for memory, no operand is
 // written to shared memory to be read again in another order, and no registers hold what another fold will need.  Two steps of
 // 2 KB a warp are what four blocks per SM have room for; three steps and three blocks 174 against 156 us (2^27 elements,
-// Zipf lengths).  The search for a run's first segment comes before the first copies: behind them its loads wait (164 -> 172 us).
+// Zipf lengths).  The search for a run's first segment comes behind the first copies: in front of them 50.2 -> 50.6 us for 5 * 10^7
+// elements in 16 segments, 53.4 -> 54.5 in 5000, 19.0 -> 20.0 for 5 * 10^6 in 10^4, but 186.9 -> 186.8 for 2^27 in 2.7 * 10^6.
+// One fold alone takes its operands through registers: it has them all before it begins, and the 128 KB per SM that copies would
+// land in are worth more as L1 to the offsets, which are read three times (us, landed / registers: 2^27 elements in segments of 4
+// 428 / 397, of 16 193 / 179, of 500 101 / 102; 5 * 10^7 in segments of 2.5 248 / 232, of 500 46.4 / 48.0; 2 * 10^7 in 6 segments
+// 23.6 / 19.4).
 struct IxLd4 { int r, c; const uint32_t* landed; };                 // four consecutive elements, and where their array's lie
 __device__ __forceinline__ Ix lane(const IxLd4& i, int j) { return Ix{i.r, i.c + j}; }
 template <int F, int P0 = kRunTime, int P1 = kRunTime>
@@ -125,6 +130,7 @@ template <class CL> constexpr int seg_array_below(int i, int so_far) {
   return so_far;
 }
 template <class CL> constexpr int seg_landing_array() {
+  if (count_if<CL>(is_segfold_root) < 2) return -2;
   int x = -1;
   for (int i = 0; i < CL::c.n; ++i)
     if (is_segfold_root(CL::c.nodes[i])) x = seg_array_below<CL>(CL::c.nodes[i].in[0], x);

@@ -22,6 +22,7 @@ static int n_pages = 0;
 static uint32_t* status_words = nullptr;     // of the last launch: where its arguments say that it reports, and as which run
 static uint32_t status_run = 0;
 static int32_t second[8];                    // of the last launch of k_hist: its second argument's first words
+static size_t seg_shared = 0;                // of the last launch of k_segfold: bytes of shared memory asked for
 
 static int note(const void* kernel, dim3 grid, dim3 block, void** args, bool coop) {
   if (launches.size() > (1u << 20)) launches.clear();
@@ -71,6 +72,7 @@ void fake_destroy_graph() {
 void fake_clear() { launches.clear(); }
 const char* fake_launches() { return launches.c_str(); }
 const int32_t* fake_second_argument() { return second; }
+size_t fake_seg_shared() { return seg_shared; }
 int fake_pages() { return n_pages; }
 uint32_t* fake_status(uint32_t* run) { *run = status_run; return status_words; }
 
@@ -139,6 +141,11 @@ int cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, int* fou
   if (found) *found = 0;
   return 0;
 }
-int cudaLaunchKernel(const void* kernel, dim3 grid, dim3 block, void** args, size_t, void*) { return note(kernel, grid, block, args, false); }
+int cudaLaunchKernel(const void* kernel, dim3 grid, dim3 block, void** args, size_t shared, void*) {
+  note(kernel, grid, block, args, false);
+  const size_t line = launches.rfind('\n', launches.size() - 2) + 1;      // (npos + 1: the first)
+  if (launches.find("k_segfold<", line) != std::string::npos) seg_shared = shared;
+  return 0;
+}
 int cudaLaunchCooperativeKernel(const void* kernel, dim3 grid, dim3 block, void** args, size_t, void*) { return note(kernel, grid, block, args, true); }
 }

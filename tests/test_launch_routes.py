@@ -243,6 +243,18 @@ result = [launches(W.diagonal_of_product(rows), [-1, -1, 0, 0, 0])[0][0] for row
     assert got == ["k_tile_rows"] * 3 + ["k_tile_pair", "k_tile_pair_tma", "k_tile_pair"]
 
 
+def test_one_segmented_fold_alone_takes_its_operands_through_registers(child):
+    """Two that share the walk have them land in shared memory: eight warps, two steps of 2 KB each."""
+    got = child("""
+fake.fake_seg_shared.restype = C.c_size_t
+result = []
+for pi in ([-1, -1, 0, 0, 0], [-1, -1, 0, 0, 1], [-1, -1, 0, 1, 2]):
+    launches(W.segmented_sums(10**6, 10**5), pi)
+    result.append(fake.fake_seg_shared())                     # of the last cluster's
+""")
+    assert got == [8 * 2 * 2048, 0, 0]
+
+
 def test_unaligned_tile_pairs_are_copied_from_2720_rows_on(child):
     got = child("""
 result = [launches(W.config2(rows), [-1, 0, 0, 0])[0][0] for rows in (2561, 2719, 2721, 64, 2560)]
