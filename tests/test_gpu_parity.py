@@ -78,6 +78,54 @@ def test_row_folds_by_clusters_of_blocks(rows):
     check_program(W.diagonal_of_product(rows), [[-1, -1, 0, 0, 0]], runs=2)
 
 
+# ... two arrays: the most rows, without 128-bit rows and with
+@pytest.mark.parametrize("rows", [2111, 2112])
+def test_row_folds_of_two_arrays_by_clusters_of_blocks(rows):
+    check_program(W.diagonal_of_product(rows), [[-1, -1, 0, 0, 0]], runs=2)
+
+
+# ... of integers, maxima and minima, one fold and two in a cluster
+@pytest.mark.parametrize("rows", [65, 128, 577, 520])
+@pytest.mark.parametrize("which", [0, 1, 2, 3])
+def test_row_folds_of_any_operator_by_clusters_of_blocks(which, rows):
+    prog = W.transposed_folds(which, rows)
+    check_program(prog, [[-1] + [0] * (len(prog.nodes) - 1)], runs=2)
+
+
+@pytest.mark.parametrize("rows", [130, 577])
+def test_row_folds_of_infinities_and_nans_by_clusters_of_blocks(rows):
+    """A sum is infinite or not a number where its terms make it so, a maximum or minimum takes no notice of what is not a number
+    and may be infinite throughout a row."""
+    import torch
+    from paper_2407_13585_b200 import binding as B
+    inf, nan = float("inf"), float("nan")
+
+    def folded(which, values):
+        prog = W.transposed_folds(which, rows)
+        inputs = W.make_inputs(prog)
+        for (r, c), v in values.items():
+            inputs[0][r, c] = v
+        got, g = gpu_run(prog, inputs, [-1] + [0] * (len(prog.nodes) - 1), B.FUSED)
+        assert g.launch_count() == 1
+        a = inputs[0].numpy()
+        with np.errstate(invalid="ignore"):
+            return got, a + a.T
+
+    got, terms = folded(3, {(5, 7): inf, (20, rows - 1): -inf, (40, 41): nan, (70, 70): inf, (70, 71): -inf, (90, 3): inf, (90, 4): inf})
+    with np.errstate(invalid="ignore"):
+        want = terms.astype(np.float64).sum(axis=1)
+    finite = np.isfinite(want)
+    assert np.isinf(want).any() and np.isnan(want).any() and finite.any()
+    assert np.array_equal(np.where(finite, 0.0, got[3]), np.where(finite, 0.0, want), equal_nan=True)
+    # the bound of an fp32 sum that the other tests use: 1e-5 of the sum of magnitudes
+    assert np.all(np.abs(got[3][finite] - want[finite]) <= 1e-5 * np.abs(terms[finite]).astype(np.float64).sum(axis=1))
+    values = {(5, 7): inf, (40, 41): nan, (64, 64): nan, (rows - 1, 2): -inf}
+    values.update({(9, c): -inf for c in range(rows)})
+    got, terms = folded(1, values)
+    assert np.all(terms[9] == -inf) and np.isnan(terms).sum() == 3
+    assert np.array_equal(got[3], np.fmax.reduce(terms, axis=1)) and np.array_equal(got[4], np.fmin.reduce(terms, axis=1))
+
+
 # iterates kept on chip, tiles inside the array beside tiles at its edges: box rows that are a multiple of three and not (two, three
 # and four iterations), copied as boxes and word by word
 @pytest.mark.parametrize("rows,cols,iters", [(1026, 640, 2), (1026, 641, 2), (4300, 392, 2), (900, 1028, 3), (900, 1027, 3), (900, 1028, 4), (901, 1030, 4)])
@@ -490,9 +538,8 @@ def compare_hist(prog, ref, got, what):
 @pytest.mark.parametrize("n,segments", [(5, 1), (64, 5), (1000, 16), (100000, 300), (1 << 20, 1 << 12), (1 << 20, 6), (1 << 22, 1 << 18),
                                         ((1 << 21) + 3, 1 << 10)])
 def test_segmented_fold(n, segments):
-    # the source is walked in tiles of 4096 elements; pieces of segments by a thread, a warp or the block according to
-    # their length; segments that cross tiles and blocks; a sum fed by a fused map and a maximum sharing the same walk;
-    # a source without 128-bit rows (the last shape)
+    # the source is walked by warps, 512 elements at a time, up to 4096 each; segments that cross steps, warps and blocks; a sum fed
+    # by a fused map and a maximum sharing the same walk; a source without 128-bit rows (the last shape)
     from paper_2407_13585_b200 import binding as B
     prog = W.segmented_sums(n, segments)
     runnable = [pi for pi in all_partitions(prog) if pi != [-1, -1, 0, 1, 0]]
@@ -541,7 +588,8 @@ def test_segmented_fold_with_skewed_and_awkward_segments():
                                         (1 << 22, 1), ((1 << 22) + 1029, 2), (148 * 32 * 512 * 4 + 3, 40)])
 def test_segmented_fold_by_warps(n, segments):
     """A warp's run is one step of 512 elements, or several; segments of one element, more than a step's worth of offsets at
-    a time, lengths whose last chunk of four is not whole; segments of many steps, two at a time, and across hundreds of blocks."""
+    a time, lengths whose last chunk of four is not whole; segments of many steps (two at a time where a fold is alone), and across
+    hundreds of blocks."""
     assert check_program(W.segmented_sums(n, segments), [[-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2]]) == 2
 
 
@@ -556,6 +604,21 @@ def test_segmented_fold_of_part_of_the_source(n, lo, hi):
     inputs = W.make_inputs(prog)
     inputs[1] = torch.from_numpy(np.linspace(lo, hi, segments + 1).astype(np.int32))
     check_program(prog, [[-1, -1, 0, 0, 0], [-1, -1, 0, 0, 1]], inputs_t=inputs, runs=2)
+
+
+# operands that do not land ahead: of two arrays, of one read backwards (with 128-bit rows and without), and one that lands beside
+# a generated one; folds that share the walk and folds alone; short segments, a long one, a part of the source only
+@pytest.mark.parametrize("n,lo,hi,segments", [(70001, 0, 70001, 3000), (70004, 513, 69990, 200), (20003, 7, 19990, 9000), (20004, 0, 20004, 20004),
+                                              (300004, 5, 299000, 2), (300003, 4096, 300003, 1), (5, 1, 5, 2)])
+def test_segmented_folds_of_other_operands(n, lo, hi, segments):
+    import torch
+    offsets = torch.from_numpy(np.linspace(lo, hi, segments + 1).astype(np.int32))
+    for prog, partitions in ((W.segmented_products(n, segments), ([-1, -1, -1, 0, 0, 0], [-1, -1, -1, 0, 1, 1], [-1, -1, -1, 0, 1, 2])),
+                             (W.segmented_reversed(n, segments), ([-1, -1, 0, 0, 0], [-1, -1, 0, 1, 2])),
+                             (W.segmented_weights(n, segments), ([-1, -1, 0, 0, 0, 0], [-1, -1, 0, 0, 0, 1]))):
+        inputs = W.make_inputs(prog)
+        inputs[prog.id("offsets")] = offsets
+        check_program(prog, list(partitions), inputs_t=inputs, runs=2)
 
 
 @pytest.mark.parametrize("tail", [0, 3])

@@ -318,6 +318,58 @@ def diagonal_of_product(rows=256):
     return Program("diagonal_of_product", nodes, [4])
 
 
+def transposed_folds(which=0, rows=256):
+    """Folds of the rows of A + transpose A: which = 0 sum and maximum of int32, 1 maximum and minimum of fp32, 2 minimum of
+    uint32, 3 the sum of fp32."""
+    dtype, ops = [("i32", ("add", "max")), ("f32", ("max", "min")), ("u32", ("min",)), ("f32", ("add",))][which]
+    sh = (rows, rows)
+    nodes = [
+        _inp("A", dtype, sh),
+        Node("backpermute", dtype, sh, (0,), 1, idx_fn="transpose", name="B"),
+        Node("zipwith", dtype, sh, (0, 1), 2, fn="add", name="C"),
+    ]
+    nodes += [Node("fold", dtype, (rows,), (2,), 1, fn=op, name="row_" + op) for op in ops]
+    return Program("transposed_folds_%d" % which, nodes, list(range(3, len(nodes))), index_bound={"A": 1 << 30})
+
+
+def segmented_products(n=1 << 10, segments=16):
+    """Sums and maxima of segments of the product of two arrays."""
+    nodes = [
+        _inp("xs", "f32", (n,)),
+        _inp("ys", "f32", (n,)),
+        _inp("offsets", "i32", (segments + 1,)),
+        Node("zipwith", "f32", (n,), (0, 1), 2, fn="mul", name="w"),
+        Node("foldseg", "f32", (segments,), (3, 2), 1, fn="add", name="sums"),
+        Node("foldseg", "f32", (segments,), (3, 2), 1, fn="max", name="maxes"),
+    ]
+    return Program("segmented_products", nodes, [4, 5])
+
+
+def segmented_reversed(n=1 << 10, segments=16):
+    """Sums and minima of segments of an array read backwards."""
+    nodes = [
+        _inp("xs", "f32", (n,)),
+        _inp("offsets", "i32", (segments + 1,)),
+        Node("backpermute", "f32", (n,), (0,), 1, idx_fn="reverse", name="r"),
+        Node("foldseg", "f32", (segments,), (2, 1), 1, fn="add", name="sums"),
+        Node("foldseg", "f32", (segments,), (2, 1), 1, fn="min", name="mins"),
+    ]
+    return Program("segmented_reversed", nodes, [3, 4])
+
+
+def segmented_weights(n=1 << 10, segments=16):
+    """Segmented sums of an array weighted by its own indices, beside its segments' maxima."""
+    nodes = [
+        _inp("xs", "f32", (n,)),
+        _inp("offsets", "i32", (segments + 1,)),
+        Node("generate", "f32", (n,), (), 0, fn="imod_to_f32", iparam=(7,), name="g"),
+        Node("zipwith", "f32", (n,), (0, 2), 2, fn="mul", name="w"),
+        Node("foldseg", "f32", (segments,), (3, 1), 1, fn="add", name="sums"),
+        Node("foldseg", "f32", (segments,), (0, 1), 1, fn="max", name="maxes"),
+    ]
+    return Program("segmented_weights", nodes, [4, 5])
+
+
 def random_scan_program(seed, n=4099, rows=0):
     """A seeded random DAG around a scan in the middle: element-wise nodes and reversals before it, then nodes
     that may read the scan (directly, or through a reversal, which no kernel follows inside a cluster), then
