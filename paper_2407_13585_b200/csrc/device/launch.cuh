@@ -448,9 +448,10 @@ struct Launcher {
   static int launch_tiles_tma(const ClusterLaunch& L, dev::Args<N>& a, int n, bool vec) {
     if constexpr (dev::tile_tma_eligible<CL>()) {
       if (!cooperative_launch_ok()) return 1;
-      // (word-by-word copies and the meeting at the end pay from here on; us staged by threads against copied, one array and
-      // two: 2561 rows 18.7 / 20.5 and 23.3 / 28.7, 2701 20.0 / 22.5 and 27.3 / 28.7, 2749 20.1 / 18.4 and 28.5 / 22.6, 2851 22.4 / 20.5
-      // and 30.6 / 26.6, 4001 32.0 / 26.8 and 71.8 / 52.2)
+      // (word-by-word copies and the meeting at the end pay from about here on, for two arrays more than for one; us staged by threads
+      // against copied, one array and two: 2561 rows 18.3 / 20.5 and 22.7 / 28.7, 2717 18.4 / 20.5 and 25.6 / 26.7, 2721 18.4 / 20.5 and
+      // 25.7 / 26.6, 2749 18.4 / 18.5 and 25.5 / 22.5, 2901 20.4 / 20.5 and 27.8 / 28.9, 3001 20.5 / 18.5 and 28.7 / 24.6, 3101 20.5 / 22.5
+      // and 28.7 / 30.7, 3501 23.9 / 24.0 and 42.7 / 39.1)
       if (!vec && n < 2720) return 1;
       dev::TileMaps maps;
       for (int i = 0; i < N; ++i)

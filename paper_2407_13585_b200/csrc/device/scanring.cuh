@@ -951,8 +951,9 @@ __global__ void __launch_bounds__((Ring<CL, RESIDENT>::THREADS), 1) k_scan_ring(
 
 // =========================================================================================
 // A warp per row (WARPS = 1: kBlock / 32 rows to a block), or a block per row with as many warps as the row has work for, up to WARPS;
-// CH chunks of four per lane at a time: all of a row's loads are under way together, which is what bounds these rows.  Rows longer than WARPS * CH * 128 elements take several such spans
-// (one warp only).
+// CH chunks of four per lane at a time: all of a row's loads are under way together, which is what bounds these rows.  A warp takes a
+// longer row in several spans; a block takes its row in one, so whoever launches it sees to it that its warps cover the row
+// and the up to three words of its first chunk that precede it: blockDim.x / 32 * CH * 128 >= C + 3 (C, where rows start on 16 bytes).
 template <class CL, int WARPS, int CH>
 __global__ void __launch_bounds__(WARPS == 1 ? kBlock : WARPS * 32, WARPS == 1 ? 1 : CH == 2 ? 3 : 2) k_scan_rows(const __grid_constant__ Args<CL::c.n> a) {
   constexpr int N = CL::c.n, NS = count_if<CL>(is_scan_root), SPAN = WARPS * CH * 128, ROWS = WARPS == 1 ? kBlock / 32 : 1;

@@ -5,7 +5,7 @@
 // The work is cut by elements, not by segments, so that a few very long segments among many
 // short ones (skewed lengths) cost what their elements cost:
 //
-//  * a warp owns kSegRun consecutive elements and walks them 512 at a time, without a barrier: the
+//  * a warp owns up to kSegMaxRun consecutive elements (seg_run) and walks them 512 at a time, without a barrier: the
 //    warps of a block meet once, at the end;
 //  * where no segment begins among the 512, every lane adds its elements to a compensated running
 //    value of its own;
@@ -21,7 +21,7 @@
 // (A block that walked tiles of 4096 elements with ten barriers each took 243 us for a sum and a maximum of 2^27 elements in 2^20
 // segments of Zipf lengths, 184 in 2^15 segments, 450 in 2^24, 42.5 for 10^6 in 10^4.  Warps on their own, with loads into
 // registers ahead of a step's work, 176, 144, 407 and 17.1; with operands that land in shared memory two steps ahead, below, and
-// without records cleared beforehand, 156, 130, 405 and 13.7: 51 % of the issue slots, the rest mostly a warp's waits for offsets
+// without records cleared beforehand, 156, 130, 405 and 13.7: 53 % of the issue slots, the rest mostly a warp's waits for offsets
 // and for the shuffles of its scan.)
 //
 // Several segmented folds of one cluster (say a sum and a maximum over the same segments) share

@@ -306,7 +306,8 @@ class FirstBlock {
 // is no counter to clear beforehand (a second thing to launch) and none to go round.  What bounds such calls is how often
 // something is launched and waited for: the chain of 2^16 elements, one run after another, 8.2 -> 4.8 us, waited for 16.5 -> 13.1;
 // of 2^18, the most that it is used for, 8.2 -> 6.2 and 15.6 -> 14.0.  400001 elements take 9.6 against 8.2 us, 2^20 12.3 against 8.2:
-// there the grid's many SMs are worth the clearing.
+// there the grid's many SMs are worth the clearing.  Several arrays, counted together (grid / cluster): two read, one stored and two
+// folds, 87381 elements 8.2 / 6.2, 10^5 8.2 / 8.2; two read, two stored and two folds, 65536 elements 8.2 / 6.1, 80000 8.2 / 8.2.
 constexpr int kFewBlocks = 8, kFewThreads = 1024;
 template <class CL> constexpr bool few_eligible() {
   if (domain_rank<CL>() > 1 || count_if<CL>(is_scalar_fold) == 0) return false;

@@ -141,7 +141,8 @@ __device__ __forceinline__ void pair_of(uint32_t p, int T, int& I, int& J) {
 
 // A tile on its way through a block's registers: asked for all at once, then put down in shared memory.  16 threads x 128 bits per
 // row, 16 rows per pass; rows that do not start on 16 bytes a word per thread, 64 to a row
-// (four words per thread, one tile after the other: 2501 rows 18.4 -> 16.7 us in k_tile_pair, 1301 rows 11.8 -> 11.5).
+// (four words per thread, one tile after the other, took longer in k_tile_pair: 2717 rows 20.2 -> 18.4 us, of two arrays 28.0 -> 25.2,
+// with the product stored as well 3001 rows 27.2 -> 22.8).
 template <bool VEC> struct TileOnItsWay {
   using WORD = std::conditional_t<VEC, uint4, uint32_t>;
   static constexpr int LINE = VEC ? 16 : 64, PASS = kBlock / LINE, STEPS = kTile / PASS;   // threads to a row, rows at a time, passes
@@ -289,9 +290,11 @@ __global__ void __launch_bounds__(kBlock) k_tile_pair(const __grid_constant__ Ar
 
 // Row folds of a small domain: a cluster of blocks to every block of rows, each with every kTrBlocks-th column tile, whose sums
 // meet in the first one's shared memory.  Every source tile is read twice (by the block of rows that it lies in and by the one
-// that it is the transpose of), which costs little where the array stays in L2, and there are no counters to clear beforehand, no
-// partial sums to write, and no block that has to come last.  us, the pair kernels against this one: 65 and 256 rows 8.2 / 4.7, 500
-// 10.3 / 4.8, 999 10.3 / 6.2, 1301 11.8 / 8.2, 1999 14.0 / 10.3, 2000 14.4 / 8.2, 2501 18.3 / 14.7, 3000 16.4 / 14.2.
+// that it is the transpose of; an array that is read one way only needs half of that, which is not made use of), which costs little
+// where the array stays in L2, and there are no counters to clear beforehand, no partial sums to write, and no block that has to
+// come last.  us, the pair kernels against this one, one array: 65 and 256 rows 8.2 / 4.7, 500 10.3 / 4.7, 999 10.3 / 6.2, 1301 11.7 /
+// 8.2, 1999 14.0 / 10.3, 2000 14.4 / 8.2, 2501 18.4 / 14.7, 3000 16.4 / 14.2; two: 256 8.2 / 4.7, 999 12.3 / 8.2, 1301 14.3 / 12.3, 1999 20.5 /
+// 14.4, 2000 14.3 / 12.3 (beyond that see use_tile_rows).
 constexpr int kTrBlocks = 8;
 template <class CL> constexpr bool tile_rows_eligible() {
   if (!tile_eligible<CL>() || staged_externals<CL>() > 2 || count_if<CL>(is_row_fold) == 0) return false;

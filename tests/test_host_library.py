@@ -460,7 +460,6 @@ def test_spin_limit_is_a_property_of_the_graph():
 
 
 def test_built_libraries_stay_small():
-    # a copy of the tree takes them along to the machine with the GPU, where copies of more than 512 MB are refused; half of that
-    # is left to what lies beside them (353 + 101 MB before the test kernels were compressed)
+    # the tree is copied from machine to machine with its built files (353 + 101 MB before the test kernels were compressed)
     from paper_2407_13585_b200 import build
     assert os.path.getsize(build.LIB) + os.path.getsize(build.TEST_LIB) < 256 << 20
